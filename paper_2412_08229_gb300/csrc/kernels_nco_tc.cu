@@ -13,8 +13,10 @@
 // Design notes from measurements on GB300 (M = 128, K = 16, BF16):
 //  * the tensor pipe spends 40 (N <= 32) to 52 (N = 80) cycles on an MMA whose A operand
 //    is in shared memory (reading the 4 KB A tile dominates), 18-24 cycles (N <= 48) when
-//    A is in TMEM; one issuing thread starts at most one MMA every ~61 cycles;
-//  * timestamps inside this kernel at 256^3: a warpgroup spends ~45k cycles on a tile,
+//    A is in TMEM; an elected issuing thread (elect_one) spends 4-9 cycles per MMA;
+//  * issuing from an elect.sync branch instead of a lane test took the 96^3 mirror step of
+//    the deep network from 0.41 to 0.32 ms; before that change,
+//    timestamps inside this kernel at 256^3: a warpgroup spends ~45k cycles on a tile,
 //    43% of it in MMA round trips (issue to completion seen: ~600 cycles for L1, ~1000
 //    for the eight L2 MMAs, which queue behind the other warpgroups' MMAs), 28% in the
 //    epilogues, 12% in barriers and 15% in the per-cell load, moments, relaxation and store;
@@ -85,9 +87,9 @@ __global__ void __launch_bounds__(kWGs * 128, 1) nco_tc_kernel(const StepArgs a0
     extern __shared__ __align__(1024) uint8_t smem[];
     constexpr int kThreads = kWGs * 128;
     const int tid = threadIdx.x;
-    const int wg = tid >> 7;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform, and seen to be
+    const int wg = warp >> 2;
     const int r = tid & 127;
-    const int warp = tid >> 5;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + bar_off<kWGs>());
     uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + bar_off<kWGs>() + 2 * kWGs * 8);
     float* fh2 = reinterpret_cast<float*>(smem + fh_off<kWGs>());
@@ -196,7 +198,7 @@ __global__ void __launch_bounds__(kWGs * 128, 1) nco_tc_kernel(const StepArgs a0
         for (int j = 0; j < kHidden; ++j) acc[j] = 0.0f;
         for (int c = 0; c < kChunks; ++c) {
             // ---- layer 1 for four group elements
-            if (r == 0) {
+            if ((warp & 3) == 0 && elect_one()) {
                 tc_fence_after();
 #pragma unroll
                 for (int kk = 0; kk < kK1 / 16; ++kk)
@@ -215,7 +217,7 @@ __global__ void __launch_bounds__(kWGs * 128, 1) nco_tc_kernel(const StepArgs a0
             if (!(ok = wg_sync_and(bid, w_ok))) break;
 
             // ---- layer 2: one MMA pair per group element, written over D1
-            if (r == 0) {
+            if ((warp & 3) == 0 && elect_one()) {
                 tc_fence_after();
 #pragma unroll
                 for (int g = 0; g < kChunkG; ++g)
@@ -235,7 +237,7 @@ __global__ void __launch_bounds__(kWGs * 128, 1) nco_tc_kernel(const StepArgs a0
                 fence_proxy_async_smem();
                 tc_fence_before();
                 if (!(ok = wg_sync_and(bid, w_ok))) break;
-                if (r == 0) {
+                if ((warp & 3) == 0 && elect_one()) {
                     tc_fence_after();
 #pragma unroll
                     for (int g = 0; g < kChunkG; ++g)

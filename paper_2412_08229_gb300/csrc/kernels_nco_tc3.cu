@@ -81,9 +81,9 @@ __global__ void __launch_bounds__(kWGs * 128, 1) nco_tc3_kernel(const StepArgs a
                                                                  int ntiles, long long limit, const FusedForce ff) {
     extern __shared__ __align__(1024) uint8_t smem[];
     const int tid = threadIdx.x;
-    const int wg = tid >> 7;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform, and seen to be
+    const int wg = warp >> 2;
     const int r = tid & 127;
-    const int warp = tid >> 5;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kBarOff);
     uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + kBarOff + 2 * kWGs * 8);
     float* fh2 = reinterpret_cast<float*>(smem + kFhOff);
@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(kWGs * 128, 1) nco_tc3_kernel(const StepArgs a
         for (int j = 0; j < kHidden; ++j) acc[j] = 0.0f;
         for (int c = 0; c < kChunks; ++c) {
             // ---- layer 1 for four group elements
-            if (r == 0) {
+            if ((warp & 3) == 0 && elect_one()) {
                 tc_fence_after();
                 mma_split(tmem + kD1Col, tmem + kA1Col, sW + kB1HiOff + c * kB1ChunkBytes,
                           sW + kB1LoOff + c * kB1ChunkBytes, 128 * kK1 / 8, id1);
@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(kWGs * 128, 1) nco_tc3_kernel(const StepArgs a
                 tmem_st_wait();
                 tc_fence_before();
                 if (!(ok = wg_sync_and(bid, w_ok))) break;
-                if (r == 0) {
+                if ((warp & 3) == 0 && elect_one()) {
                     tc_fence_after();
 #pragma unroll
                     for (int e = 0; e < 2; ++e)
@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(kWGs * 128, 1) nco_tc3_kernel(const StepArgs a
                     tmem_st_wait();
                     tc_fence_before();
                     if (!(ok = wg_sync_and(bid, w_ok))) break;
-                    if (r == 0) {
+                    if ((warp & 3) == 0 && elect_one()) {
                         tc_fence_after();
 #pragma unroll
                         for (int e = 0; e < 2; ++e)

@@ -84,9 +84,10 @@ __global__ void __launch_bounds__(kThreads, 1) nco_tcp_kernel(const StepArgs a0,
                                                               long long limit, const FusedForce ff) {
     extern __shared__ __align__(1024) uint8_t smem[];
     const int tid = threadIdx.x;
-    const int warp = tid >> 5, lane_id = tid & 31;
-    const int pipe = tid >> 8;
-    const int s = (tid >> 7) & 1;  // warpgroup within the pipeline
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform, and seen to be
+    const int lane_id = tid & 31;
+    const int pipe = warp >> 3;
+    const int s = (warp >> 2) & 1;  // warpgroup within the pipeline
     const int r = tid & 127;       // cell of the tile, TMEM lane
     const int wq = warp & 3;       // TMEM lane quarter of this warp
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kBarOff) + pipe * kBarsPerPipe;
@@ -133,8 +134,7 @@ __global__ void __launch_bounds__(kThreads, 1) nco_tcp_kernel(const StepArgs a0,
     float* mbuf = reinterpret_cast<float*>(smem + kPipeOff + pipe * kPipeBytes);
     float* accbuf = reinterpret_cast<float*>(smem + kPipeOff + pipe * kPipeBytes + 2 * kMBufBytes);
     const int bid = 1 + 2 * pipe + s;
-    const bool l2_issuer = wq == 0 && lane_id == 0;
-    const bool l1_issuer = wq == 1 && lane_id == 0;
+    const bool l2_warp = wq == 0, l1_warp = wq == 1;  // each issues from one elected lane
     constexpr uint32_t idesc = idesc_bf16(128, kN);
 
     // forced steps: warpgroup 0's fixed-point projection sums of the velocities it loads
@@ -147,7 +147,6 @@ __global__ void __launch_bounds__(kThreads, 1) nco_tcp_kernel(const StepArgs a0,
             mma_bf16_ta(tD1, tA1 + 8 * kk, smem_desc(sB1 + P * kB1PairBytes + kk * 256, 128, 128 * kK1 / 8), idesc,
                         kk);
         mma_commit(bar_l1);
-        ++c_l1;
     };
     bool ok = true;
     int it = 0;
@@ -219,9 +218,10 @@ __global__ void __launch_bounds__(kThreads, 1) nco_tcp_kernel(const StepArgs a0,
             ++n_a1;
             if (!(ok = wg_sync_and(bid, ok && w && wa))) break;
         }
-        if (l1_issuer) {
+        if (l1_warp) {
             tc_fence_after();
-            issue_l1(s);
+            if (elect_one()) issue_l1(s);
+            ++c_l1;
         }
         float acc[kHidden];
 #pragma unroll
@@ -256,17 +256,20 @@ __global__ void __launch_bounds__(kThreads, 1) nco_tcp_kernel(const StepArgs a0,
             }
             tc_fence_before();
             if (!(ok = wg_sync_and(bid, ok && w1 && w2))) break;
-            if (l2_issuer) {
+            if (l2_warp) {
                 tc_fence_after();
+                if (elect_one()) {
 #pragma unroll
-                for (int kk = 0; kk < kK2 / 16; ++kk)
-                    mma_bf16_ta(tD2, tA2 + 8 * kk, smem_desc(sB2 + kk * 256, 128, 128 * kK2 / 8), idesc, kk);
-                mma_commit(bar_l2);
+                    for (int kk = 0; kk < kK2 / 16; ++kk)
+                        mma_bf16_ta(tD2, tA2 + 8 * kk, smem_desc(sB2 + kk * 256, 128, 128 * kK2 / 8), idesc, kk);
+                    mma_commit(bar_l2);
+                }
                 ++c_l2;
             }
-            if (l1_issuer && i + 1 < kPairsPerWg) {
+            if (l1_warp && i + 1 < kPairsPerWg) {
                 tc_fence_after();
-                issue_l1(2 * (i + 1) + s);
+                if (elect_one()) issue_l1(2 * (i + 1) + s);
+                ++c_l1;
             }
             w2 = wait_phase(bar_l2, n_l2 & 1u, limit);
             ++n_l2;
@@ -335,8 +338,8 @@ __global__ void __launch_bounds__(kThreads, 1) nco_tcp_kernel(const StepArgs a0,
         if (r == 0) atomicOr(a0.status, 2);
         // wait, with the full limit, for the last commit of each issuer: no MMA may still use
         // TMEM when it is released
-        if (l1_issuer && c_l1 > 0) drained = wait_phase(bar_l1, (c_l1 - 1u) & 1u);
-        if (l2_issuer && c_l2 > 0) drained = wait_phase(bar_l2, (c_l2 - 1u) & 1u);
+        if (l1_warp && c_l1 > 0) drained = wait_phase(bar_l1, (c_l1 - 1u) & 1u);
+        if (l2_warp && c_l2 > 0) drained = wait_phase(bar_l2, (c_l2 - 1u) & 1u);
     }
     tc_fence_before();
     if (!__syncthreads_and(drained)) {

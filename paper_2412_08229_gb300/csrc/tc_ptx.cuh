@@ -40,6 +40,18 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
            (static_cast<uint32_t>(M >> 4) << 24);
 }
 
+// True in one lane of the (converged) warp, the same one at every call. Issuing tcgen05.mma and
+// commit from an elect.sync branch, not from a lane == 0 test, matters: the compiler then
+// knows that a single thread issues and feeds the instruction's uniform operands directly
+// (GB300: 4-9 cycles per MMA and 10 per commit, against 45 each from a lane test, for which
+// it has to serialise over possible lanes). 256^3 mixed NCO step 4.70 -> 3.62 ms, 128^3
+// split-BF16 step 1.70 -> 1.10 ms.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t one;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(one)::"memory");
+    return one != 0;
+}
+
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }
