@@ -636,7 +636,7 @@ def batching_form(P, torch, steps=500, warmup=3):
         init(b[i], i)
     stream = torch.cuda.Stream()  # a timing stream; the batch runs on its own stream
     shape = P.lbm_batch_autotune(b)
-    out["autotune_tile_shape"] = {0: "pairs of group elements across two warpgroups (2 tiles per SM)"}.get(
+    out["autotune_tile_shape"] = {0: "pairs of group elements across two warpgroups (3 tiles per SM)"}.get(
         shape, f"chunks of four group elements per warpgroup, {shape} warpgroups per SM")
     P.lbm_batch_step(b, warmup, use_graph=True)
     torch.cuda.synchronize()

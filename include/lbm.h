@@ -312,7 +312,7 @@ lbm_status lbm_batch_set_weights(lbm_batch* b, const float* theta, int n);
 
 /* Autotuner of the tile shape of the batched network kernel: time it on the current state
  * without advancing it in each shape and keep the fastest; *choice (may be NULL) receives
- * the shape. Shapes: 0 = pairs of group elements shared by two warpgroups per tile (two
+ * the shape. Shapes: 0 = pairs of group elements worked on by two warpgroups per tile (three
  * tiles in flight per SM, every MMA operand A in tensor memory, the default); 2, 3, 4 =
  * chunks of four group elements per warpgroup with that many warpgroups (tiles in flight)
  * per SM. The shapes differ in the rounding order of the network's FP32 sums (all within

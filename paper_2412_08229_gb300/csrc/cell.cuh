@@ -16,17 +16,20 @@ namespace lbm {
 template <int STORAGE> struct Store;
 template <> struct Store<LBM_STORE_F32> {
     using T = float;
+    static __device__ __forceinline__ float cvt(T v) { return v; }
     static __device__ __forceinline__ float ld(const T* p) { return __ldg(p); }
     static __device__ __forceinline__ void st(T* p, float v) { *p = v; }
 };
 template <> struct Store<LBM_STORE_F16_DEV> {
     using T = __half;
-    static __device__ __forceinline__ float ld(const T* p) { return __half2float(__ldg(p)); }
+    static __device__ __forceinline__ float cvt(T v) { return __half2float(v); }
+    static __device__ __forceinline__ float ld(const T* p) { return cvt(__ldg(p)); }
     static __device__ __forceinline__ void st(T* p, float v) { *p = __float2half_rn(v); }
 };
 template <> struct Store<LBM_STORE_BF16_DEV> {
     using T = __nv_bfloat16;
-    static __device__ __forceinline__ float ld(const T* p) { return __bfloat162float(__ldg(p)); }
+    static __device__ __forceinline__ float cvt(T v) { return __bfloat162float(v); }
+    static __device__ __forceinline__ float ld(const T* p) { return cvt(__ldg(p)); }
     static __device__ __forceinline__ void st(T* p, float v) { *p = __float2bfloat16_rn(v); }
 };
 
@@ -103,14 +106,11 @@ __device__ __forceinline__ void load_pulled(const void* src, const Dims& d, int 
     }
 }
 
-// The same pull with, for periodic boxes, the wrapped source offsets of the three axes
-// formed once per cell (fewer instructions per load; more registers live, which the
-// register-lean step kernels can afford and the tensor-core kernel cannot).
-template <int STORAGE, int BC>
-__device__ __forceinline__ void load_pulled_offsets(const void* src, const Dims& d, int x, int y, int z,
-                                                    float* df) {
-    using S = Store<STORAGE>;
-    const typename S::T* base = static_cast<const typename S::T*>(src);
+// Calls f(integral_constant i, ip, src) for the 27 pulled populations: population ip of cell
+// src. For periodic boxes the wrapped source offsets of the three axes are formed once per
+// cell (fewer instructions per load; more registers live).
+template <int BC, typename F>
+__device__ __forceinline__ void for_pulled(const Dims& d, int x, int y, int z, F&& f) {
     if constexpr (BC == LBM_BC_PERIODIC) {
         // source offsets along each axis for c = +1 (from the cell below) and c = -1
         // (from the cell above), wrapped once per cell instead of once per population
@@ -126,11 +126,25 @@ __device__ __forceinline__ void load_pulled_offsets(const void* src, const Dims&
             if constexpr (cx != 0) s += ox[cx > 0 ? 0 : 1];
             if constexpr (cy != 0) s += oy[cy > 0 ? 0 : 1];
             if constexpr (cz != 0) s += oz[cz > 0 ? 0 : 1];
-            df[i] = S::ld(base + static_cast<size_t>(i) * d.ncell + s);
+            f(Ic, i, s);
         });
     } else {
-        load_pulled<STORAGE, BC>(src, d, x, y, z, df);
+        static_for<Q>([&](auto Ic) {
+            int ip, s;
+            pull_source<BC>(x, y, z, decltype(Ic)::value, d, ip, s);
+            f(Ic, ip, s);
+        });
     }
+}
+
+template <int STORAGE, int BC>
+__device__ __forceinline__ void load_pulled_offsets(const void* src, const Dims& d, int x, int y, int z,
+                                                    float* df) {
+    using S = Store<STORAGE>;
+    const typename S::T* base = static_cast<const typename S::T*>(src);
+    for_pulled<BC>(d, x, y, z, [&](auto Ic, int ip, int s) {
+        df[decltype(Ic)::value] = S::ld(base + static_cast<size_t>(ip) * d.ncell + s);
+    });
 }
 
 template <int STORAGE>
@@ -147,15 +161,19 @@ struct Macro {
     float rho, drho, ux, uy, uz;
 };
 
-__device__ __forceinline__ Macro macro_from_moments(const float* m, float drho) {
+__device__ __forceinline__ Macro macro_from(float m0, float m1, float m3, float m9, float drho) {
     Macro r;
-    r.rho = m[0];
+    r.rho = m0;
     r.drho = drho;
     const float s = (1.0f / kSqrt3) / r.rho;
-    r.ux = m[1] * s;
-    r.uy = m[3] * s;
-    r.uz = m[9] * s;
+    r.ux = m1 * s;
+    r.uy = m3 * s;
+    r.uz = m9 * s;
     return r;
+}
+
+__device__ __forceinline__ Macro macro_from_moments(const float* m, float drho) {
+    return macro_from(m[0], m[1], m[3], m[9], drho);
 }
 
 // m = M f in tensor order from deviations; returns rho - 1 separately.

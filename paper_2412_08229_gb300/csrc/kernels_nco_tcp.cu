@@ -2,31 +2,51 @@
 // Sec. II.B (eq. gconv_m) on the tcgen05 tensor cores, pipelined over pairs of group
 // elements with every MMA operand A and accumulator in tensor memory (TMEM).
 //
-// One persistent CTA per SM runs two tile pipelines; a pipeline is two warpgroups that
-// share one tile of 128 cells (one cell per thread and TMEM lane). The 48 elements g of
-// O_h form 24 pairs (2P, 2P + 1); warpgroup s of a pipeline takes the pairs P = 2i + s,
-// i = 0..11, each with its own TMEM regions:
-//   L1  D1[128 x 48] = A1[128 x 32] . B1_P^T  A1 = (m in the printed order, 1, 0, 0) in TMEM,
+// One persistent CTA per SM runs three chains. A chain owns tiles of 128 cells (one cell per
+// thread and TMEM lane) and walks the 24 pairs P = (2P, 2P + 1) of elements of O_h:
+//   L1  D1[128 x 48] = A1[128 x 32] . B1_P^T  A1 = (m in the printed order, 1, 0, ..) in TMEM,
 //                                            B1_P rows (e, j) = ((W1 P_g)[j,:], b1[j]), g = 2P + e;
 //   L2  D2[128 x 48] = A2[128 x 48] . B2^T    A2 = (relu(h_a), 1, 0, 0, 0, relu(h_b), 1, 0, 0, 0)
-//                                            in TMEM (BF16), B2 = the block-diagonal pair of
-//                                            (W2 | b2), so one chain of three MMAs serves both;
+//                                            in BF16, B2 = the block-diagonal pair of (W2 | b2),
+//                                            so one chain of three MMAs serves both;
 //   L3  on the CUDA cores: h = sum_g relu(D2) in FP32, tau~ = W3 h / 48 + b3 (layer 3 is
 //       affine, so the group mean moves inside it).
-// Per pair a warpgroup converts D1 to A2 (relu, BF16), lets its L2 issuer start layer 2 and
-// its L1 issuer start layer 1 of its next pair into the freed D1, then folds D2 into its
-// group sum while the tensor pipe runs that layer 1. TMEM per pipeline (256 of the SM's 512
-// columns): D1[2] at 0 and 48, D2[2] at 96 and 144, A1 at 192, A2[2] at 208 and 232.
-// At a tile boundary warpgroup 0 loads the next tile (populations, moments, A1) while
-// warpgroup 1 adds warpgroup 0's group sums to its own, forms the rates and relaxes and
-// stores the previous tile (the moments pass through shared memory, double-buffered).
-// The handoffs between the warpgroups never let a barrier run two phases ahead of its
-// waiter (a parity wait cannot tell those apart): warpgroup 1 releases A1 once per tile
-// (after its last layer-1 MMA of the tile completed), and the group sums go through one
-// barrier per tile parity, as their buffers do. Every wait is bounded in clock cycles; a wait that runs out latches a status flag, the
-// warpgroups leave their loops, each MMA issuer waits (full limit) for its last commit, and
-// TMEM is released only when every issuer drained. B operands use the K-major, no-swizzle
-// core-matrix layout of tc_ptx.cuh.
+// A2 is written over the upper half of the D1 it was made from, so a chain needs 160 TMEM
+// columns - D1[2], D2, A1 - and three chains fit. Each chain has two warpgroups and a warp:
+// the converters load the tile, form the moments and A1 and turn each D1 into A2; the summers
+// fold each D2 into the group sum, form the rates, relax and store; the issuer warp does
+// nothing but wait and issue MMAs. The next tile's populations are loaded into registers
+// half-way through the walk; the moments reach the summers through shared memory,
+// double-buffered.
+//
+// What bounds it (128^3, mixed form, ncu): instruction issue, 71 % of the cycles with 197
+// instructions per pair of elements and warp, then the chain's own latency (~840 cycles per
+// pair); tensor pipe 44 % (five N 48 MMAs of 24.5 cycles per pair and tile), FMA pipe 44 %,
+// DRAM 6 %. The 256^3 mixed step takes 2.97 ms, 3.36 ms with two tiles of two warpgroups per SM
+// that both converted and summed, waiting for each pair's layer 2 before the next (325 cycles per
+// pair and SM, here 275). What each part brought, 256^3, from 3.36 ms: relu on the FMA pipe, 32-bit
+// offsets and A2 in place with three chains 3.27; converters and summers apart 3.16; an issuer
+// warp 3.11; named barriers instead of polls 3.05; D2 read whole before the sum and layer 1 two
+// pairs ahead 2.97.
+//
+// Hand-overs, per chain (n = 0..23 of a tile, b = n & 1):
+//   a1full            A1 of the tile written (4 converter warps)      -> issuer: layer 1 of pairs 0, 1
+//   a2full[b]         A2 of pair n written (4 converter warps)        -> issuer, with
+//   d2free            D2 of pair n - 1 read (4 summer warps, who
+//                     arrive once before the first tile)              -> issuer: layer 2 of pair n
+//   CONV[b]           layer 1 of pair n + 1 complete                  issuer -> converters
+//   SUM               layer 2 of pair n complete                      issuer -> summers; layer 1 of
+//                     pair n + 2 then goes into buffer b, which that layer 2 has read
+// The first three and the MMA commits are mbarriers, polled by the issuer alone; CONV and SUM are
+// named barriers, in which warps block without taking issue slots (with every warp polling,
+// polls were a third of the instructions). The next phase of each follows a hand-over that its
+// waiters make after their wait (two pairs on for those with [b]). The moments go through the
+// mbarriers mready[t & 1] / mfree[t & 1], complete by the time they are waited on but for the
+// pipeline's start.
+// Every poll is bounded in clock cycles. When one of a commit runs out the issuer polls no more
+// commits and raises the chain's abort flag; the chain walks through its remaining tiles without storing, the
+// issuer commits once more and waits (full limit) for that, and TMEM is released only when all
+// have drained. B operands use the K-major, no-swizzle core-matrix layout of tc_ptx.cuh.
 #include <cstring>
 
 #include "force.cuh"
@@ -40,13 +60,16 @@ namespace {
 
 constexpr int kTile = 128;
 constexpr int kG = 48;
-constexpr int kPairs = kG / 2;          // 24 pairs of group elements
-constexpr int kPairsPerWg = kPairs / 2;  // 12
-constexpr int kN = 48;                   // 2 elements x 20 hidden units + 8 padding rows
-constexpr int kK1 = 32;                  // 27 moments + bias input + pad
-constexpr int kK2 = 48;                  // 2 x (20 hidden + bias input + 3 pad)
-constexpr int kPipes = 2;
-constexpr int kThreads = kPipes * 256;
+constexpr int kPairs = kG / 2;  // 24 pairs of group elements
+constexpr int kN = 48;          // 2 elements x 20 hidden units + 8 padding rows
+constexpr int kK1 = 32;         // 27 moments + bias input + pad
+constexpr int kK2 = 48;         // 2 x (20 hidden + bias input + 3 pad)
+constexpr int kChains = 3;
+constexpr int kPrefetchPair = 12;  // the next tile's loads are issued after this pair
+constexpr int kThreads = kChains * 256 + 128;  // converters, summers, one warpgroup of issuers
+// registers a thread of each warpgroup holds: together the launch's 72 per thread
+constexpr int kConverterRegs = 72, kSummerRegs = 88, kIssuerRegs = 24;
+static_assert(kChains * (kConverterRegs + kSummerRegs) + kIssuerRegs == (2 * kChains + 1) * 72, "what one gives another takes");
 
 // weight image = shared-memory image: 24 B1 pairs, the block-diagonal B2, W3 and b3 (floats)
 constexpr uint32_t kB1PairBytes = kN * kK1 * 2;  // 3072
@@ -56,297 +79,373 @@ constexpr uint32_t kB2Bytes = kN * kK2 * 2;                  // 4608
 constexpr uint32_t kW3Off = kB2Off + kB2Bytes;
 constexpr uint32_t kB3Off = kW3Off + kOut * kHidden * 4;
 constexpr uint32_t kWeightBytes = kB3Off + 16;  // 78672
-static_assert(kWeightBytes % 16 == 0, "weight image copies in 16-byte vectors");
+static_assert(kWeightBytes % 16 == 0, "the weight image is one bulk copy");
 
-// per pipeline: moments and rho - 1 of two tiles, warpgroup 0's group sums of two tiles
+// the moments and rho - 1 of two tiles of every chain
 constexpr int kMVals = Q + 1;
-constexpr uint32_t kMBufBytes = kMVals * kTile * 4;     // 14336
-constexpr uint32_t kAccBufBytes = kHidden * kTile * 4;  // 10240
-constexpr uint32_t kPipeBytes = 2 * kMBufBytes + 2 * kAccBufBytes;
-constexpr uint32_t kPipeOff = (kWeightBytes + 1023) / 1024 * 1024;
-constexpr uint32_t kBarOff = kPipeOff + kPipes * kPipeBytes;
-// l1[2], l2[2] (commits); A1 written; group sums written, one per tile parity; A1 free
-constexpr int kBarsPerPipe = 8;
-// forced steps: 2 F^ as floats and the block's projection sums
-constexpr uint32_t kFhOff = kBarOff + kPipes * kBarsPerPipe * 8 + 16;
-constexpr uint32_t kRedOff = kFhOff + 6 * kForcedModes * 4;
+constexpr uint32_t kMBufFloats = kMVals * kTile;
+constexpr uint32_t kMOff = (kWeightBytes + 127) / 128 * 128;
+constexpr uint32_t kBarOff = kMOff + kChains * 2 * kMBufFloats * 4;
+// mbarriers: the commits of layer 1 per buffer and of layer 2, then the hand-overs
+enum { kL1 = 0, kL2 = 2, kA1Full = 3, kA2Full = 4, kD2Free = 6, kMReady = 7, kMFree = 9, kDrain = 11, kBarsPerChain = 12 };
+enum { kBarConv = 1, kBarSum = 7 };  // named: + 2 chain + b, + chain
+// after the chains' barriers: the weight copy's barrier, the TMEM base, the chains' abort
+// flags, then (forced steps) 2 F^ as floats and the block's projection sums
+constexpr uint32_t kWBarOff = kBarOff + kChains * kBarsPerChain * 8;
+constexpr uint32_t kAbortOff = kWBarOff + 16;
+constexpr uint32_t kFhOff = kAbortOff + 16;
+constexpr uint32_t kRedOff = (kFhOff + 6 * kForcedModes * 4 + 7) / 8 * 8;
 constexpr uint32_t kSmemBytes = kRedOff + frc::kProjValues * 8;
-static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
+static_assert(kBarOff % 8 == 0 && kSmemBytes <= 227 * 1024, "shared memory budget");
 
 constexpr uint32_t kTmemCols = 512;
-constexpr uint32_t kTmemPerPipe = 256;
-constexpr uint32_t kD1Col = 0, kD2Col = 96, kA1Col = 192, kA2Col = 208;  // + 48 s, + 48 s, -, + 24 s
-static_assert(kA2Col + 2 * 24 == kTmemPerPipe, "TMEM budget of a pipeline");
+constexpr uint32_t kTmemPerChain = 160;
+constexpr uint32_t kD1Cols = 48, kD2Col = 96, kA1Col = 144;  // D1[b] at 48 b
+constexpr uint32_t kA2InD1 = 24;                              // A2 = the upper half of a D1 buffer
+static_assert(kChains * kTmemPerChain <= kTmemCols && kA1Col + 16 == kTmemPerChain, "TMEM budget");
+
+// The populations a cell pulls, as stored (27 registers), from the wrapped offsets of
+// load_pulled_offsets.
+template <int STORAGE, int BC>
+__device__ __forceinline__ void load_raw(const StepArgs& a, long long cell, typename Store<STORAGE>::T* raw) {
+    int x, y, z;
+    cell_coords(cell, a.d, x, y, z);
+    using T = typename Store<STORAGE>::T;
+    const T* base = static_cast<const T*>(a.src);
+    const uint32_t plane = static_cast<uint32_t>(a.d.ncell);  // 27 planes stay below 2^31 elements
+    for_pulled<BC>(a.d, x, y, z, [&](auto Ic, int ip, int src) {
+        raw[decltype(Ic)::value] = __ldg(base + (static_cast<uint32_t>(ip) * plane + static_cast<uint32_t>(src)));
+    });
+}
 
 template <int STORAGE, int BC, bool FORCED, bool BATCHED>
-__global__ void __launch_bounds__(kThreads, 1) nco_tcp_kernel(const StepArgs a0, const BatchTiles bt,
+__global__ void __launch_bounds__(kThreads, 1) nco_tcp_kernel(const __grid_constant__ StepArgs a0, const BatchTiles bt,
                                                               const uint8_t* __restrict__ wimg, int ntiles,
                                                               long long limit, const FusedForce ff) {
     extern __shared__ __align__(1024) uint8_t smem[];
     const int tid = threadIdx.x;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform, and seen to be
-    const int lane_id = tid & 31;
-    const int pipe = warp >> 3;
-    const int s = (warp >> 2) & 1;  // warpgroup within the pipeline
-    const int r = tid & 127;       // cell of the tile, TMEM lane
-    const int wq = warp & 3;       // TMEM lane quarter of this warp
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kBarOff) + pipe * kBarsPerPipe;
-    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + kBarOff + kPipes * kBarsPerPipe * 8);
+    // warps 0..11 convert, 12..23 sum, 24..26 issue (27 has no part)
+    const bool issuer = warp >= kChains * 8, summer = !issuer && warp >= kChains * 4;
+    const int chain = issuer ? warp - kChains * 8 : (warp >> 2) - (summer ? kChains : 0);
+    const int wq = warp & 3;  // TMEM lane quarter of this warp
+    const int r = tid & 127;  // cell of the tile, TMEM lane
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kBarOff) + chain * kBarsPerChain;
+    uint64_t* bar_w = reinterpret_cast<uint64_t*>(smem + kWBarOff);
+    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + kWBarOff + 8);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kAbortOff) + chain;
     float* fh2 = reinterpret_cast<float*>(smem + kFhOff);
     unsigned long long* red = reinterpret_cast<unsigned long long*>(smem + kRedOff);
 
-    // ---- set-up: weights to shared memory, barriers, TMEM
-    for (uint32_t i = tid * 16; i < kWeightBytes; i += kThreads * 16)
-        *reinterpret_cast<uint4*>(smem + i) = *reinterpret_cast<const uint4*>(wimg + i);
+    // ---- set-up: barriers, the weights' bulk copy (in flight until the first layer 1), TMEM
+    if (tid == 0) {
+        for (int c = 0; c < kChains; ++c) {
+            uint64_t* b = reinterpret_cast<uint64_t*>(smem + kBarOff) + c * kBarsPerChain;
+            for (int k = 0; k < kBarsPerChain; ++k)
+                mbar_init(&b[k], k >= kA1Full && k < kDrain ? 4 : 1);
+        }
+        for (int c = 0; c < 4; ++c) *(reinterpret_cast<volatile int*>(smem + kAbortOff) + c) = 0;
+        mbar_init(bar_w, 1);
+        fence_mbar_init();
+        mbar_expect_tx(bar_w, kWeightBytes);
+        bulk_load(smem_u32(smem), wimg, kWeightBytes, bar_w);
+    }
     if (FORCED) {
         frc::load_fh2(ff.fhat, fh2);
         if (tid < frc::kProjValues) red[tid] = 0ull;
     }
-    if (tid == 0) {
-        for (int p = 0; p < kPipes; ++p) {
-            uint64_t* b = reinterpret_cast<uint64_t*>(smem + kBarOff) + p * kBarsPerPipe;
-            for (int k = 0; k < 4; ++k) mbar_init(&b[k], 1);  // one tcgen05.commit each
-            mbar_init(&b[4], 128);                             // warpgroup 0 wrote A1
-            mbar_init(&b[5], 128);                             // warpgroup 0 wrote its group sums (even tile)
-            mbar_init(&b[6], 128);                             // ... (odd tile)
-            mbar_init(&b[7], 128);                             // warpgroup 1's last layer 1 of a tile completed
-        }
-        fence_mbar_init();
-    }
     if (warp == 0) tmem_alloc(tmem_holder, kTmemCols);
-    fence_proxy_async_smem();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
 
-    uint64_t* bar_l1 = &bars[s];       // this warpgroup's layer-1 commits
-    uint64_t* bar_l2 = &bars[2 + s];   // this warpgroup's layer-2 commits
-    uint64_t* bar_a1 = &bars[4];
-    uint64_t* bar_acc = &bars[5];      // + (tile & 1)
-    uint64_t* bar_a1free = &bars[7];   // warpgroup 1 no longer reads the tile's A1
-    const uint32_t tbase = *tmem_holder + static_cast<uint32_t>(pipe) * kTmemPerPipe;
+    // the allocation of all columns starts at column 0: TMEM addresses are constants
+    const uint32_t tbase = static_cast<uint32_t>(chain) * kTmemPerChain;
+    if (*tmem_holder != 0) *abort_flag = 1;
     const uint32_t lanes = static_cast<uint32_t>(wq * 32) << 16;
-    const uint32_t tD1 = tbase + kD1Col + 48 * s, tD2 = tbase + kD2Col + 48 * s;
-    const uint32_t tA1 = tbase + kA1Col, tA2 = tbase + kA2Col + 24 * s;
-    const uint32_t sB1 = smem_u32(smem + kB1Off), sB2 = smem_u32(smem + kB2Off);
-    const float* W3 = reinterpret_cast<const float*>(smem + kW3Off);
-    const float* b3 = reinterpret_cast<const float*>(smem + kB3Off);
-    float* mbuf = reinterpret_cast<float*>(smem + kPipeOff + pipe * kPipeBytes);
-    float* accbuf = reinterpret_cast<float*>(smem + kPipeOff + pipe * kPipeBytes + 2 * kMBufBytes);
-    const int bid = 1 + 2 * pipe + s;
-    const bool l2_warp = wq == 0, l1_warp = wq == 1;  // each issues from one elected lane
-    constexpr uint32_t idesc = idesc_bf16(128, kN);
-
-    // forced steps: warpgroup 0's fixed-point projection sums of the velocities it loads
-    long long pacc[3] = {0, 0, 0};
-    // completions waited on (the parity of the next wait) and commits made (the drain)
-    uint32_t n_l1 = 0, n_l2 = 0, n_a1 = 0, c_l1 = 0, c_l2 = 0;
-    auto issue_l1 = [&](int P) {
-#pragma unroll
-        for (int kk = 0; kk < kK1 / 16; ++kk)
-            mma_bf16_ta(tD1, tA1 + 8 * kk, smem_desc(sB1 + P * kB1PairBytes + kk * 256, 128, 128 * kK1 / 8), idesc,
-                        kk);
-        mma_commit(bar_l1);
+    float* mst = reinterpret_cast<float*>(smem + kMOff) + chain * 2 * kMBufFloats + r;
+    const int lane_id = tid & 31;
+    // bounded wait; one that runs out raises the abort flag
+    auto wait = [&](uint64_t* bar, uint32_t parity, long long cycles) {
+        if (!mbar_try_wait(bar, parity) && !wait_phase(bar, parity, cycles)) *abort_flag = 1;
     };
-    bool ok = true;
-    int it = 0;
-    for (int gtile = blockIdx.x * kPipes + pipe; gtile < ntiles; gtile += gridDim.x * kPipes, ++it) {
-        int tile = gtile;
-        StepArgs a = a0;
-        if (BATCHED) {  // the instance owning this tile
-            const int inst = __ldg(&bt.tile_inst[gtile]);
-            a = bt.inst[inst];
-            tile = gtile - static_cast<int>(__ldg(&bt.tile_begin[inst]));
+    auto args_of = [&bt](int gt, int& tile, const StepArgs*& ap) {
+        tile = gt;
+        if constexpr (BATCHED) {  // the instance owning this tile
+            const int inst = __ldg(&bt.tile_inst[gt]);
+            tile = gt - static_cast<int>(__ldg(&bt.tile_begin[inst]));
+            ap = bt.inst + inst;
         }
-        const long long cell = static_cast<long long>(tile) * kTile + r;
-        const bool valid = cell < a.d.ncell;
-        bool w = true;
-        if (s == 0) {
-            // A1 is free once warpgroup 1's last layer-1 MMA of the previous tile has completed,
-            // which warpgroup 1 signals once per tile, so the barrier is at most one phase
-            // ahead of or behind this wait (the result is made uniform: the A1 store below is
-            // a warp-collective instruction)
-            if (it > 0)
-                w = wg_sync_and(bid, wait_phase(bar_a1free, static_cast<uint32_t>(it - 1) & 1u, limit));
-            float m[Q];
-            float drho = 0.0f;
-            int x = 0, y = 0, z = 0;
-            Macro q{};
-            if (valid) {
-                cell_coords(cell, a.d, x, y, z);
-                float df[Q];
-                load_pulled<STORAGE, BC>(a.src, a.d, x, y, z, df);
-                drho = moments_from_dev(df, m);
-                q = macro_from_moments(m, drho);
-                if (!(q.rho >= a.rho_min && q.rho <= a.rho_max)) atomicOr(a.status, 1);
-                if (BATCHED && a.u_out) {
-                    a.u_out[cell] = q.ux;
-                    a.u_out[a.d.ncell + cell] = q.uy;
-                    a.u_out[2 * a.d.ncell + cell] = q.uz;
+    };
+    // tiles in rounds over the SMs, so that a small grid spreads over them before it shares one
+    const int stride = static_cast<int>(gridDim.x) * kChains;
+    int gtile = static_cast<int>(blockIdx.x + gridDim.x * chain);
+    bool drained = true;
+
+    if (issuer) {
+        reg_dec<kIssuerRegs>();
+        // one copy of the loop per chain, so that every operand but the pair's descriptor is constant
+        auto run = [&](auto Cc) {
+            constexpr uint32_t base = decltype(Cc)::value * kTmemPerChain;
+            constexpr uint32_t idesc = idesc_bf16(128, kN);
+            const uint64_t db1 = smem_desc(smem_u32(smem + kB1Off), 128, 128 * kK1 / 8);
+            const uint64_t db2 = smem_desc(smem_u32(smem + kB2Off), 128, 128 * kK2 / 8);
+            auto issue_l1 = [&](int P, int b) {
+#pragma unroll
+                for (int kk = 0; kk < kK1 / 16; ++kk)
+                    mma_bf16_ta(base + kD1Cols * b, base + kA1Col + 8 * kk, db1 + (P * kB1PairBytes + kk * 256) / 16, idesc, kk);
+                mma_commit(&bars[kL1 + b]);
+            };
+            bool ok = *abort_flag == 0;
+            auto poll_mma = [&](uint64_t* bar, uint32_t parity) {
+                if (ok && !mbar_try_wait(bar, parity)) {
+                    ok = wait_phase(bar, parity, limit);
+                    if (!ok) *abort_flag = 1;
                 }
-            } else {
+                tc_fence_after();
+                tc_fence_before();
+            };
+            auto poll_warps = [&](uint64_t* bar, uint32_t parity) {  // also after an abort: keeps pace with the other warps
+                wait(bar, parity, kDefaultWaitCycles);
+                tc_fence_after();
+            };
+            for (int it = 0; gtile < ntiles; gtile += stride, ++it) {
+                poll_warps(&bars[kA1Full], static_cast<uint32_t>(it) & 1u);
+                if (it == 0) wait(bar_w, 0, kDefaultWaitCycles);  // the weights have arrived
+                if (elect_one()) {
+                    issue_l1(0, 0);
+                    issue_l1(1, 1);
+                }
+                if (limit <= 0) {  // gives up at the first wait
+                    ok = false;
+                    *abort_flag = 1;
+                }
+                poll_mma(&bars[kL1], 0);
+                bar_arrive<160>(kBarConv + 2 * chain);
+#pragma unroll 1
+                for (int n2 = 0; n2 < kPairs; n2 += 2) {
 #pragma unroll
-                for (int e = 0; e < Q; ++e) m[e] = 0.0f;
-                m[0] = 1.0f;
+                    for (int b = 0; b < 2; ++b) {  // pair n = n2 + b, in buffer b
+                        const uint32_t half = static_cast<uint32_t>(n2 >> 1);
+                        poll_warps(&bars[kA2Full + b], half & 1u);
+                        poll_warps(&bars[kD2Free], b);
+                        if (elect_one()) {
+#pragma unroll
+                            for (int kk = 0; kk < kK2 / 16; ++kk)
+                                mma_bf16_ta(base + kD2Col, base + kD1Cols * b + kA2InD1 + 8 * kk, db2 + kk * 16, idesc, kk);
+                            mma_commit(&bars[kL2]);
+                        }
+                        if (b == 0 || n2 + 2 < kPairs) {  // a pair n + 1 follows
+                            poll_mma(&bars[kL1 + (b ^ 1)], (half + b) & 1u);
+                            bar_arrive<160>(kBarConv + 2 * chain + (b ^ 1));
+                        }
+                        poll_mma(&bars[kL2], b);
+                        bar_arrive<160>(kBarSum + chain);
+                        if (n2 + 2 < kPairs && elect_one()) issue_l1(n2 + b + 2, b);
+                    }
+                }
             }
-            float* mb = mbuf + (it & 1) * kMVals * kTile;
+            if (__any_sync(0xffffffffu, !ok)) {
+                // one more commit and a wait, with the full limit, for all this lane issued: no MMA
+                // may still use TMEM when it is released
+                if (elect_one()) mma_commit(&bars[kDrain]);
+                drained = wait_phase(&bars[kDrain], 0) && wait_phase(bar_w, 0);
+            }
+        };
+        if (chain == 0) run(std::integral_constant<int, 0>{});
+        else if (chain == 1) run(std::integral_constant<int, 1>{});
+        else if (chain == 2) run(std::integral_constant<int, 2>{});
+    } else if (!summer) {
+        const uint32_t tA1 = tbase + kA1Col;
+        typename Store<STORAGE>::T raw[Q];
+        auto prefetch = [&](int gt) {
+            if (gt >= ntiles) return;
+            int tile;
+            const StepArgs* ap = &a0;
+            args_of(gt, tile, ap);
+            const long long cell = static_cast<long long>(tile) * kTile + r;
+            if (cell < ap->d.ncell) load_raw<STORAGE, BC>(*ap, cell, raw);
+        };
+        prefetch(gtile);
+        for (int it = 0; gtile < ntiles; gtile += stride, ++it) {
+            int tile;
+            const StepArgs* ap = &a0;
+            args_of(gtile, tile, ap);
+            const StepArgs& a = *ap;
+            const long long cell = static_cast<long long>(tile) * kTile + r;
+            const bool valid = cell < a.d.ncell;
+            if (it >= 2) wait(&bars[kMFree + (it & 1)], static_cast<uint32_t>((it >> 1) - 1) & 1u, kDefaultWaitCycles);
+            {
+                float m[Q];
+                float drho = 0.0f;
+                if (valid) {
+                    float df[Q];
 #pragma unroll
-            for (int e = 0; e < Q; ++e) mb[e * kTile + r] = m[e];
-            mb[Q * kTile + r] = drho;
-            uint32_t p[16];  // A1 row r: the raw moments in the printed order of Sec. II.B, then the bias input 1
-            static_for<13>([&](auto K) {
-                constexpr int k = decltype(K)::value;
-                p[k] = pack_bf16(m[kPrintedE<2 * k>], m[kPrintedE<2 * k + 1>]);
-            });
-            p[13] = pack_bf16(m[kPrintedE<26>], 1.0f);
-            p[14] = 0u;
-            p[15] = 0u;
-            if (w) {  // the previous tile's layer 1 may still read A1 otherwise
+                    for (int i = 0; i < Q; ++i) df[i] = Store<STORAGE>::cvt(raw[i]);
+                    drho = moments_from_dev(df, m);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < Q; ++e) m[e] = 0.0f;
+                    m[0] = 1.0f;
+                }
+                float* mb = mst + (it & 1) * kMBufFloats;
+#pragma unroll
+                for (int e = 0; e < Q; ++e) mb[e * kTile] = m[e];
+                mb[Q * kTile] = drho;
+                // (after the transform: a branch among its sums has the compiler fuse other products
+                // in the batched kernel, and an instance has to stay bit-identical to its own steps)
+                if (valid && !(m[0] >= a.rho_min && m[0] <= a.rho_max)) atomicOr(a.status, 1);
+                uint32_t p[16];  // A1 row r: the raw moments in the printed order of Sec. II.B, then the bias input 1
+                static_for<13>([&](auto K) {
+                    constexpr int k = decltype(K)::value;
+                    p[k] = pack_bf16(m[kPrintedE<2 * k>], m[kPrintedE<2 * k + 1>]);
+                });
+                p[13] = pack_bf16(m[kPrintedE<26>], 1.0f);
+                p[14] = 0u;
+                p[15] = 0u;
                 tmem_st16(tA1 + lanes, p);
                 tmem_st_wait();
+                tc_fence_before();
+                __syncwarp();
+                mbar_arrive_lane0(&bars[kA1Full], lane_id);
+                mbar_arrive_lane0(&bars[kMReady + (it & 1)], lane_id);
             }
-            tc_fence_before();
-            mbar_arrive(bar_a1);
             if (FORCED && ff.proj) {  // this tile's velocities into the next step's projection
+                float* mb = mst + (it & 1) * kMBufFloats;
+                Macro q{};
+                int x = 0, y = 0, z = 0;
+                if (valid) {
+                    cell_coords(cell, a.d, x, y, z);
+                    q = macro_from(mb[0], mb[1 * kTile], mb[3 * kTile], mb[9 * kTile], 0.0f);
+                }
                 frc::Cx ph[kForcedModes];
                 frc::cell_phases(x, y, z, a.d, ff.tab, ph);
-                frc::project_warp(q.ux, q.uy, q.uz, ph, lane_id, pacc, ff.scale);
+                long long pacc[3] = {0, 0, 0};
+                frc::project_warp(q.ux, q.uy, q.uz, ph, tid & 31, pacc, ff.scale);
+                frc::proj_to_shared(red, pacc, tid & 31);
             }
-        }
-        {
-            const bool wa = wait_phase(bar_a1, n_a1 & 1u, limit);
-            ++n_a1;
-            if (!(ok = wg_sync_and(bid, ok && w && wa))) break;
-        }
-        if (l1_warp) {
-            tc_fence_after();
-            if (elect_one()) issue_l1(s);
-            ++c_l1;
-        }
-        float acc[kHidden];
+#pragma unroll 1
+            for (int n2 = 0; n2 < kPairs; n2 += 2) {
 #pragma unroll
-        for (int j = 0; j < kHidden; ++j) acc[j] = 0.0f;
-        bool w2 = true;
-        for (int i = 0; i < kPairsPerWg; ++i) {
-            const bool w1 = wait_phase(bar_l1, n_l1 & 1u, limit);
-            ++n_l1;
-            tc_fence_after();
-            if (s == 1 && i == kPairsPerWg - 1) mbar_arrive(bar_a1free);  // its last layer 1 read A1
-            {  // D1 of the pair -> (relu in BF16, 1, 0) per element = A2
-                uint32_t v[40];
-                tmem_ld16(tD1 + lanes, v);
-                tmem_ld16(tD1 + lanes + 16, v + 16);
-                tmem_ld8(tD1 + lanes + 32, v + 32);
-                tmem_ld_wait();
-                uint32_t h[24];
+                for (int b = 0; b < 2; ++b) {  // pair n = n2 + b, in buffer b
+                    bar_sync<160>(kBarConv + 2 * chain + b);
+                    tc_fence_after();
+                    // D1 of the pair -> relu in BF16 = A2, over the upper half of the same buffer
+                    const uint32_t t = tbase + lanes + kD1Cols * b;
+                    uint32_t v[kHidden], h[24];
 #pragma unroll
-                for (int k = 0; k < 10; ++k) {
-                    h[k] = pack_bf16_relu(as_f(v[2 * k]), as_f(v[2 * k + 1]));
-                    h[12 + k] = pack_bf16_relu(as_f(v[20 + 2 * k]), as_f(v[21 + 2 * k]));
+                    for (int e = 0; e < 2; ++e) {  // one element of the pair after the other: fewer registers
+                        tmem_ld16(t + kHidden * e, v);
+                        tmem_ld4(t + kHidden * e + 16, v + 16);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int k = 0; k < 10; ++k) h[12 * e + k] = pack_bf16_relu(as_f(v[2 * k]), as_f(v[2 * k + 1]));
+                    }
+                    h[10] = h[22] = kBf16One;
+                    h[11] = h[23] = 0u;
+#pragma unroll
+                    for (int k = 0; k < 24; k += 8) tmem_st8(t + kA2InD1 + k, h + k);
+                    tmem_st_wait();
+                    tc_fence_before();
+                    __syncwarp();
+                    mbar_arrive_lane0(&bars[kA2Full + b], lane_id);
                 }
-                h[10] = kBf16One;
-                h[11] = 0u;
-                h[22] = kBf16One;
-                h[23] = 0u;
-                // three 8-column stores: A2 of warpgroup 1 starts 8-, not 16-column aligned
-                tmem_st8(tA2 + lanes, h);
-                tmem_st8(tA2 + lanes + 8, h + 8);
-                tmem_st8(tA2 + lanes + 16, h + 16);
-                tmem_st_wait();
+                if (n2 == kPrefetchPair) prefetch(gtile + stride);
             }
-            tc_fence_before();
-            if (!(ok = wg_sync_and(bid, ok && w1 && w2))) break;
-            if (l2_warp) {
-                tc_fence_after();
-                if (elect_one()) {
+        }
+    } else {
+        reg_inc<kSummerRegs>();
+        const uint32_t tD2 = tbase + kD2Col + lanes;
+        const float4* W3 = reinterpret_cast<const float4*>(smem + kW3Off);
+        const float* b3 = reinterpret_cast<const float*>(smem + kB3Off);
+        mbar_arrive_lane0(&bars[kD2Free], lane_id);  // D2 is free
+        for (int it = 0; gtile < ntiles; gtile += stride, ++it) {
+            // 2 relu(h) summed over the even and over the odd pairs
+            float acc[2][kHidden];
 #pragma unroll
-                    for (int kk = 0; kk < kK2 / 16; ++kk)
-                        mma_bf16_ta(tD2, tA2 + 8 * kk, smem_desc(sB2 + kk * 256, 128, 128 * kK2 / 8), idesc, kk);
-                    mma_commit(bar_l2);
-                }
-                ++c_l2;
-            }
-            if (l1_warp && i + 1 < kPairsPerWg) {
-                tc_fence_after();
-                if (elect_one()) issue_l1(2 * (i + 1) + s);
-                ++c_l1;
-            }
-            w2 = wait_phase(bar_l2, n_l2 & 1u, limit);
-            ++n_l2;
-            tc_fence_after();
-            {  // relu of the pair's layer-2 outputs, summed over the group
-                uint32_t v[40];
-                tmem_ld16(tD2 + lanes, v);
-                tmem_ld16(tD2 + lanes + 16, v + 16);
-                tmem_ld8(tD2 + lanes + 32, v + 32);
-                tmem_ld_wait();
-                tc_fence_before();  // D2 read before this warpgroup's next layer 2 overwrites it
+            for (int j = 0; j < kHidden; ++j) acc[0][j] = acc[1][j] = 0.0f;
+#pragma unroll 1
+            for (int n2 = 0; n2 < kPairs; n2 += 2) {
 #pragma unroll
-                for (int j = 0; j < kHidden; j += 2) {
-                    add2_relu(acc[j], acc[j + 1], as_f(v[j]), as_f(v[j + 1]));
-                    add2_relu(acc[j], acc[j + 1], as_f(v[kHidden + j]), as_f(v[kHidden + j + 1]));
+                for (int b = 0; b < 2; ++b) {
+                    bar_sync<160>(kBarSum + chain);
+                    tc_fence_after();
+                    uint32_t v[40];
+                    tmem_ld16(tD2, v);
+                    tmem_ld16(tD2 + 16, v + 16);
+                    tmem_ld8(tD2 + 32, v + 32);
+                    tmem_ld_wait();
+                    tc_fence_before();
+                    __syncwarp();
+                    mbar_arrive_lane0(&bars[kD2Free], lane_id);  // before the sum: layer 2 of the next pair waits for it
+#pragma unroll
+                    for (int j = 0; j < kHidden; j += 2) {
+                        add2_relu2(acc[b][j], acc[b][j + 1], as_f(v[j]), as_f(v[j + 1]));
+                        add2_relu2(acc[b][j], acc[b][j + 1], as_f(v[kHidden + j]), as_f(v[kHidden + j + 1]));
+                    }
                 }
             }
-        }
-        if (!ok) break;
-        if (!(ok = wg_sync_and(bid, w2))) break;
-        float* ab = accbuf + (it & 1) * kHidden * kTile;
-        if (s == 0) {  // hand this warpgroup's group sums to warpgroup 1
-#pragma unroll
-            for (int j = 0; j < kHidden; ++j) ab[j * kTile + r] = acc[j];
-            mbar_arrive(bar_acc + (it & 1));
-        } else {
-            // one barrier per tile parity (as for the buffers): warpgroup 0 may hand over the
-            // next tile's sums before this wait, but not the one after (it needs bar_a1free)
-            const bool wa = wait_phase(bar_acc + (it & 1), static_cast<uint32_t>(it >> 1) & 1u, limit);
-            if (!(ok = wg_sync_and(bid, wa))) break;
-            if (valid) {
+            wait(&bars[kMReady + (it & 1)], static_cast<uint32_t>(it >> 1) & 1u, kDefaultWaitCycles);
+            if (it == 0) wait(bar_w, 0, kDefaultWaitCycles);  // W3 and b3, before this thread first reads them
+            int tile;
+            const StepArgs* ap = &a0;
+            args_of(gtile, tile, ap);
+            const StepArgs& a = *ap;
+            const long long cell = static_cast<long long>(tile) * kTile + r;
+            if (cell < a.d.ncell && !*abort_flag) {
                 float rates[kOut];
 #pragma unroll
-                for (int n = 0; n < kOut; ++n) {
+                for (int j = 0; j < kHidden; ++j) acc[0][j] += acc[1][j];
+#pragma unroll
+                for (int k = 0; k < kOut; ++k) {
                     float t = 0.0f;
 #pragma unroll
-                    for (int j = 0; j < kHidden; ++j) t = fmaf(W3[n * kHidden + j], acc[j] + ab[j * kTile + r], t);
-                    rates[n] = rate_from_output(t * (1.0f / 48.0f) + b3[n]);
+                    for (int j = 0; j < kHidden; j += 4) {
+                        const float4 w = W3[(k * kHidden + j) / 4];
+                        t = fmaf(w.x, acc[0][j], t);
+                        t = fmaf(w.y, acc[0][j + 1], t);
+                        t = fmaf(w.z, acc[0][j + 2], t);
+                        t = fmaf(w.w, acc[0][j + 3], t);
+                    }
+                    rates[k] = rate_from_output(t * (0.5f / 48.0f) + b3[k]);
                 }
-                const float* mb = mbuf + (it & 1) * kMVals * kTile;
-                float m[Q];
-#pragma unroll
-                for (int e = 0; e < Q; ++e) m[e] = mb[e * kTile + r];
-                const float drho = mb[Q * kTile + r];
-                const Macro q = macro_from_moments(m, drho);
-                float df[Q];
-                relax_to_populations(m, drho, q, 1.0f / a.tau, rates, df);
+                float F[3];
                 if (FORCED) {  // F(x) from this step's coefficients
                     int x, y, z;
                     cell_coords(cell, a.d, x, y, z);
                     frc::Cx ph[kForcedModes];
                     frc::cell_phases(x, y, z, a.d, ff.tab, ph);
-                    float F[3];
                     frc::synth_force(fh2, ph, F);
-                    add_kupershtokh(df, q, F[0], F[1], F[2]);
-                } else if (BATCHED && a.force) {
-                    add_kupershtokh(df, q, a.force[cell], a.force[a.d.ncell + cell], a.force[2 * a.d.ncell + cell]);
                 }
+                const float* mb = mst + (it & 1) * kMBufFloats;
+                float m[Q];
+#pragma unroll
+                for (int e = 0; e < Q; ++e) m[e] = mb[e * kTile];
+                const float drho = mb[Q * kTile];
+                const Macro q = macro_from_moments(m, drho);
+                if (BATCHED && a.u_out) {
+                    a.u_out[cell] = q.ux;
+                    a.u_out[a.d.ncell + cell] = q.uy;
+                    a.u_out[2 * a.d.ncell + cell] = q.uz;
+                }
+                float df[Q];
+                relax_to_populations(m, drho, q, 1.0f / a.tau, rates, df);
+                if (FORCED) add_kupershtokh(df, q, F[0], F[1], F[2]);
+                else if (BATCHED && a.force)
+                    add_kupershtokh(df, q, a.force[cell], a.force[a.d.ncell + cell], a.force[2 * a.d.ncell + cell]);
                 store_cell<STORAGE>(a.dst, a.d, cell, df);
             }
+            __syncwarp();
+            mbar_arrive_lane0(&bars[kMFree + (it & 1)], lane_id);
         }
     }
-    if (FORCED && ff.proj && s == 0) frc::proj_to_shared(red, pacc, lane_id);
-    bool drained = true;
-    if (!ok) {
-        if (r == 0) atomicOr(a0.status, 2);
-        // wait, with the full limit, for the last commit of each issuer: no MMA may still use
-        // TMEM when it is released
-        if (l1_warp && c_l1 > 0) drained = wait_phase(bar_l1, (c_l1 - 1u) & 1u);
-        if (l2_warp && c_l2 > 0) drained = wait_phase(bar_l2, (c_l2 - 1u) & 1u);
-    }
+    if (lane_id == 0 && *abort_flag) atomicOr(a0.status, 2);
     tc_fence_before();
     if (!__syncthreads_and(drained)) {
         if (tid == 0) atomicOr(a0.status, 4);  // MMAs still running: TMEM is left allocated
         return;
     }
-    if (FORCED && ff.proj && ok) frc::proj_to_global(red, ff.proj);
+    if (FORCED && ff.proj && *abort_flag == 0) frc::proj_to_global(red, ff.proj);
     if (warp == 0) {
         tc_fence_after();
         tmem_dealloc(*tmem_holder, kTmemCols);
@@ -360,8 +459,7 @@ cudaError_t launch_tcp_t(const StepArgs& a, const BatchTiles& bt, const void* w,
     const cudaError_t e =
         ensure_dynamic_smem(nco_tcp_kernel<STORAGE, BC, FORCED, BATCHED>, static_cast<int>(kSmemBytes), attr);
     if (e != cudaSuccess) return e;
-    int grid = (ntiles + kPipes - 1) / kPipes;
-    if (grid > sm_count()) grid = sm_count();
+    const int grid = ntiles < sm_count() ? ntiles : sm_count();
     if (grid < 1) return cudaSuccess;
     nco_tcp_kernel<STORAGE, BC, FORCED, BATCHED>
         <<<grid, kThreads, kSmemBytes, s>>>(a, bt, static_cast<const uint8_t*>(w), ntiles, wait, ff);

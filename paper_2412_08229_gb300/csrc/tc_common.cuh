@@ -53,6 +53,17 @@ __device__ __forceinline__ bool wg_sync_and(int id, bool ok) {
     return out != 0;
 }
 
+// Named barrier `id` of N threads: wait for it, or arrive without waiting. Blocked warps take no
+// issue slots, unlike warps that poll an mbarrier.
+template <int N>
+__device__ __forceinline__ void bar_sync(int id) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(N) : "memory");
+}
+template <int N>
+__device__ __forceinline__ void bar_arrive(int id) {
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(N) : "memory");
+}
+
 __device__ __forceinline__ float as_f(uint32_t u) { return __uint_as_float(u); }
 
 
@@ -75,6 +86,18 @@ __device__ __forceinline__ void relax_to_populations(const float* m, float drho,
 __device__ __forceinline__ void add2_relu(float& a0, float& a1, float b0, float b1) {
     b0 = fmaxf(b0, 0.0f);
     b1 = fmaxf(b1, 0.0f);
+    asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%0, %1};\n\tmov.b64 y, {%2, %3};\n\t"
+        "add.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
+        : "+f"(a0), "+f"(a1)
+        : "f"(b0), "f"(b1));
+}
+
+// (a0, a1) += 2 (relu(b0), relu(b1)): 2 relu(b) = b + |b| exactly, which runs on the FMA pipe
+// (one cycle per warp instruction) where max runs on the ALU pipe (two). A sum of doubled
+// terms is the doubled sum, bit for bit.
+__device__ __forceinline__ void add2_relu2(float& a0, float& a1, float b0, float b1) {
+    b0 = b0 + fabsf(b0);
+    b1 = b1 + fabsf(b1);
     asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%0, %1};\n\tmov.b64 y, {%2, %3};\n\t"
         "add.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
         : "+f"(a0), "+f"(a1)
