@@ -19,21 +19,22 @@ constexpr int kNumTheta = 27 * 20 + 20 + 20 * 20 + 20 + 20 * 4 + 4;  // 1064 (Se
 constexpr int kNumThetaDeep = kNumTheta + 20 * 20 + 20;  // 1484: a third hidden layer of 20 (Sec. IV)
 constexpr int kForcedModes = 16;  // half-space integer modes with 1 <= |k| <= 2
 
-// Network parameters handed to the FP32 step kernel by value (they live in the
-// kernel's constant parameter bank, so FFMAs read them without loads).
+// Parameters of the FP32 network as its kernels lay them out in shared memory (copied as a
+// whole from device memory at the start of a block).
 // W1p[p] = W1 with its columns rearranged for axis permutation p: the input of
-// group element (p, s) is then sgn(s, t) * m_t in tensor order t (see nco_f32).
-struct NetParams {
-    float W1p[6][kHidden][Q];
-    float b1[kHidden];
+// group element (p, s) is then sgn(s, t) * m_t in tensor order t (net_f32.cuh).
+struct alignas(16) NetParams {
+    float W1p[6][kHidden][28];         // 27 columns, then b1: rows of seven 16-byte quadruples
     float W2[kHidden][kHidden];
-    float b2[kHidden];
-    float W3[kOut][kHidden];  // output layer
+    float W2T[kHidden][kHidden];       // transposed, for the cotangents
+    float Wd[kHidden][kHidden];        // third hidden layer (deep network only)
+    float WdT[kHidden][kHidden];
+    float b2[kHidden], bd[kHidden];
+    float W3[kOut][kHidden];           // output layer
     float b3[kOut];
-    float Wd[kHidden][kHidden];  // third hidden layer (deep network only)
-    float bd[kHidden];
-    int deep;                    // 1: 27-20-20-20-4, 0: 27-20-20-4
+    int deep;                          // 1: 27-20-20-20-4, 0: 27-20-20-4
 };
+static_assert(sizeof(NetParams) % 16 == 0, "copied in 16-byte vectors");
 
 // One symmetry g = (A, t) of the Taylor-Green flow that maps the block of the periodic
 // box next to the reduced domain [0, pi/2]^3 in direction (rx, ry, rz) onto the domain:
@@ -104,12 +105,14 @@ struct FusedForce;  // the in-kernel forcing of a forced step (declared with the
 // elements across two warpgroups, kernels_nco_tcp.cu, two-layer network only; 2, 3, 4:
 // chunks of four elements per warpgroup, kernels_nco_tc.cu, with that many warpgroups per
 // SM in batches). The per-tile arithmetic of one shape does not depend on the warpgroup count.
+// net_weights: the context's weights in device memory, a NetParams for the FP32 network or
+// the packed operands of a tensor-core network; deep: a third hidden layer.
 // wait_cycles: limit of the main MMA-completion waits of the pair-pipelined and split
 // tensor-core kernels (kept out of StepArgs: a larger argument block made the CUDA-core
 // network kernel spill).
 // ff: the in-kernel forcing of a forced step (nullptr: unforced; a.force is then not read).
 cudaError_t launch_step(const StepArgs& a, const FusedForce* ff, int op, int storage, int bc, int net_prec,
-                        const NetParams* net, const void* tc_weights, int tc_shape, long long wait_cycles,
+                        bool deep, const void* net_weights, int tc_shape, long long wait_cycles,
                         cudaStream_t s);
 cudaError_t launch_init_eq(const Dims& d, int storage, int bc, const float* rho, const float* u,
                            void* dst, cudaStream_t s);
@@ -122,6 +125,10 @@ cudaError_t launch_macroscopic(const Dims& d, int storage, int bc, const void* s
 cudaError_t launch_kinetic_energy(const Dims& d, int storage, int bc, const void* src,
                                   double* partials, int npartials, double* out, cudaStream_t s);
 int kinetic_energy_blocks(const Dims& d);
+
+// FP32 network on the CUDA cores (kernels_nco_f32.cu)
+cudaError_t launch_step_nco_f32(const StepArgs& a, const FusedForce* ff, int storage, int bc, bool deep,
+                                const NetParams* d_net, cudaStream_t s);
 
 // Tensor-core network (kernels_nco_tc.cu)
 size_t nco_tc_weight_bytes();
@@ -230,8 +237,8 @@ int adjoint_grad_len(bool deep);
 cudaError_t launch_adjoint_seed(const Dims& d, int storage, int bc, const void* state, const float* du,
                                 const float* drho, float ke_scale, bool accumulate, float* lam, cudaStream_t s);
 cudaError_t launch_adjoint_step(const Dims& d, int storage, int bc, const void* state, const float* lam_in,
-                                float* lam_out, double* grad, float tau, const float* force, const NetParams& net,
-                                cudaStream_t s);
+                                float* lam_out, double* grad, float tau, const float* force, bool deep,
+                                const NetParams* d_net, cudaStream_t s);
 void adjoint_fold_gradient(const double* acc, bool deep, float* out);
 
 // Host-side group tables and parameter packing (lbm_abi.cu)

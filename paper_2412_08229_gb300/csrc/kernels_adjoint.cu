@@ -16,58 +16,57 @@
 // forward kernel's form), and so are the first layer's cotangents: with E[c][j] =
 // sum_s (-1)^popcount(s & c) delta h1[s][j], the cotangent of m_t is sum_j W1p[j][t]
 // E[c(t)][j] and dW1p[j][t] = sum over cells of m_t E[c(t)][j], c(t) the parity class of
-// moment t. Each thread keeps the 8 x 20 values of its cell (h1, then delta h1, then E) in
-// a row of shared memory. Weight gradients: per sign vector the block stages (delta h2, h1;
-// with the third hidden layer also delta h3, h2) of its 128 cells and accumulates
-// register-blocked outer products, per permutation (E, m) for the first layer, flushed to
-// FP64 global accumulators with atomics.
-// Layout of the accumulator (doubles): [dW1p (6 x 20 x 27, the W1 columns rearranged per
-// axis permutation) | db1 | dW2 | db2 | (dWd | dbd, third hidden layer) | dW3 | db3]; the
-// host folds dW1p back to the printed column order of W1.
+// moment t.
+//
+// A block has twelve warps (net_f32.cuh) and a tile of 32 cells (two-layer network) or 16
+// (third hidden layer). h1 of every column stays in shared memory from the forward to the
+// backward part; of the last hidden layer only the signs are kept (20 bits per column), so
+// nothing of the forward is computed twice. The weight gradients are outer products summed
+// over columns: a lane has 10 x 6 outputs, 60 FMAs for 15 floats read.
+//
+// What bounds it (32^3, ncu): shared-memory latency and bandwidth between bursts of FMAs
+// (wavefronts 55 %, issue 47 %, three warps a scheduler). One step: 32^3 225 us, with the
+// third hidden layer 409 us, 16^3 40 and 67 us; before (one thread per cell, the forward
+// computed twice, outer products by 40 of 128 threads): 723, 1137, 232 and 359 us.
 //
 // Observations of the kinetic energy k = (1/2)<|u|^2> at intermediate steps (the loss of
 // Sec. IV is a function of k(t)) enter as extra seeds added to lam_t when the reverse
 // sweep passes step t: dk/df_i = (1/cells) sum_a u_a (c_ia - u_a) / rho.
 #include "cell.cuh"
+#include "net_f32.cuh"
 
 namespace lbm {
 
-constexpr int kAdjThreads = 128;
-
+// Gradient accumulator (doubles) in the flat parameter order W1 (printed columns), b1, W2,
+// b2, (Wd, bd: third hidden layer), W3, b3.
 template <bool DEEP>
 struct GradLayout {
-    static constexpr int kB1 = 6 * kHidden * Q;                 // dW1p first
+    static constexpr int kB1 = kHidden * Q;
     static constexpr int kW2 = kB1 + kHidden;
     static constexpr int kB2 = kW2 + kHidden * kHidden;
-    static constexpr int kWd = kB2 + kHidden;                   // third hidden layer
+    static constexpr int kWd = kB2 + kHidden;
     static constexpr int kBd = kWd + kHidden * kHidden;
     static constexpr int kW3 = DEEP ? kBd + kHidden : kB2 + kHidden;
     static constexpr int kB3 = kW3 + kOut * kHidden;
-    static constexpr int kLen = kB3 + kOut;                     // 3764 or 4184
+    static constexpr int kLen = kB3 + kOut;
 };
+static_assert(GradLayout<false>::kLen == kNumTheta && GradLayout<true>::kLen == kNumThetaDeep, "parameter order");
 
 int adjoint_grad_len(bool deep) { return deep ? GradLayout<true>::kLen : GradLayout<false>::kLen; }
 
-__device__ __forceinline__ int adj_odd_mask(int t) {
-    return ((ex_of(t) == 1) << 2) | ((ey_of(t) == 1) << 1) | (ez_of(t) == 1);
+// Column of W1p[p] that printed column k of W1 went to (the moment permutation of the
+// element with axis permutation p and no reflection).
+struct PermColumns {
+    unsigned char t[6][Q];
+};
+constexpr PermColumns make_perm_columns() {
+    PermColumns r{};
+    const GroupTables g = make_group();
+    for (int p = 0; p < 6; ++p)
+        for (int k = 0; k < Q; ++k) r.t[p][k] = static_cast<unsigned char>(g.mperm_t[p * 8][kPrinted.e[k]]);
+    return r;
 }
-
-// y[s] <- sum_c (-1)^popcount(s & c) y[c], in place (its own inverse up to a factor 8)
-__device__ __forceinline__ void wht8(float* y) {
-#pragma unroll
-    for (int bit = 1; bit < 8; bit <<= 1)
-#pragma unroll
-        for (int c = 0; c < 8; ++c)
-            if (!(c & bit)) {
-                const float u = y[c], v = y[c | bit];
-                y[c] = u + v;
-                y[c | bit] = u - v;
-            }
-}
-
-// a thread's row of first-layer values: [s * kHidden + j], padded so that the rows of a
-// warp's threads fall in different banks
-constexpr int kHbStride = 8 * kHidden + 1;
+__constant__ PermColumns kPermColumns = make_perm_columns();
 
 // Inverse of the pull map: the (x, i) whose pulled value is population j of cell y.
 template <int BC>
@@ -130,409 +129,477 @@ struct AdjArgs {
     double* grad;        // GradLayout<DEEP>::kLen accumulators
     float tau;
     const float* force;  // forced step: the force field of step t (3 planes), else null
-    int nparts;          // blocks per tile, each backpropagating 6 / nparts axis permutations
 };
 
-// Shared staging of one group element for the whole block (the last two arrays only with
-// the third hidden layer).
-template <bool DEEP>
-struct AdjStage {
-    float dh2[kAdjThreads][kHidden];
-    float h1x[kAdjThreads][24];   // h1 (20), 1 (bias), pad
-    float xm[kAdjThreads][28];    // moments (27, tensor order), 1 (bias)
-    float dh3[DEEP ? kAdjThreads : 1][kHidden];
-    float h2x[DEEP ? kAdjThreads : 1][24];  // h2 (20), 1 (bias), pad
-};
+constexpr int kAdjThreads = 32 * kNetWarps;
+constexpr int kGradBlock = kHidden * kHidden + kHidden;  // dW and db of a 20 x 20 layer
 
-template <bool DEEP>
+// LANES lanes share a cell, each holding COLS of the half's four sign vectors.
+template <bool DEEP, int LANES>
 struct AdjShared {
-    AdjStage<DEEP> st;
-    float hb[kAdjThreads * kHbStride];  // per cell: h1, delta h1, then E of the 8 sign vectors
-    NetParams net;                      // weights, read with run-time group indices
-    float tail[kAdjThreads][24];        // per cell: gbar (4), group mean of the last hidden layer (20)
+    static constexpr int kCells = 32 / LANES;
+    static constexpr int kCols = 4 / LANES;
+    static constexpr int kRow = net_row(kCols);
+    // per warp: the staged cotangents of one column per lane (32 x 20), the partial sums of
+    // the last hidden layer, and at the end the weight gradients of the hidden layers and of
+    // the warp's half of W1p
+    static constexpr int kD1 = DEEP ? 2 * kGradBlock : kGradBlock;
+    static constexpr int kStage = (kD1 + (Q + 1) * kHalf + 3) / 4 * 4;
+    static_assert(kStage >= 32 * kHidden, "stage holds a column per lane");
+    static_assert(2 * Q * kCells <= 32 * kRow, "the moment cotangents fit a warp's rows");
+
+    NetParams net;
+    float h1[kNetWarps][32][kRow];  // h1, then delta h1, then E, then the partial cotangent of m
+    float h2[DEEP ? kNetWarps : 1][32][DEEP ? kRow : 4];  // h2, then delta h2 (third hidden layer)
+    float stage[kNetWarps][kStage];
+    float m[kCells][28];      // moments (tensor order), 1 (the bias input)
+    float mu[kCells][28];     // mu*, then the relaxation's part of dL/dm
+    float dm[Q][kCells];
+    float hsum[kCells][kHidden];
+    float v3[kCells][kHidden];  // cotangent of the last hidden layer, the same for every group element
+    float gbar[kCells][kOut];
+    float rates[kCells][kOut];
 };
 
-template <int STORAGE, int BC, bool DEEP>
-__global__ void __launch_bounds__(kAdjThreads, 1) adjoint_step_kernel(const AdjArgs a,
-                                                                      const __grid_constant__ NetParams netp) {
+// Outer products summed over columns: a warp's 20 x 21 gradient (W | b) in tiles of 10 x 5
+// (and the bias column) over 2 x 4 lanes; the four groups of eight lanes take the rows
+// r = 0..31 of a column in turn.
+struct OuterTile {
+    float a[kHalf][6];
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int j = 0; j < kHalf; ++j)
+#pragma unroll
+            for (int k = 0; k < 6; ++k) a[j][k] = 0.0f;
+    }
+    // rows r of d (stride ds) times rows r of h (stride hs)
+    __device__ __forceinline__ void add(const float* d, int ds, const float* h, int hs, int lane) {
+        const int grp = lane >> 3, jt = (lane >> 2) & 1, kt = lane & 3;
+        d += grp * ds + jt * kHalf;
+        h += grp * hs + kt * 5;
+#pragma unroll 1
+        for (int r = 0; r < 32; r += 4, d += 4 * ds, h += 4 * hs) {
+            float dv[kHalf], hv[5];
+#pragma unroll
+            for (int j = 0; j < kHalf; j += 2) {
+                const float2 t = *reinterpret_cast<const float2*>(d + j);
+                dv[j] = t.x;
+                dv[j + 1] = t.y;
+            }
+#pragma unroll
+            for (int k = 0; k < 5; ++k) hv[k] = h[k];
+#pragma unroll
+            for (int j = 0; j < kHalf; ++j) {
+#pragma unroll
+                for (int k = 0; k < 5; ++k) a[j][k] = fmaf(dv[j], hv[k], a[j][k]);
+                a[j][5] += dv[j];
+            }
+        }
+    }
+    // sums over the four groups to out: [j][k] (20 x 20), then the bias column
+    __device__ __forceinline__ void flush(float* out, int lane) {
+        const int jt = (lane >> 2) & 1, kt = lane & 3;
+#pragma unroll
+        for (int j = 0; j < kHalf; ++j)
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                float v = a[j][k];
+                v += __shfl_xor_sync(0xffffffffu, v, 8);
+                v += __shfl_xor_sync(0xffffffffu, v, 16);
+                if (lane < 8) {
+                    if (k < 5) out[(jt * kHalf + j) * kHidden + kt * 5 + k] = v;
+                    else if (kt == 0) out[kHidden * kHidden + jt * kHalf + j] = v;
+                }
+            }
+    }
+};
+
+template <int STORAGE, int BC, bool DEEP, int LANES>
+__global__ void __launch_bounds__(kAdjThreads, (!DEEP && LANES == 2) ? 2 : 1)
+    adjoint_step_kernel(const AdjArgs a, const NetParams* __restrict__ net_in) {
     using GL = GradLayout<DEEP>;
+    using SH = AdjShared<DEEP, LANES>;
+    constexpr int kCells = SH::kCells, C = SH::kCols, kRow = SH::kRow;
     extern __shared__ __align__(16) uint8_t adj_smem_raw[];
-    AdjShared<DEEP>& sh = *reinterpret_cast<AdjShared<DEEP>*>(adj_smem_raw);
-    AdjStage<DEEP>& st = sh.st;
+    SH& sh = *reinterpret_cast<SH*>(adj_smem_raw);
     const NetParams& net = sh.net;
     const int tid = threadIdx.x;
-    {
-        const float* srcw = reinterpret_cast<const float*>(&netp);
-        float* dstw = reinterpret_cast<float*>(&sh.net);
-        for (int i = tid; i < static_cast<int>(sizeof(NetParams) / 4); i += kAdjThreads) dstw[i] = srcw[i];
-        __syncthreads();
-    }
-    // small grids: nparts blocks share a tile, block `part` backpropagating the group
-    // elements of axis permutations [part, part + 1) * 6 / nparts; every part recomputes the
-    // forward, part 0 alone adds the relaxation terms and the output-layer gradient
-    const long long tile = blockIdx.x / a.nparts;
-    const int part = static_cast<int>(blockIdx.x % a.nparts);
-    const int p_begin = part * (6 / a.nparts), p_end = p_begin + 6 / a.nparts;
-    const long long cell = tile * kAdjThreads + tid;
-    const bool valid = cell < a.d.ncell;
+    const int lane = tid & 31;
+    const int w = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform, and seen to be
+    const int p = w >> 1, half = w & 1;
+    const int l = lane & 15, og = lane >> 4;  // the rows l and l + 16, units [10 og, 10 og + 10)
+    const long long cell0 = static_cast<long long>(blockIdx.x) * kCells;
 
-    // ---- forward recompute of this cell
-    float m[Q];
-    float drho = 0.0f;
-    float lam[Q];
-    int x = 0, y = 0, z = 0;
-    if (valid) {
-        cell_coords(cell, a.d, x, y, z);
-        float df[Q];
-        load_pulled<STORAGE, BC>(a.state, a.d, x, y, z, df);
-        drho = moments_from_dev(df, m);
-#pragma unroll
-        for (int jj = 0; jj < Q; ++jj) {
-            int i, dst;
-            push_target<BC>(x, y, z, jj, a.d, i, dst);
-            lam[jj] = a.lam_in[static_cast<size_t>(i) * a.d.ncell + dst];
-        }
-    } else {
-#pragma unroll
-        for (int e = 0; e < Q; ++e) {
-            m[e] = 0.0f;
-            lam[e] = 0.0f;
-        }
-        m[0] = 1.0f;
-    }
-
-    // this thread's row of first-layer values; first_layer(p) fills it with relu(W1p x^(s) +
-    // b1) of the 8 sign vectors s of permutation p
-    float* hb = sh.hb + tid * kHbStride;
-    auto first_layer = [&](int p) {
-#pragma unroll 2
-        for (int j = 0; j < kHidden; ++j) {
-            float y[8];
-#pragma unroll
-            for (int c = 0; c < 8; ++c) y[c] = 0.0f;
-#pragma unroll
-            for (int t = 0; t < Q; ++t) y[adj_odd_mask(t)] = fmaf(net.W1p[p][j][t], m[t], y[adj_odd_mask(t)]);
-            wht8(y);
-#pragma unroll
-            for (int sv = 0; sv < 8; ++sv) hb[sv * kHidden + j] = fmaxf(y[sv] + net.b1[j], 0.0f);
-        }
-    };
-
-    // group sum of the last hidden layer (h2, or h3 with the third hidden layer)
-    float hsum[kHidden];
-#pragma unroll
-    for (int j = 0; j < kHidden; ++j) hsum[j] = 0.0f;
-#pragma unroll 1
-    for (int p = 0; p < 6; ++p) {
-        first_layer(p);
-#pragma unroll 1
-        for (int sv = 0; sv < 8; ++sv) {
-            float h1[kHidden];
-#pragma unroll
-            for (int j = 0; j < kHidden; ++j) h1[j] = hb[sv * kHidden + j];
-            if constexpr (DEEP) {
-                float h2[kHidden];
-#pragma unroll 2
-                for (int j = 0; j < kHidden; ++j) {
-                    float acc = net.b2[j];
-#pragma unroll
-                    for (int k = 0; k < kHidden; ++k) acc = fmaf(net.W2[j][k], h1[k], acc);
-                    h2[j] = fmaxf(acc, 0.0f);
-                }
-#pragma unroll 2
-                for (int j = 0; j < kHidden; ++j) {
-                    float acc = net.bd[j];
-#pragma unroll
-                    for (int k = 0; k < kHidden; ++k) acc = fmaf(net.Wd[j][k], h2[k], acc);
-                    hsum[j] += fmaxf(acc, 0.0f);
-                }
+    // ---- moments (warp 0) and cotangents in moment space (warp 1) of the tile's cells
+    if (w < 2 && lane < kCells) {
+        const long long cell = cell0 + lane;
+        float v[Q];
+        if (cell < a.d.ncell) {
+            int x, y, z;
+            cell_coords(cell, a.d, x, y, z);
+            if (w == 0) {
+                float df[Q];
+                load_pulled<STORAGE, BC>(a.state, a.d, x, y, z, df);
+                moments_from_dev(df, v);
             } else {
-#pragma unroll 2
-                for (int j = 0; j < kHidden; ++j) {
-                    float acc = net.b2[j];
 #pragma unroll
-                    for (int k = 0; k < kHidden; ++k) acc = fmaf(net.W2[j][k], h1[k], acc);
-                    hsum[j] += fmaxf(acc, 0.0f);
+                for (int j = 0; j < Q; ++j) {
+                    int i, dst;
+                    push_target<BC>(x, y, z, j, a.d, i, dst);
+                    v[j] = a.lam_in[static_cast<size_t>(i) * a.d.ncell + dst];
                 }
+                populations_transpose_inplace(v);  // mu* = M^-T lam* (tensor order)
             }
+        } else {  // a cell past the end: no cotangent, so it adds nothing
+#pragma unroll
+            for (int e = 0; e < Q; ++e) v[e] = 0.0f;
+            if (w == 0) v[0] = 1.0f;
         }
+        float* dst = w == 0 ? sh.m[lane] : sh.mu[lane];
+#pragma unroll
+        for (int e = 0; e < Q; ++e) dst[e] = v[e];
+        dst[Q] = 1.0f;
     }
-    float ttil[kOut], tau_n[kOut], rates[kOut];
-#pragma unroll
-    for (int n = 0; n < kOut; ++n) {
-        float acc = 0.0f;
-#pragma unroll
-        for (int j = 0; j < kHidden; ++j) acc = fmaf(net.W3[n][j], hsum[j], acc);
-        ttil[n] = acc * (1.0f / 48.0f) + net.b3[n];
-        tau_n[n] = 0.5f / (1.0f + expf(ttil[n])) + 0.5f;
-        rates[n] = 1.0f / tau_n[n];
-    }
-#pragma unroll
-    for (int j = 0; j < kHidden; ++j) sh.tail[tid][4 + j] = hsum[j] * (1.0f / 48.0f);
+    if (w >= 2) load_params(&sh.net, net_in, tid - 64, kAdjThreads - 64);
+    __syncthreads();
 
-    // ---- cotangents in moment space
-    populations_transpose_inplace(lam);  // lam now holds mu* = M^-T lam* (tensor order)
-    const float omega_nu = 1.0f / a.tau;
-    float dm[Q];
-    float gw[kOut] = {0.0f, 0.0f, 0.0f, 0.0f};
-    const float rho = m[0];
-    const float irho = 1.0f / rho;
+    // ---- first layer
+    float* const rows = &sh.h1[w][0][0];
+    float* const row = sh.h1[w][l];
+    {
+        float m[2 / LANES][28];
 #pragma unroll
-    for (int e = 0; e < Q; ++e) dm[e] = 0.0f;
+        for (int k = 0; k < 2 / LANES; ++k)
 #pragma unroll
-    for (int e = 0; e < Q; ++e) {
-        const int n = order_of(e);
-        const float mu = lam[e];
-        if (n <= 1) {
-            dm[e] += mu;
-        } else if (n == 2) {
-            dm[e] += (1.0f - omega_nu) * mu;
-            // m^eq_e = m_a m_b / m_0 for the axes a, b of component e
-            const int ex = ex_of(e), ey = ey_of(e), ez = ez_of(e);
-            int ia = -1, ib = -1, axa = 0, axb = 0;
-            const int cnt[3] = {ex, ey, ez};
-            const int idx[3] = {1, 3, 9};
+            for (int e = 0; e < 28; e += 4)
+                *reinterpret_cast<float4*>(&m[k][e]) = *reinterpret_cast<const float4*>(&sh.m[l + 16 * k][e]);
+        first_layer<LANES>(net, p, half, lane, m, &sh.h1[2 * p][0][0]);
+    }
+    pair_sync(p);
+
+    // ---- the layers up to the group sum; mask[r][c] keeps which units of the last hidden layer
+    // are on in column c of row l + 16 r (unit j in bit 31 - j)
+    uint32_t mask[2][C];
+    {
+        float acc[2][C][kHalf];
+        set_bias(net.b2, lane, acc);
+        mat_vec<C>(net.W2, lane, acc, RowColumns<C>{row});
+        if constexpr (DEEP) {
+            float* const row2 = sh.h2[w][l];
+            store_relu(row2, lane, acc);
+            __syncwarp();
+            set_bias(net.bd, lane, acc);
+            mat_vec<C>(net.Wd, lane, acc, RowColumns<C>{row2});
+        }
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                if (cnt[k] == 2) { ia = idx[k]; ib = idx[k]; axa = axb = k; }
-                if (cnt[k] == 1) {
-                    if (ia < 0) { ia = idx[k]; axa = k; }
-                    else { ib = idx[k]; axb = k; }
+        for (int r = 0; r < 2; ++r) {
+            float hs[kHalf];
+#pragma unroll
+            for (int o = 0; o < kHalf; ++o) hs[o] = 0.0f;
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                uint32_t k = 0u;
+#pragma unroll
+                for (int o = 0; o < kHalf; ++o) {
+                    const float h = fmaxf(acc[r][c][o], 0.0f);
+                    hs[o] += h;
+                    k = __funnelshift_l(__float_as_uint(0.0f - h), k, 1);  // the sign of -h: h > 0
                 }
+                k <<= og ? 32 - kHidden : 32 - kHalf;
+                mask[r][c] = k | __shfl_xor_sync(0xffffffffu, k, 16);
             }
-            const float ma = m[ia], mb = m[ib];
-            const float c = omega_nu * mu;
-            dm[ia] += c * mb * irho;
-            dm[ib] += c * ma * irho;
-            dm[0] -= c * ma * mb * irho * irho;
-            if (a.force && valid) {
-                // Kupershtokh source (Sec. II.A) in moment space: its only state-dependent part
-                // is order 2, dm*_ab = 3 ((j + F)_a (j + F)_b - j_a j_b) / rho with m_a = sqrt3 j_a,
-                // i.e. (sqrt3 (m_a F_b + F_a m_b) + 3 F_a F_b) / rho; the force is an input
-                const float Fa = a.force[static_cast<size_t>(axa) * a.d.ncell + cell];
-                const float Fb = a.force[static_cast<size_t>(axb) * a.d.ncell + cell];
-                const float src = (kSqrt3 * (ma * Fb + Fa * mb) + 3.0f * Fa * Fb) * irho;
-                dm[ia] += mu * kSqrt3 * Fb * irho;
-                dm[ib] += mu * kSqrt3 * Fa * irho;
-                dm[0] -= mu * src * irho;
-            }
-        } else {
-            dm[e] += (1.0f - rates[n - 3]) * mu;
-            gw[n - 3] -= mu * m[e];
+#pragma unroll
+            for (int o = 0; o < kHalf; o += 2)
+                *reinterpret_cast<float2*>(&sh.stage[w][(l + 16 * r) * kHidden + og * kHalf + o]) = make_float2(hs[o], hs[o + 1]);
         }
     }
-    if (part != 0) {  // the relaxation's own terms belong to part 0; the rates' cotangent gw to all
+    __syncthreads();
+    for (int i = tid; i < kCells * kHidden; i += kAdjThreads) {  // group sum, i = cell * 20 + unit
+        float v = 0.0f;
+#pragma unroll
+        for (int q = 0; q < kNetWarps; ++q)
+#pragma unroll
+            for (int l = 0; l < LANES; ++l) v += sh.stage[q][i + l * kCells * kHidden];
+        (&sh.hsum[0][0])[i] = v;
+    }
+    __syncthreads();
+    if (tid < kOut * kCells) {  // rates and the cotangents of tau~, one (cell, output) per thread
+        const int n = tid / kCells, c = tid % kCells;
+        float t = 0.0f;
+#pragma unroll
+        for (int j = 0; j < kHidden; ++j) t = fmaf(net.W3[n][j], sh.hsum[c][j], t);
+        t = t * (1.0f / 48.0f) + net.b3[n];
+        const float e = expf(t);
+        const float tau_n = 0.5f / (1.0f + e) + 0.5f;
+        float gw = 0.0f;
+#pragma unroll
+        for (int k = 0; k < Q; ++k)
+            if (order_of(k) >= 3)
+                gw -= order_of(k) == n + 3 ? sh.mu[c][k] * sh.m[c][k] : 0.0f;
+        // d omega / d tau~ = sigma (1 - sigma) / (2 tau_n^2), sigma = 1 / (1 + e^{tau~})
+        const float sg = 1.0f / (1.0f + e);
+        sh.rates[c][n] = 1.0f / tau_n;
+        sh.gbar[c][n] = cell0 + c < a.d.ncell ? gw * sg * (1.0f - sg) / (2.0f * tau_n * tau_n) : 0.0f;
+    }
+    __syncthreads();
+    for (int i = tid; i < kCells * kHidden; i += kAdjThreads) {  // W3^T gbar / 48
+        const int c = i / kHidden, j = i % kHidden;
+        float v = 0.0f;
+#pragma unroll
+        for (int n = 0; n < kOut; ++n) v = fmaf(net.W3[n][j], sh.gbar[c][n], v);
+        sh.v3[c][j] = v * (1.0f / 48.0f);
+    }
+    __syncthreads();
+
+    // ---- the relaxation's part of dL/dm, one warp (the others run ahead)
+    if (w == kNetWarps - 1 && lane < kCells) {
+        const long long cell = cell0 + lane;
+        const bool valid = cell < a.d.ncell;
+        const float* m = sh.m[lane];
+        float* mu_row = sh.mu[lane];
+        const float omega_nu = 1.0f / a.tau;
+        const float irho = 1.0f / m[0];
+        float dm[Q];
 #pragma unroll
         for (int e = 0; e < Q; ++e) dm[e] = 0.0f;
-    }
-    // d omega / d tau~ = sigma (1 - sigma) / (2 tau_n^2), sigma = 1 / (1 + e^{tau~})
-    float gbar[kOut];
 #pragma unroll
-    for (int n = 0; n < kOut; ++n) {
-        const float sg = 1.0f / (1.0f + expf(ttil[n]));
-        gbar[n] = valid ? gw[n] * sg * (1.0f - sg) / (2.0f * tau_n[n] * tau_n[n]) : 0.0f;
-        sh.tail[tid][n] = gbar[n];
-    }
-    // cotangent of the last hidden layer (the same for every group element): W3^T gbar / 48
-    float v3[kHidden];
+        for (int e = 0; e < Q; ++e) {
+            const int n = order_of(e);
+            const float mu = mu_row[e];
+            if (n <= 1) {
+                dm[e] += mu;
+            } else if (n == 2) {
+                dm[e] += (1.0f - omega_nu) * mu;
+                // m^eq_e = m_a m_b / m_0 for the axes a, b of component e
+                const int ex = ex_of(e), ey = ey_of(e), ez = ez_of(e);
+                int ia = -1, ib = -1, axa = 0, axb = 0;
+                const int cnt[3] = {ex, ey, ez};
+                const int idx[3] = {1, 3, 9};
 #pragma unroll
-    for (int j = 0; j < kHidden; ++j) {
-        float acc = 0.0f;
-#pragma unroll
-        for (int n = 0; n < kOut; ++n) acc = fmaf(net.W3[n][j], gbar[n], acc);
-        v3[j] = acc * (1.0f / 48.0f);
-    }
-
-    // ---- backward through the 48 copies of Phi, with block-level weight gradients
-    // thread roles in the outer-product accumulation
-    const bool w2_role = tid < 40;                 // dW2|db2 (and dWd|dbd): rows 2r.., cols 6c.. (20 x 24)
-    const bool w1_role = tid >= 40 && tid < 110;   // dW1p|db1: rows 2r.., cols 4c.. (20 x 28)
-    const int w2_r = (tid % 10) * 2, w2_c = (tid / 10) * 6;
-    const int w1_r = ((tid - 40) % 10) * 2, w1_c = ((tid - 40) / 10) * 4;
-    float acc2[2][6], accd[2][6], acc1[2][4];
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-#pragma unroll
-        for (int v = 0; v < 6; ++v) {
-            acc2[u][v] = 0.0f;
-            accd[u][v] = 0.0f;
-        }
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc1[u][v] = 0.0f;
-    }
-    // the moments and the bias input of every cell, for the first layer's weight gradient
-#pragma unroll
-    for (int t = 0; t < Q; ++t) st.xm[tid][t] = m[t];
-    st.xm[tid][Q] = 1.0f;
-    // the first-layer gradient columns of this thread and their parity classes (the bias
-    // column Q belongs to class 0: all its signs are +)
-    int w1_cls[4];
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-        const int col = w1_role ? w1_c + v : 0;
-        w1_cls[v] = col < Q ? adj_odd_mask(col) : 0;
-    }
-#pragma unroll 1
-    for (int p = p_begin; p < p_end; ++p) {
-        first_layer(p);
-#pragma unroll 1
-        for (int sv = 0; sv < 8; ++sv) {
-            float h1[kHidden];
-#pragma unroll
-            for (int j = 0; j < kHidden; ++j) h1[j] = hb[sv * kHidden + j];
-            float dh2[kHidden];
-            if constexpr (DEEP) {
-                float h2[kHidden];
-#pragma unroll 2
-                for (int j = 0; j < kHidden; ++j) {
-                    float acc = net.b2[j];
-#pragma unroll
-                    for (int k = 0; k < kHidden; ++k) acc = fmaf(net.W2[j][k], h1[k], acc);
-                    h2[j] = fmaxf(acc, 0.0f);
+                for (int k = 0; k < 3; ++k) {
+                    if (cnt[k] == 2) { ia = idx[k]; ib = idx[k]; axa = axb = k; }
+                    if (cnt[k] == 1) {
+                        if (ia < 0) { ia = idx[k]; axa = k; }
+                        else { ib = idx[k]; axb = k; }
+                    }
                 }
-                float dh3[kHidden];
-#pragma unroll 2
-                for (int j = 0; j < kHidden; ++j) {
-                    float acc = net.bd[j];
-#pragma unroll
-                    for (int k = 0; k < kHidden; ++k) acc = fmaf(net.Wd[j][k], h2[k], acc);
-                    dh3[j] = acc > 0.0f ? v3[j] : 0.0f;
+                const float ma = m[ia], mb = m[ib];
+                const float c = omega_nu * mu;
+                dm[ia] += c * mb * irho;
+                dm[ib] += c * ma * irho;
+                dm[0] -= c * ma * mb * irho * irho;
+                if (a.force && valid) {
+                    // Kupershtokh source (Sec. II.A) in moment space: its only state-dependent part
+                    // is order 2, dm*_ab = 3 ((j + F)_a (j + F)_b - j_a j_b) / rho with m_a = sqrt3 j_a,
+                    // i.e. (sqrt3 (m_a F_b + F_a m_b) + 3 F_a F_b) / rho; the force is an input
+                    const float Fa = a.force[static_cast<size_t>(axa) * a.d.ncell + cell];
+                    const float Fb = a.force[static_cast<size_t>(axb) * a.d.ncell + cell];
+                    const float src = (kSqrt3 * (ma * Fb + Fa * mb) + 3.0f * Fa * Fb) * irho;
+                    dm[ia] += mu * kSqrt3 * Fb * irho;
+                    dm[ib] += mu * kSqrt3 * Fa * irho;
+                    dm[0] -= mu * src * irho;
                 }
-#pragma unroll 2
-                for (int k = 0; k < kHidden; ++k) {
-                    float acc = 0.0f;
-#pragma unroll
-                    for (int j = 0; j < kHidden; ++j) acc = fmaf(net.Wd[j][k], dh3[j], acc);
-                    dh2[k] = h2[k] > 0.0f ? acc : 0.0f;
-                }
-#pragma unroll
-                for (int j = 0; j < kHidden; ++j) {
-                    st.dh3[tid][j] = dh3[j];
-                    st.h2x[tid][j] = h2[j];
-                }
-                st.h2x[tid][kHidden] = 1.0f;
-#pragma unroll
-                for (int k = kHidden + 1; k < 24; ++k) st.h2x[tid][k] = 0.0f;
             } else {
-#pragma unroll 2
-                for (int j = 0; j < kHidden; ++j) {
-                    float acc = net.b2[j];
-#pragma unroll
-                    for (int k = 0; k < kHidden; ++k) acc = fmaf(net.W2[j][k], h1[k], acc);
-                    dh2[j] = acc > 0.0f ? v3[j] : 0.0f;
-                }
+                dm[e] += (1.0f - sh.rates[lane][n - 3]) * mu;
             }
-            // delta h1 replaces h1 in this thread's row
-#pragma unroll 2
-            for (int k = 0; k < kHidden; ++k) {
-                float acc = 0.0f;
-#pragma unroll
-                for (int j = 0; j < kHidden; ++j) acc = fmaf(net.W2[j][k], dh2[j], acc);
-                hb[sv * kHidden + k] = h1[k] > 0.0f ? acc : 0.0f;
-            }
-            // stage this sign vector for the second-layer weight-gradient outer products
-#pragma unroll
-            for (int j = 0; j < kHidden; ++j) {
-                st.dh2[tid][j] = dh2[j];
-                st.h1x[tid][j] = h1[j];
-            }
-            st.h1x[tid][kHidden] = 1.0f;
-#pragma unroll
-            for (int k = kHidden + 1; k < 24; ++k) st.h1x[tid][k] = 0.0f;
-            __syncthreads();
-            if (w2_role) {
-                for (int c = 0; c < kAdjThreads; ++c) {
-                    const float r0 = st.dh2[c][w2_r], r1 = st.dh2[c][w2_r + 1];
-#pragma unroll
-                    for (int v = 0; v < 6; ++v) {
-                        const float cv = st.h1x[c][w2_c + v];
-                        acc2[0][v] = fmaf(r0, cv, acc2[0][v]);
-                        acc2[1][v] = fmaf(r1, cv, acc2[1][v]);
-                    }
-                    if constexpr (DEEP) {
-                        const float d0 = st.dh3[c][w2_r], d1 = st.dh3[c][w2_r + 1];
-#pragma unroll
-                        for (int v = 0; v < 6; ++v) {
-                            const float cv = st.h2x[c][w2_c + v];
-                            accd[0][v] = fmaf(d0, cv, accd[0][v]);
-                            accd[1][v] = fmaf(d1, cv, accd[1][v]);
-                        }
-                    }
-                }
-            }
-            __syncthreads();
         }
-        // E[c][j] = sum_s (-1)^popcount(s & c) delta h1[s][j], in place, and the first
-        // layer's cotangent of m: sum_s sgn(s, t) (W1p^T delta h1[s])_t = (W1p^T E[c(t)])_t
-#pragma unroll 2
-        for (int j = 0; j < kHidden; ++j) {
-            float e[8];
 #pragma unroll
-            for (int c = 0; c < 8; ++c) e[c] = hb[c * kHidden + j];
-            wht8(e);
-#pragma unroll
-            for (int c = 0; c < 8; ++c) hb[c * kHidden + j] = e[c];
-#pragma unroll
-            for (int t = 0; t < Q; ++t) dm[t] = fmaf(net.W1p[p][j][t], e[adj_odd_mask(t)], dm[t]);
-        }
-        __syncthreads();  // every cell's E is in place
-        if (w1_role) {  // dW1p[j][t] += sum over cells of E[c(t)][j] m_t (db1 through the bias column)
-            for (int c = 0; c < kAdjThreads; ++c) {
-                const float* ec = sh.hb + c * kHbStride;
-#pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    const float cv = st.xm[c][w1_c + v];
-                    acc1[0][v] = fmaf(ec[w1_cls[v] * kHidden + w1_r], cv, acc1[0][v]);
-                    acc1[1][v] = fmaf(ec[w1_cls[v] * kHidden + w1_r + 1], cv, acc1[1][v]);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < 2; ++u)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    const int j = w1_r + u, col = w1_c + v;
-                    if (col < Q) atomicAdd(&a.grad[p * kHidden * Q + j * Q + col], static_cast<double>(acc1[u][v]));
-                    else if (col == Q) atomicAdd(&a.grad[GL::kB1 + j], static_cast<double>(acc1[u][v]));
-                    acc1[u][v] = 0.0f;
-                }
-        }
-        __syncthreads();  // the rows are refilled by the next permutation
+        for (int e = 0; e < Q; ++e) mu_row[e] = dm[e];
     }
-    if (w2_role) {
-#pragma unroll
-        for (int u = 0; u < 2; ++u)
-#pragma unroll
-            for (int v = 0; v < 6; ++v) {
-                const int j = w2_r + u, col = w2_c + v;
-                if (col < kHidden) atomicAdd(&a.grad[GL::kW2 + j * kHidden + col], static_cast<double>(acc2[u][v]));
-                else if (col == kHidden) atomicAdd(&a.grad[GL::kB2 + j], static_cast<double>(acc2[u][v]));
-                if constexpr (DEEP) {
-                    if (col < kHidden) atomicAdd(&a.grad[GL::kWd + j * kHidden + col], static_cast<double>(accd[u][v]));
-                    else if (col == kHidden) atomicAdd(&a.grad[GL::kBd + j], static_cast<double>(accd[u][v]));
-                }
-            }
-    }
-    // output layer: dW3[n][j] += gbar_n * hmean_j, db3[n] += gbar_n (block sums via shared memory)
-    __syncthreads();
-    if (part == 0 && tid < kOut * (kHidden + 1)) {
-        const int n = tid / (kHidden + 1), j = tid % (kHidden + 1);
-        float acc = 0.0f;
-        for (int c = 0; c < kAdjThreads; ++c) acc = fmaf(sh.tail[c][n], j < kHidden ? sh.tail[c][4 + j] : 1.0f, acc);
-        if (j < kHidden) atomicAdd(&a.grad[GL::kW3 + n * kHidden + j], static_cast<double>(acc));
-        else atomicAdd(&a.grad[GL::kB3 + n], static_cast<double>(acc));
-    }
+    __syncwarp();
 
-    // ---- lam_t = M^T dL/dm (summed over the parts of a tile into a zeroed buffer)
-    if (valid) {
-        moments_transpose_inplace(dm);
-        float* out = a.lam_out + cell;
-        if (a.nparts == 1) {
+    // units j..j+3 of the last hidden layer's cotangent where they are on: v3 of the cell at a
+    // row, and the bits k of a column
+    auto masked = [](const float4& v, uint32_t k) {
+        return make_float4(static_cast<int>(k) < 0 ? v.x : 0.0f, static_cast<int>(k << 1) < 0 ? v.y : 0.0f,
+                           static_cast<int>(k << 2) < 0 ? v.z : 0.0f, static_cast<int>(k << 3) < 0 ? v.w : 0.0f);
+    };
+    auto v3_at = [&](int r, int j) { return *reinterpret_cast<const float4*>(&sh.v3[r % kCells][j]); };
+    auto last_columns = [&](int j, float4(&v)[2][C]) {
 #pragma unroll
-            for (int i = 0; i < Q; ++i) out[static_cast<size_t>(i) * a.d.ncell] = dm[i];
-        } else {
+        for (int r = 0; r < 2; ++r) {
+            const float4 t = v3_at(l + 16 * r, j);
 #pragma unroll
-            for (int i = 0; i < Q; ++i) atomicAdd(out + static_cast<size_t>(i) * a.d.ncell, dm[i]);
+            for (int c = 0; c < C; ++c) v[r][c] = masked(t, mask[r][c] << j);
         }
+    };
+    // weight gradient of the layer above the columns h: (v3 masked) times h, a column of every
+    // row staged at a time
+    auto last_layer_grad = [&](const float* h, float* out) {
+        OuterTile t;
+        t.clear();
+        float* const st = sh.stage[w];
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            const uint32_t k = og ? mask[1][c] : mask[0][c];
+#pragma unroll
+            for (int j = 0; j < kHidden; j += 4)
+                *reinterpret_cast<float4*>(st + lane * kHidden + j) = masked(v3_at(lane, j), k << j);
+            __syncwarp();
+            t.add(st, kHidden, h + c * kHidden, kRow, lane);
+            __syncwarp();
+        }
+        t.flush(out, lane);
+    };
+    // acc where the unit is on in x replaces x
+    auto gate_into = [&](float* x, const float(&acc)[2][C][kHalf]) {
+        x += og * kHalf;
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int c = 0; c < C; ++c)
+#pragma unroll
+                for (int o = 0; o < kHalf; o += 2) {
+                    float2* const q = reinterpret_cast<float2*>(x + 16 * r * kRow + c * kHidden + o);
+                    const float2 h = *q;
+                    *q = make_float2(h.x > 0.0f ? acc[r][c][o] : 0.0f, h.y > 0.0f ? acc[r][c][o + 1] : 0.0f);
+                }
+    };
+
+    // ---- backward through the hidden layers
+    if constexpr (DEEP) {
+        float* const rows2 = &sh.h2[w][0][0];
+        float* const row2 = sh.h2[w][l];
+        last_layer_grad(rows2, sh.stage[w]);
+        {
+            float acc[2][C][kHalf] = {};
+            mat_vec<C>(net.WdT, lane, acc, last_columns);
+            gate_into(row2, acc);  // delta h2
+        }
+        __syncwarp();
+        {
+            OuterTile t;
+            t.clear();
+#pragma unroll 1
+            for (int c = 0; c < C; ++c) t.add(rows2 + c * kHidden, kRow, rows + c * kHidden, kRow, lane);
+            t.flush(sh.stage[w] + kGradBlock, lane);
+        }
+        __syncwarp();
+        float acc[2][C][kHalf] = {};
+        mat_vec<C>(net.W2T, lane, acc, RowColumns<C>{row2});
+        gate_into(row, acc);  // delta h1
+    } else {
+        last_layer_grad(rows, sh.stage[w]);
+        float acc[2][C][kHalf] = {};
+        mat_vec<C>(net.W2T, lane, acc, last_columns);
+        gate_into(row, acc);  // delta h1
+    }
+    pair_sync(p);
+
+    // ---- first layer: E of class c in place of delta h1 of sign vector c, and the cotangent of
+    // m through the lane's five units
+    {
+        using At = ColumnOf<LANES>;
+        constexpr int NC = 2 / LANES;
+        float dm[NC][Q];
+#pragma unroll
+        for (int k = 0; k < NC; ++k)
+#pragma unroll
+            for (int t = 0; t < Q; ++t) dm[k][t] = 0.0f;
+        const int j0 = half * kHalf + og * 5;
+        float* const q = &sh.h1[2 * p][l][j0];
+#pragma unroll 1
+        for (int i = 0; i < 5; ++i) {
+            float wt[28];
+#pragma unroll
+            for (int t = 0; t < 28; t += 4)
+                *reinterpret_cast<float4*>(wt + t) = *reinterpret_cast<const float4*>(&net.W1p[p][j0 + i][t]);
+#pragma unroll
+            for (int k = 0; k < NC; ++k) {
+                float e[8];
+                auto at = [&](int s) -> float& {
+                    return q[(At::half(s) * 32 + At::row(s) + 16 * k) * kRow + At::col(s) * kHidden + i];
+                };
+#pragma unroll
+                for (int s = 0; s < 8; ++s) e[s] = at(s);
+                wht<8>(e);
+#pragma unroll
+                for (int s = 0; s < 8; ++s) at(s) = e[s];
+#pragma unroll
+                for (int t = 0; t < Q; ++t) dm[k][t] = fmaf(wt[t], e[odd_mask(t)], dm[k][t]);
+            }
+        }
+        pair_sync(p);
+        // dW1p[j][t] = sum over cells of E[c(t)][j] m_t, lane t (lane 27: db1, the bias input of class 0)
+        {
+            const int t = lane < Q ? lane : Q;
+            const int ex = t % 3, ey = (t / 3) % 3, ez = t / 9;
+            const int c = t < Q ? ((ex == 1) << 2) | ((ey == 1) << 1) | (ez == 1) : 0;
+            const float* er = &sh.h1[2 * p + At::half(c)][At::row(c)][At::col(c) * kHidden + half * kHalf];
+            float g[kHalf];
+#pragma unroll
+            for (int j = 0; j < kHalf; ++j) g[j] = 0.0f;
+#pragma unroll 2
+            for (int r = 0; r < kCells; ++r) {
+                const float mt = sh.m[r][t];
+#pragma unroll
+                for (int j = 0; j < kHalf; j += 2) {
+                    const float2 v = *reinterpret_cast<const float2*>(er + r * kRow + j);
+                    g[j] = fmaf(v.x, mt, g[j]);
+                    g[j + 1] = fmaf(v.y, mt, g[j + 1]);
+                }
+            }
+            if (lane <= Q) {
+#pragma unroll
+                for (int j = 0; j < kHalf; ++j) sh.stage[w][SH::kD1 + t * kHalf + j] = g[j];
+            }
+        }
+        pair_sync(p);
+        // the rows are free: the two five-unit parts of the cells' cotangents, [t][og][cell]
+#pragma unroll
+        for (int t = 0; t < Q; ++t)
+#pragma unroll
+            for (int k = 0; k < NC; ++k) rows[(2 * t + og) * kCells + l + 16 * k] = dm[k][t];
+    }
+    __syncthreads();
+    for (int i = tid; i < Q * kCells; i += kAdjThreads) {  // the twelve warps' parts and the relaxation's
+        const int t = i / kCells, c = i % kCells;
+        float v = sh.mu[c][t];
+#pragma unroll
+        for (int q = 0; q < kNetWarps; ++q)
+#pragma unroll
+            for (int g = 0; g < 2; ++g) v += (&sh.h1[q][0][0])[(2 * t + g) * kCells + c];
+        sh.dm[t][c] = v;
+    }
+    __syncthreads();
+
+    if (w == 0) {  // lam_t = M^T dL/dm
+        const long long cell = cell0 + lane;
+        if (lane < kCells && cell < a.d.ncell) {
+            float v[Q];
+#pragma unroll
+            for (int e = 0; e < Q; ++e) v[e] = sh.dm[e][lane];
+            moments_transpose_inplace(v);
+#pragma unroll
+            for (int i = 0; i < Q; ++i) a.lam_out[static_cast<size_t>(i) * a.d.ncell + cell] = v[i];
+        }
+        return;
+    }
+    // parameter gradients of the tile, one per thread: sums over the warps (W1: the six
+    // permutations' columns that a printed column went to), added in FP64
+    for (int i = tid - 32; i < GL::kLen; i += kAdjThreads - 32) {
+        float v = 0.0f;
+        if (i < GL::kW2) {
+            const int j = i < GL::kB1 ? i / Q : i - GL::kB1, k = i < GL::kB1 ? i % Q : Q;
+            const int h = j >= kHalf, jo = j - h * kHalf;
+#pragma unroll
+            for (int q = 0; q < 6; ++q) {
+                const int t = k < Q ? kPermColumns.t[q][k] : Q;
+                v += sh.stage[2 * q + h][SH::kD1 + t * kHalf + jo];
+            }
+        } else if (i < GL::kW3) {
+            // stage: with the third hidden layer (Wd | bd) then (W2 | b2), else (W2 | b2)
+            int o = i - GL::kW2;
+            if (DEEP) o = o < kGradBlock ? o + kGradBlock : o - kGradBlock;
+#pragma unroll
+            for (int q = 0; q < kNetWarps; ++q) v += sh.stage[q][o];
+        } else {
+            const int o = i - GL::kW3;
+            const int n = o < kOut * kHidden ? o / kHidden : o - kOut * kHidden;
+            for (int c = 0; c < kCells; ++c)
+                v = fmaf(sh.gbar[c][n], o < kOut * kHidden ? sh.hsum[c][o % kHidden] * (1.0f / 48.0f) : 1.0f, v);
+        }
+        atomicAdd(&a.grad[i], static_cast<double>(v));
     }
 }
 
@@ -581,78 +648,41 @@ cudaError_t launch_adjoint_seed(const Dims& d, int storage, int bc, const void* 
     return cudaGetLastError();
 }
 
-template <int BC, bool DEEP>
-static cudaError_t launch_adjoint_step_t(const AdjArgs& a, const NetParams& net, cudaStream_t s) {
-    constexpr size_t smem = sizeof(AdjShared<DEEP>);
+template <int BC, bool DEEP, int LANES>
+static cudaError_t launch_adjoint_step_t(const AdjArgs& a, const NetParams* net, cudaStream_t s) {
+    using SH = AdjShared<DEEP, LANES>;
+    constexpr size_t smem = sizeof(SH);
+    static_assert(smem <= 227 * 1024, "shared memory budget");
     static std::atomic<unsigned long long> attr{0};  // one set of per-device flags per instantiation
-    {
-        const cudaError_t e = ensure_dynamic_smem(adjoint_step_kernel<LBM_STORE_F32, BC, DEEP>, static_cast<int>(smem),
-                                                  attr);
-        if (e != cudaSuccess) return e;
-    }
-    const long long tiles = (a.d.ncell + kAdjThreads - 1) / kAdjThreads;
-    if (a.nparts > 1) {
-        const cudaError_t e = cudaMemsetAsync(a.lam_out, 0, sizeof(float) * Q * static_cast<size_t>(a.d.ncell), s);
-        if (e != cudaSuccess) return e;
-    }
-    const dim3 grid(static_cast<unsigned>(tiles * a.nparts));
-    adjoint_step_kernel<LBM_STORE_F32, BC, DEEP><<<grid, kAdjThreads, smem, s>>>(a, net);
+    const cudaError_t e = ensure_dynamic_smem(adjoint_step_kernel<LBM_STORE_F32, BC, DEEP, LANES>,
+                                              static_cast<int>(smem), attr);
+    if (e != cudaSuccess) return e;
+    const unsigned grid = static_cast<unsigned>((a.d.ncell + SH::kCells - 1) / SH::kCells);
+    adjoint_step_kernel<LBM_STORE_F32, BC, DEEP, LANES><<<grid, kAdjThreads, smem, s>>>(a, net);
     return cudaGetLastError();
 }
 
-template <bool DEEP>
-static cudaError_t launch_adjoint_step_bc(const AdjArgs& a, int bc, const NetParams& net, cudaStream_t s) {
+template <int BC>
+static cudaError_t launch_adjoint_step_bc(const AdjArgs& a, bool deep, const NetParams* net, cudaStream_t s) {
+    return deep ? launch_adjoint_step_t<BC, true, 2>(a, net, s) : launch_adjoint_step_t<BC, false, 1>(a, net, s);
+}
+
+cudaError_t launch_adjoint_step(const Dims& d, int storage, int bc, const void* state, const float* lam_in,
+                                float* lam_out, double* grad, float tau, const float* force, bool deep,
+                                const NetParams* d_net, cudaStream_t s) {
+    if (storage != LBM_STORE_F32) return cudaErrorInvalidValue;
+    const AdjArgs a{d, state, lam_in, lam_out, grad, tau, force};
     switch (bc) {
-        case LBM_BC_PERIODIC: return launch_adjoint_step_t<LBM_BC_PERIODIC, DEEP>(a, net, s);
-        case LBM_BC_MIRROR: return launch_adjoint_step_t<LBM_BC_MIRROR, DEEP>(a, net, s);
-        case LBM_BC_TGV_REDUCED: return launch_adjoint_step_t<LBM_BC_TGV_REDUCED, DEEP>(a, net, s);
+        case LBM_BC_PERIODIC: return launch_adjoint_step_bc<LBM_BC_PERIODIC>(a, deep, d_net, s);
+        case LBM_BC_MIRROR: return launch_adjoint_step_bc<LBM_BC_MIRROR>(a, deep, d_net, s);
+        case LBM_BC_TGV_REDUCED: return launch_adjoint_step_bc<LBM_BC_TGV_REDUCED>(a, deep, d_net, s);
         default: return cudaErrorInvalidValue;
     }
 }
 
-cudaError_t launch_adjoint_step(const Dims& d, int storage, int bc, const void* state, const float* lam_in,
-                                float* lam_out, double* grad, float tau, const float* force, const NetParams& net,
-                                cudaStream_t s) {
-    if (storage != LBM_STORE_F32) return cudaErrorInvalidValue;
-    // grids of fewer tiles than SMs (the small domains of training): split the 6 axis
-    // permutations of a tile over 2, 3 or 6 blocks so that every SM gets work; from one tile
-    // per SM on, the forward that every part recomputes costs more than it brings
-    // (measured: 16^3 with 32 tiles, 6 parts, 1.74 x faster; 32^3 with 256 tiles, 2 parts,
-    // 15 % slower)
-    const long long tiles = (d.ncell + kAdjThreads - 1) / kAdjThreads;
-    const long long want = sm_count();
-    const int nparts = tiles >= want ? 1 : tiles * 2 >= want ? 2 : tiles * 3 >= want ? 3 : 6;
-    AdjArgs a{d, state, lam_in, lam_out, grad, tau, force, nparts};
-    return net.deep ? launch_adjoint_step_bc<true>(a, bc, net, s) : launch_adjoint_step_bc<false>(a, bc, net, s);
-}
-
-// Fold the accumulator into the flat parameter order W1, b1, W2, b2, (Wd, bd), W3, b3 (W1
-// in the printed column order): dW1[j][k] = sum_p dW1p[p][j][t_p(k)].
-template <bool DEEP>
-static void fold_gradient(const double* acc, float* out) {
-    using GL = GradLayout<DEEP>;
-    const GroupTables& g = group_tables();
-    for (int j = 0; j < kHidden; ++j)
-        for (int k = 0; k < Q; ++k) {
-            double v = 0.0;
-            for (int p = 0; p < 6; ++p) v += acc[p * kHidden * Q + j * Q + g.mperm_t[p * 8][kPrinted.e[k]]];
-            out[j * Q + k] = static_cast<float>(v);
-        }
-    float* o = out + kHidden * Q;
-    for (int j = 0; j < kHidden; ++j) *o++ = static_cast<float>(acc[GL::kB1 + j]);
-    for (int j = 0; j < kHidden * kHidden; ++j) *o++ = static_cast<float>(acc[GL::kW2 + j]);
-    for (int j = 0; j < kHidden; ++j) *o++ = static_cast<float>(acc[GL::kB2 + j]);
-    if (DEEP) {
-        for (int j = 0; j < kHidden * kHidden; ++j) *o++ = static_cast<float>(acc[GL::kWd + j]);
-        for (int j = 0; j < kHidden; ++j) *o++ = static_cast<float>(acc[GL::kBd + j]);
-    }
-    for (int j = 0; j < kOut * kHidden; ++j) *o++ = static_cast<float>(acc[GL::kW3 + j]);
-    for (int j = 0; j < kOut; ++j) *o++ = static_cast<float>(acc[GL::kB3 + j]);
-}
-
 void adjoint_fold_gradient(const double* acc, bool deep, float* out) {
-    if (deep) fold_gradient<true>(acc, out);
-    else fold_gradient<false>(acc, out);
+    const int n = adjoint_grad_len(deep);
+    for (int i = 0; i < n; ++i) out[i] = static_cast<float>(acc[i]);
 }
 
 }  // namespace lbm

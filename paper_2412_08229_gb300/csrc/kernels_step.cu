@@ -1,5 +1,5 @@
 // kernels_step.cu - the fused pull-stream-collide step (Sec. II.A-B) with the BGK, KBC
-// and FP32 neural-collision operators, plus state set/get, macroscopic fields and the
+// and REG operators, plus state set/get, macroscopic fields and the
 // FP64 kinetic-energy reduction.
 //
 // One thread per cell; consecutive threads take consecutive x, so every one of the 27
@@ -16,101 +16,10 @@ namespace lbm {
 
 constexpr int kStepThreads = 128;
 
-// ---------------------------------------------------------------------------
-// FP32 invariant network N_Phi (Sec. II.B, eq. gconv_m) evaluated per cell.
-// The 48 elements of O_h are (axis permutation p, sign vector s). For element (p, s)
-// the network input in the printed moment order is P_g m; with the columns of W1
-// rearranged per p (W1p, built on the host from the group tables) the first layer
-// reads sgn(s, t) * m_t in tensor order t, where sgn flips the moments that are odd
-// in a reflected axis: sgn(s, t) = (-1)^popcount(s & c(t)) with c(t) the parity class of
-// t (which axes t is odd in). Grouping the first layer's sum by class, the 8 sign
-// vectors of one permutation are an 8-point Walsh-Hadamard transform of the 8 class
-// sums y_c = sum_{t in class c} W1p[:, t] m_t: 20 x 27 MAC and 20 x 24 additions per
-// permutation instead of 8 x 20 x 27 MAC. The relu'd first-layer outputs of the 8 sign
-// vectors are staged in shared memory, one column per thread, and read back per sign
-// vector for the layers after it. The output layer is affine, so the group mean is taken
-// on the last hidden layer first (h2, or h3 for the 1484-parameter network with a third
-// hidden layer).
-// ---------------------------------------------------------------------------
-constexpr int kNcoThreads = 64;  // block of the FP32 network kernel: 8 x 20 x 64 floats of staging
-
-__device__ __forceinline__ int odd_mask(int t) {
-    return ((ex_of(t) == 1) << 2) | ((ey_of(t) == 1) << 1) | (ez_of(t) == 1);
-}
-
-__device__ __forceinline__ void nco_rates_f32(const float* m, const NetParams& net, float* rates) {
-    __shared__ float h1s[8 * kHidden * kNcoThreads];  // [s][j][thread]: each thread its own column
-    float* col = h1s + threadIdx.x;
-    float acc[kHidden];
-#pragma unroll
-    for (int j = 0; j < kHidden; ++j) acc[j] = 0.0f;
-#pragma unroll 1
-    for (int p = 0; p < 6; ++p) {
-#pragma unroll
-        for (int j = 0; j < kHidden; ++j) {
-            float y[8];
-#pragma unroll
-            for (int c = 0; c < 8; ++c) y[c] = 0.0f;
-#pragma unroll
-            for (int t = 0; t < Q; ++t) y[odd_mask(t)] = fmaf(net.W1p[p][j][t], m[t], y[odd_mask(t)]);
-            // H[s] = sum_c (-1)^popcount(s & c) y[c], in place
-#pragma unroll
-            for (int bit = 1; bit < 8; bit <<= 1)
-#pragma unroll
-                for (int c = 0; c < 8; ++c)
-                    if (!(c & bit)) {
-                        const float u = y[c], v = y[c | bit];
-                        y[c] = u + v;
-                        y[c | bit] = u - v;
-                    }
-#pragma unroll
-            for (int sv = 0; sv < 8; ++sv) col[(sv * kHidden + j) * kNcoThreads] = fmaxf(y[sv] + net.b1[j], 0.0f);
-        }
-#pragma unroll 1
-        for (int sv = 0; sv < 8; ++sv) {
-            float h1[kHidden];
-#pragma unroll
-            for (int j = 0; j < kHidden; ++j) h1[j] = col[(sv * kHidden + j) * kNcoThreads];
-            if (net.deep) {  // 27-20-20-20-4: a third hidden layer before the group sum
-                float h2[kHidden];
-#pragma unroll
-                for (int j = 0; j < kHidden; ++j) {
-                    float a = net.b2[j];
-#pragma unroll
-                    for (int k = 0; k < kHidden; ++k) a = fmaf(net.W2[j][k], h1[k], a);
-                    h2[j] = fmaxf(a, 0.0f);
-                }
-#pragma unroll
-                for (int j = 0; j < kHidden; ++j) {
-                    float a = net.bd[j];
-#pragma unroll
-                    for (int k = 0; k < kHidden; ++k) a = fmaf(net.Wd[j][k], h2[k], a);
-                    acc[j] += fmaxf(a, 0.0f);
-                }
-            } else {
-#pragma unroll
-                for (int j = 0; j < kHidden; ++j) {
-                    float a = net.b2[j];
-#pragma unroll
-                    for (int k = 0; k < kHidden; ++k) a = fmaf(net.W2[j][k], h1[k], a);
-                    acc[j] += fmaxf(a, 0.0f);
-                }
-            }
-        }
-    }
-#pragma unroll
-    for (int n = 0; n < kOut; ++n) {
-        float a = 0.0f;
-#pragma unroll
-        for (int j = 0; j < kHidden; ++j) a = fmaf(net.W3[n][j], acc[j], a);
-        rates[n] = rate_from_output(a * (1.0f / 48.0f) + net.b3[n]);
-    }
-}
-
 // Collision of one cell's pulled deviations df, in place; reports a density outside the
 // window and returns the cell's pre-collision macroscopic state.
 template <int OP>
-__device__ __forceinline__ Macro collide_cell(const StepArgs& a, float* df, const NetParams* net) {
+__device__ __forceinline__ Macro collide_cell(const StepArgs& a, float* df) {
     Macro q;
     if constexpr (OP == LBM_OP_KBC) {  // needs only rho, u and the second-order moments
         float s2[6];
@@ -125,27 +34,23 @@ __device__ __forceinline__ Macro collide_cell(const StepArgs& a, float* df, cons
         const float omega = 1.0f / a.tau;
         if constexpr (OP == LBM_OP_BGK) {
             collide_bgk(df, q, omega);
-        } else if constexpr (OP == LBM_OP_REG) {  // orders 3..6 relaxed with rate 1
+        } else {  // REG: orders 3..6 relaxed with rate 1
             const float ones[kOut] = {1.0f, 1.0f, 1.0f, 1.0f};
             collide_mrt(df, m, q, omega, ones);
-        } else {
-            float rates[kOut];
-            nco_rates_f32(m, *net, rates);
-            collide_mrt(df, m, q, omega, rates);
         }
     }
     return q;
 }
 
 template <int OP, int STORAGE, int BC>
-__device__ __forceinline__ void step_body(const StepArgs& a, const NetParams* net) {
+__device__ __forceinline__ void step_body(const StepArgs& a) {
     const long long cell = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (cell >= a.d.ncell) return;
     int x, y, z;
     cell_coords(cell, a.d, x, y, z);
     float df[Q];
     load_pulled_offsets<STORAGE, BC>(a.src, a.d, x, y, z, df);
-    collide_cell<OP>(a, df, net);
+    collide_cell<OP>(a, df);
     store_cell<STORAGE>(a.dst, a.d, cell, df);
 }
 
@@ -156,7 +61,7 @@ __device__ __forceinline__ void step_body(const StepArgs& a, const NetParams* ne
 // coefficients (force.cuh). Every lane of a warp takes part in the projection; lanes past
 // the last cell contribute zero.
 template <int OP, int STORAGE, int BC>
-__device__ __forceinline__ void step_body_forced(const StepArgs& a, const FusedForce& ff, const NetParams* net) {
+__device__ __forceinline__ void step_body_forced(const StepArgs& a, const FusedForce& ff) {
     __shared__ float fh2[kForcedModes * 6];
     __shared__ unsigned long long red[frc::kProjValues];
     frc::load_fh2(ff.fhat, fh2);
@@ -175,7 +80,7 @@ __device__ __forceinline__ void step_body_forced(const StepArgs& a, const FusedF
         if (valid) {
             cell_coords(cell, a.d, x, y, z);
             load_pulled_offsets<STORAGE, BC>(a.src, a.d, x, y, z, df);
-            q = collide_cell<OP>(a, df, net);
+            q = collide_cell<OP>(a, df);
         }
         frc::Cx p[kForcedModes];
         frc::cell_phases(x, y, z, a.d, ff.tab, p);
@@ -197,16 +102,8 @@ __device__ __forceinline__ void step_body_forced(const StepArgs& a, const FusedF
 template <int OP, int STORAGE, int BC, bool FORCED>
 __global__ void __launch_bounds__(kStepThreads, OP == LBM_OP_KBC && !FORCED ? 7 : 1)
     step_kernel(const StepArgs a, const FusedForce ff) {
-    if constexpr (FORCED) step_body_forced<OP, STORAGE, BC>(a, ff, nullptr);
-    else step_body<OP, STORAGE, BC>(a, nullptr);
-}
-
-template <int STORAGE, int BC, bool FORCED>
-__global__ void __launch_bounds__(kNcoThreads) step_nco_f32_kernel(const StepArgs a,
-                                                                    const __grid_constant__ NetParams net,
-                                                                    const FusedForce ff) {
-    if constexpr (FORCED) step_body_forced<LBM_OP_NCO, STORAGE, BC>(a, ff, &net);
-    else step_body<LBM_OP_NCO, STORAGE, BC>(a, &net);
+    if constexpr (FORCED) step_body_forced<OP, STORAGE, BC>(a, ff);
+    else step_body<OP, STORAGE, BC>(a);
 }
 
 // Blocks of a forced launch: as many as are resident at once (the grid strides over the
@@ -238,45 +135,37 @@ static cudaError_t launch_op(const StepArgs& a, const FusedForce& ff, cudaStream
 }
 
 template <int STORAGE, int BC, bool FORCED>
-static cudaError_t launch_step_t(const StepArgs& a, const FusedForce& ff, int op, const NetParams* net,
-                                 cudaStream_t s) {
+static cudaError_t launch_step_t(const StepArgs& a, const FusedForce& ff, int op, cudaStream_t s) {
     if (op == LBM_OP_BGK) return launch_op<LBM_OP_BGK, STORAGE, BC, FORCED>(a, ff, s);
     if (op == LBM_OP_KBC) return launch_op<LBM_OP_KBC, STORAGE, BC, FORCED>(a, ff, s);
-    if (op == LBM_OP_REG) return launch_op<LBM_OP_REG, STORAGE, BC, FORCED>(a, ff, s);
-    unsigned grid = static_cast<unsigned>((a.d.ncell + kNcoThreads - 1) / kNcoThreads);
-    if constexpr (FORCED) {
-        static std::atomic<int> occ{0};
-        grid = forced_grid(step_nco_f32_kernel<STORAGE, BC, true>, kNcoThreads, occ, a.d.ncell);
-    }
-    step_nco_f32_kernel<STORAGE, BC, FORCED><<<grid, kNcoThreads, 0, s>>>(a, *net, ff);
-    return cudaGetLastError();
+    return launch_op<LBM_OP_REG, STORAGE, BC, FORCED>(a, ff, s);
 }
 
 // Forcing runs on periodic boxes only (contexts refuse it on the other boundaries).
 template <int STORAGE>
-static cudaError_t launch_step_s(const StepArgs& a, const FusedForce* ff, int op, int bc, const NetParams* net,
-                                 cudaStream_t s) {
+static cudaError_t launch_step_s(const StepArgs& a, const FusedForce* ff, int op, int bc, cudaStream_t s) {
     const FusedForce none{};
     if (ff) {
         if (bc != LBM_BC_PERIODIC) return cudaErrorInvalidValue;
-        return launch_step_t<STORAGE, LBM_BC_PERIODIC, true>(a, *ff, op, net, s);
+        return launch_step_t<STORAGE, LBM_BC_PERIODIC, true>(a, *ff, op, s);
     }
-    if (bc == LBM_BC_PERIODIC) return launch_step_t<STORAGE, LBM_BC_PERIODIC, false>(a, none, op, net, s);
-    if (bc == LBM_BC_TGV_REDUCED) return launch_step_t<STORAGE, LBM_BC_TGV_REDUCED, false>(a, none, op, net, s);
-    return launch_step_t<STORAGE, LBM_BC_MIRROR, false>(a, none, op, net, s);
+    if (bc == LBM_BC_PERIODIC) return launch_step_t<STORAGE, LBM_BC_PERIODIC, false>(a, none, op, s);
+    if (bc == LBM_BC_TGV_REDUCED) return launch_step_t<STORAGE, LBM_BC_TGV_REDUCED, false>(a, none, op, s);
+    return launch_step_t<STORAGE, LBM_BC_MIRROR, false>(a, none, op, s);
 }
 
-cudaError_t launch_step(const StepArgs& a, const FusedForce* ff, int op, int storage, int bc, int net_prec,
-                        const NetParams* net, const void* tc_weights, int tc_shape, long long wait_cycles,
-                        cudaStream_t s) {
+cudaError_t launch_step(const StepArgs& a, const FusedForce* ff, int op, int storage, int bc, int net_prec, bool deep,
+                        const void* net_weights, int tc_shape, long long wait_cycles, cudaStream_t s) {
     if (op == LBM_OP_NCO && net_prec == LBM_NET_BF16)
-        return launch_step_nco_tc(a, ff, storage, bc, net && net->deep, tc_shape, wait_cycles, tc_weights, s);
+        return launch_step_nco_tc(a, ff, storage, bc, deep, tc_shape, wait_cycles, net_weights, s);
     if (op == LBM_OP_NCO && net_prec == LBM_NET_BF16X3)
-        return launch_step_nco_tc3(a, ff, storage, bc, net && net->deep, tc_weights, wait_cycles, s);
+        return launch_step_nco_tc3(a, ff, storage, bc, deep, net_weights, wait_cycles, s);
+    if (op == LBM_OP_NCO)
+        return launch_step_nco_f32(a, ff, storage, bc, deep, static_cast<const NetParams*>(net_weights), s);
     switch (storage) {
-        case LBM_STORE_F32: return launch_step_s<LBM_STORE_F32>(a, ff, op, bc, net, s);
-        case LBM_STORE_F16_DEV: return launch_step_s<LBM_STORE_F16_DEV>(a, ff, op, bc, net, s);
-        default: return launch_step_s<LBM_STORE_BF16_DEV>(a, ff, op, bc, net, s);
+        case LBM_STORE_F32: return launch_step_s<LBM_STORE_F32>(a, ff, op, bc, s);
+        case LBM_STORE_F16_DEV: return launch_step_s<LBM_STORE_F16_DEV>(a, ff, op, bc, s);
+        default: return launch_step_s<LBM_STORE_BF16_DEV>(a, ff, op, bc, s);
     }
 }
 

@@ -26,7 +26,7 @@ struct lbm_ctx {
     float tau = 0.5f;
     bool have_weights = false;
     NetParams* net = nullptr;  // host copy handed to FP32 NCO launches by value
-    void* tc_w = nullptr;      // device: packed BF16 operands of the tensor-core network
+    void* net_w = nullptr;     // device: NetParams of the FP32 network or the packed operands of a tensor-core network
     int* d_status = nullptr;
     double* d_partials = nullptr;
     int npart = 0;
@@ -255,27 +255,24 @@ void make_net_params(const float* theta, bool deep, NetParams* out) {
     const float* W3 = deep ? bd + kHidden : b2 + kHidden;
     const float* b3 = W3 + kOut * kHidden;
     const GroupTables& g = group_tables();
+    *out = NetParams{};
     for (int p = 0; p < 6; ++p) {
         const int gp = p * 8;  // element with axis permutation p and no reflection
-        for (int j = 0; j < kHidden; ++j)
-            for (int k = 0; k < Q; ++k) {
-                const int t = g.mperm_t[gp][kPrinted.e[k]];
-                out->W1p[p][j][t] = W1[j * Q + k];
-            }
+        for (int j = 0; j < kHidden; ++j) {
+            for (int k = 0; k < Q; ++k) out->W1p[p][j][g.mperm_t[gp][kPrinted.e[k]]] = W1[j * Q + k];
+            out->W1p[p][j][Q] = b1[j];
+        }
     }
-    std::memcpy(out->b1, b1, sizeof(out->b1));
-    std::memcpy(out->W2, W2, sizeof(out->W2));
+    for (int j = 0; j < kHidden; ++j)
+        for (int k = 0; k < kHidden; ++k) {
+            out->W2[j][k] = out->W2T[k][j] = W2[j * kHidden + k];
+            if (deep) out->Wd[j][k] = out->WdT[k][j] = Wd[j * kHidden + k];
+        }
     std::memcpy(out->b2, b2, sizeof(out->b2));
     std::memcpy(out->W3, W3, sizeof(out->W3));
     std::memcpy(out->b3, b3, sizeof(out->b3));
+    if (deep) std::memcpy(out->bd, bd, sizeof(out->bd));
     out->deep = deep ? 1 : 0;
-    if (deep) {
-        std::memcpy(out->Wd, Wd, sizeof(out->Wd));
-        std::memcpy(out->bd, bd, sizeof(out->bd));
-    } else {
-        std::memset(out->Wd, 0, sizeof(out->Wd));
-        std::memset(out->bd, 0, sizeof(out->bd));
-    }
 }
 
 }  // namespace lbm
@@ -430,7 +427,7 @@ lbm_status lbm_destroy(lbm_ctx* c) {
                         c->adj_lam[0] || c->adj_lam[1];
     free_recording(c);
     free_adjoint(c);
-    void* devs[] = {c->buf_base[0], c->buf_base[1], c->tc_w, c->d_status, c->d_partials, c->d_scalar, c->d_stage,
+    void* devs[] = {c->buf_base[0], c->buf_base[1], c->net_w, c->d_status, c->d_partials, c->d_scalar, c->d_stage,
                     c->d_fft, c->d_E, c->d_force, c->d_u, c->d_fproj, c->d_fhat, c->d_draws, c->d_sym,
                     c->d_fconst, c->d_ftab};
     for (void* p : devs)
@@ -507,8 +504,9 @@ lbm_status lbm_create(const lbm_config* cfg, void* stream, lbm_ctx** out) {
     c->npart = kinetic_energy_blocks(c->d);
     alloc(reinterpret_cast<void**>(&c->d_partials), sizeof(double) * c->npart);
     alloc(reinterpret_cast<void**>(&c->d_scalar), sizeof(double) * 2);
-    if (cfg->op == LBM_OP_NCO && cfg->net_precision == LBM_NET_BF16) alloc(&c->tc_w, nco_tc_weight_bytes());
-    if (cfg->op == LBM_OP_NCO && cfg->net_precision == LBM_NET_BF16X3) alloc(&c->tc_w, nco_tc3_weight_bytes());
+    if (cfg->op == LBM_OP_NCO && cfg->net_precision == LBM_NET_F32) alloc(&c->net_w, sizeof(NetParams));
+    if (cfg->op == LBM_OP_NCO && cfg->net_precision == LBM_NET_BF16) alloc(&c->net_w, nco_tc_weight_bytes());
+    if (cfg->op == LBM_OP_NCO && cfg->net_precision == LBM_NET_BF16X3) alloc(&c->net_w, nco_tc3_weight_bytes());
     if (cfg->boundary == LBM_BC_TGV_REDUCED) {
         SymRegion table[27];
         if (!tgv_reduced_table(table) && st == LBM_OK) st = fail(c, LBM_ERR_STATE, "reduced Taylor-Green table");
@@ -637,13 +635,16 @@ lbm_status nco_set_weights(lbm_ctx* c, const float* theta, int n) {
         if (!c->net) return fail(c, LBM_ERR_OOM, "nco_set_weights: host allocation failed");
     }
     make_net_params(h.data(), deep, c->net);
-    drop_step_graphs(c);  // the FP32 network's parameters are kernel arguments of the captured steps
-    if (c->tc_w) {
+    drop_step_graphs(c);  // the captured steps are those of the old network's depth
+    if (c->net_w && c->cfg.net_precision == LBM_NET_F32) {
+        LBM_CK(c, cudaMemcpyAsync(c->net_w, c->net, sizeof(NetParams), cudaMemcpyHostToDevice, c->stream));
+        LBM_CK(c, cudaStreamSynchronize(c->stream));
+    } else if (c->net_w) {
         const bool split = c->cfg.net_precision == LBM_NET_BF16X3;
         std::vector<unsigned char> packed(split ? nco_tc3_weight_bytes() : nco_tc_weight_bytes());
         if (split) nco_tc3_pack_weights(h.data(), deep, packed.data());
         else nco_tc_pack_weights(h.data(), deep, packed.data());
-        LBM_CK(c, cudaMemcpyAsync(c->tc_w, packed.data(), packed.size(), cudaMemcpyHostToDevice, c->stream));
+        LBM_CK(c, cudaMemcpyAsync(c->net_w, packed.data(), packed.size(), cudaMemcpyHostToDevice, c->stream));
         LBM_CK(c, cudaStreamSynchronize(c->stream));  // `packed` is pageable and goes out of scope
     }
     c->have_weights = true;
@@ -752,7 +753,7 @@ static lbm_status enqueue_step(lbm_ctx* c, int p, cudaStream_t s, const double* 
         ff = FusedForce{c->d_fhat, c->d_ftab, c->d_fproj, c->fscale};
     }
     LBM_CK(c, launch_step(a, forced ? &ff : nullptr, c->cfg.op, c->cfg.storage, c->cfg.boundary,
-                          c->cfg.net_precision, c->net, c->tc_w, c->tc_shape, c->wait_cycles, s));
+                          c->cfg.net_precision, c->net && c->net->deep, c->net_w, c->tc_shape, c->wait_cycles, s));
     return LBM_OK;
 }
 
@@ -979,14 +980,14 @@ static lbm_status backward_sweep(lbm_ctx* c, const char* who, const float* dL_du
             // the recorded force of step t (the forward's projection is not needed again)
             const FusedForce ff{forced ? rec_fhat_at(c, t) : nullptr, c->d_ftab, nullptr, c->fscale};
             LBM_CK(c, launch_step(a, forced ? &ff : nullptr, c->cfg.op, c->cfg.storage, c->cfg.boundary,
-                                  c->cfg.net_precision, c->net, c->tc_w, c->tc_shape, c->wait_cycles, c->stream));
+                                  c->cfg.net_precision, c->net && c->net->deep, c->net_w, c->tc_shape, c->wait_cycles, c->stream));
         }
         for (long long t = b0 - 1; t >= a0; --t) {
             void* state_t = c->adj_work[static_cast<size_t>(t - a0)];
             if (forced) LBM_CK(c, launch_force_synth(c->d, rec_fhat_at(c, t), c->d_ftab, c->d_force, c->stream));
             LBM_CK(c, launch_adjoint_step(c->d, c->cfg.storage, c->cfg.boundary, state_t, c->adj_lam[li],
                                           c->adj_lam[1 - li], c->adj_grad, c->tau, forced ? c->d_force : nullptr,
-                                          *c->net, c->stream));
+                                          deep, static_cast<const NetParams*>(c->net_w), c->stream));
             li = 1 - li;
             const float ks = scale_at(t);
             if (ks != 0.0f)
@@ -1242,7 +1243,7 @@ lbm_status enqueue_batch_step(lbm_batch* b, int phase) {
     LBM_BCK(b, launch_force_batch(b->d_fitems, b->nforced, b->max_proj_blocks, b->max_forced_cells, b->d_counter, 0,
                                   b->stream));
     LBM_BCK(b, launch_step_nco_tc_batch(b->d_inst + phase * n, b->d_tile_begin, b->d_tile_inst, static_cast<int>(n),
-                                        b->ntiles, b->storage, b->shape, b->d_status, b->ctx[0]->tc_w, b->stream));
+                                        b->ntiles, b->storage, b->shape, b->d_status, b->ctx[0]->net_w, b->stream));
     LBM_BCK(b, launch_force_batch(b->d_fitems, b->nforced, b->max_proj_blocks, b->max_forced_cells, b->d_counter, 1,
                                   b->stream));
     if (b->nforced > 0) LBM_BCK(b, launch_counter_increment(b->d_counter, b->stream));
@@ -1382,7 +1383,7 @@ lbm_status lbm_batch_step(lbm_batch* b, int nsteps, int use_graph) {
         // step counter from device memory, so the graphs outlive re-uploads
         destroy_graphs(b);
         LBM_BCK(b, launch_step_nco_tc_batch(b->d_inst, b->d_tile_begin, b->d_tile_inst, static_cast<int>(b->ctx.size()),
-                                            0, b->storage, b->shape, b->d_status, b->ctx[0]->tc_w,
+                                            0, b->storage, b->shape, b->d_status, b->ctx[0]->net_w,
                                             b->stream));  // sets the kernel attributes, no work
         for (int p = 0; p < 2; ++p) {
             cudaGraph_t g = nullptr;
@@ -1445,11 +1446,11 @@ lbm_status lbm_batch_autotune(lbm_batch* b, int* choice) {
         // the state does not advance
         for (int rep = 0; rep < 2; ++rep)
             LBM_BCK(b, launch_step_nco_tc_batch(b->d_inst, b->d_tile_begin, b->d_tile_inst, static_cast<int>(b->ctx.size()),
-                                                b->ntiles, b->storage, shape, b->d_status, b->ctx[0]->tc_w, b->stream));
+                                                b->ntiles, b->storage, shape, b->d_status, b->ctx[0]->net_w, b->stream));
         LBM_BCK(b, cudaEventRecord(e0, b->stream));
         for (int rep = 0; rep < 3; ++rep)
             LBM_BCK(b, launch_step_nco_tc_batch(b->d_inst, b->d_tile_begin, b->d_tile_inst, static_cast<int>(b->ctx.size()),
-                                                b->ntiles, b->storage, shape, b->d_status, b->ctx[0]->tc_w, b->stream));
+                                                b->ntiles, b->storage, shape, b->d_status, b->ctx[0]->net_w, b->stream));
         LBM_BCK(b, cudaEventRecord(e1, b->stream));
         LBM_BCK(b, cudaEventSynchronize(e1));
         float ms = 0.0f;
