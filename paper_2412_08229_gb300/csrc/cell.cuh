@@ -35,6 +35,42 @@ template <> struct Store<LBM_STORE_BF16_DEV> {
 
 __device__ __forceinline__ float wgt(int i) { return static_cast<float>(weight(i)); }
 
+// One axis of a signed permutation with a quarter-period shift: sign * v_perm (+ k).
+struct SymAxis {
+    int perm, sign, k;
+    __device__ __forceinline__ int pick(int v0, int v1, int v2) const {
+        return sign * (perm == 0 ? v0 : perm == 1 ? v1 : v2);
+    }
+};
+
+// Appendix A: a node (sx, sy, sz) outside [0, pi/2]^3 lies in one of the 26 neighbouring
+// blocks; the flow symmetry g = (A, t) of that block brings it back, and a direction c becomes
+// A c, whose index goes to ip. In doubled units of the spacing h (node j at 2j + 1, t = 2N k,
+// period 8N), the image of coordinate s is sign * (2 s_perm + 1) + 2N k; one period is enough
+// to wrap it, since |2 s + 1| <= 2N + 1 and k <= 3. A node inside is left as it is.
+__device__ __forceinline__ void tgv_reduced_image(const Dims& d, int& sx, int& sy, int& sz, int cx, int cy, int cz,
+                                                  int& ip) {
+    const int n = d.nx;
+    const int rx = sx < 0 ? -1 : (sx >= n ? 1 : 0), ry = sy < 0 ? -1 : (sy >= n ? 1 : 0),
+              rz = sz < 0 ? -1 : (sz >= n ? 1 : 0);
+    if (rx | ry | rz) {
+        const int4 q = __ldg(reinterpret_cast<const int4*>(d.sym + 9 * (rz + 1) + 3 * (ry + 1) + (rx + 1)));
+        int j[3], c[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const SymAxis g{(q.x >> (8 * a)) & 3, static_cast<signed char>(q.y >> (8 * a)), (q.z >> (8 * a)) & 3};
+            int v = g.pick(2 * sx + 1, 2 * sy + 1, 2 * sz + 1) + 2 * n * g.k;
+            v = v < 0 ? v + 8 * n : (v >= 8 * n ? v - 8 * n : v);
+            j[a] = (v - 1) >> 1;
+            c[a] = g.pick(cx, cy, cz);
+        }
+        sx = j[0];
+        sy = j[1];
+        sz = j[2];
+        ip = 9 * (c[2] + 1) + 3 * (c[1] + 1) + (c[0] + 1);
+    }
+}
+
 // Pull map of the streaming step (Sec. II.A): population i of cell (x,y,z) at t+1 is
 // population ip of cell `src` at t (post-collision). Periodic: src = x - c_i wrapped.
 // Mirror (Appendix A, octant with nodes half a spacing from the planes): when x - c_i
@@ -51,30 +87,8 @@ __device__ __forceinline__ void pull_source(int x, int y, int z, int i, const Di
         sz = sz < 0 ? sz + d.nz : (sz >= d.nz ? sz - d.nz : sz);
         ip = i;
     } else if (BC == LBM_BC_TGV_REDUCED) {
-        // Appendix A: a source outside [0, pi/2]^3 lies in one of the 26 neighbouring
-        // blocks; the flow symmetry g = (A, t) of that block brings it back. In doubled
-        // units of the spacing h (node j at 2j + 1, t = 2N k, period 8N), the image of
-        // coordinate s is sign * (2 s_perm + 1) + 2N k.
-        const int n = d.nx;
-        const int rx = sx < 0 ? -1 : (sx >= n ? 1 : 0), ry = sy < 0 ? -1 : (sy >= n ? 1 : 0),
-                  rz = sz < 0 ? -1 : (sz >= n ? 1 : 0);
         ip = i;
-        if (rx | ry | rz) {
-            const SymRegion& g = d.sym[9 * (rz + 1) + 3 * (ry + 1) + (rx + 1)];
-            const int s2[3] = {2 * sx + 1, 2 * sy + 1, 2 * sz + 1};
-            int j[3];
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                int v = g.sign[a] * s2[g.perm[a]] + 2 * n * g.k[a];
-                v %= 8 * n;
-                if (v < 0) v += 8 * n;
-                j[a] = (v - 1) >> 1;
-            }
-            sx = j[0];
-            sy = j[1];
-            sz = j[2];
-            ip = g.pmap[i];
-        }
+        tgv_reduced_image(d, sx, sy, sz, cx, cy, cz, ip);
     } else {
         const bool fx = sx < 0 || sx >= d.nx, fy = sy < 0 || sy >= d.ny, fz = sz < 0 || sz >= d.nz;
         sx = fx ? x : sx;

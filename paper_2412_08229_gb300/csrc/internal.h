@@ -39,9 +39,10 @@ static_assert(sizeof(NetParams) % 16 == 0, "copied in 16-byte vectors");
 // One symmetry g = (A, t) of the Taylor-Green flow that maps the block of the periodic
 // box next to the reduced domain [0, pi/2]^3 in direction (rx, ry, rz) onto the domain:
 // (A x)_a = sign[a] x_perm[a], t_a = k[a] pi/2; pmap[i] = index of A c_i.
-struct SymRegion {
-    signed char perm[3], sign[3], k[3], pad;
-    unsigned char pmap[27], pad2;
+// The first twelve bytes are read by one load.
+struct alignas(16) SymRegion {
+    signed char perm[4], sign[4], k[4];
+    unsigned char pmap[28];
 };
 
 // SMs of the current device (grid sizing), looked up once per device

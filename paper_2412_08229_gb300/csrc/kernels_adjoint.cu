@@ -98,25 +98,7 @@ __device__ __forceinline__ void push_target(int y0, int y1, int y2, int j, const
         // g_r(q) with velocity A c_j. This inverts the pull, which takes the source
         // g_r(x - c_i) for a source outside the domain: g_r is the only symmetry mapping
         // block r onto the domain, so g_r^-1 is the one for the block g_r(domain).
-        const int nn = d.nx;
-        const int rx = x[0] < 0 ? -1 : (x[0] >= nn ? 1 : 0), ry = x[1] < 0 ? -1 : (x[1] >= nn ? 1 : 0),
-                  rz = x[2] < 0 ? -1 : (x[2] >= nn ? 1 : 0);
-        if (rx | ry | rz) {
-            const SymRegion& g = d.sym[9 * (rz + 1) + 3 * (ry + 1) + (rx + 1)];
-            const int q2[3] = {2 * x[0] + 1, 2 * x[1] + 1, 2 * x[2] + 1};
-            int xi[3];
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                int v = g.sign[a] * q2[g.perm[a]] + 2 * nn * g.k[a];
-                v %= 8 * nn;
-                if (v < 0) v += 8 * nn;
-                xi[a] = (v - 1) >> 1;
-            }
-            x[0] = xi[0];
-            x[1] = xi[1];
-            x[2] = xi[2];
-            i = g.pmap[j];
-        }
+        tgv_reduced_image(d, x[0], x[1], x[2], c[0], c[1], c[2], i);
     }
     dst = (x[2] * d.ny + x[1]) * d.nx + x[0];
 }
@@ -231,36 +213,85 @@ __global__ void __launch_bounds__(kAdjThreads, (!DEEP && LANES == 2) ? 2 : 1)
     const long long cell0 = static_cast<long long>(blockIdx.x) * kCells;
 
     // ---- moments (warp 0) and cotangents in moment space (warp 1) of the tile's cells
-    if (w < 2 && lane < kCells) {
-        const long long cell = cell0 + lane;
-        float v[Q];
-        if (cell < a.d.ncell) {
-            int x, y, z;
-            cell_coords(cell, a.d, x, y, z);
-            if (w == 0) {
-                float df[Q];
-                load_pulled<STORAGE, BC>(a.state, a.d, x, y, z, df);
-                moments_from_dev(df, v);
-            } else {
+    if constexpr (BC == LBM_BC_TGV_REDUCED) {
+        // the boundary's branches serialise a warp's 27 loads: spread over the block (into the
+        // rows of h1) they run side by side (16^3, third hidden layer: 77 -> 69 us a step;
+        // on the other boundaries the extra barrier costs more, 32^3 225 -> 236 us)
+        load_params(&sh.net, net_in, tid, kAdjThreads);
+        {
+            constexpr int kPer = kAdjThreads / kCells;
+            float* const raw = &sh.h1[0][0][0];
+            const long long cell = cell0 + tid % kCells;
+            const bool valid = cell < a.d.ncell;
+            int x = 0, y = 0, z = 0;
+            if (valid) cell_coords(cell, a.d, x, y, z);
+            using S = Store<STORAGE>;
 #pragma unroll
-                for (int j = 0; j < Q; ++j) {
-                    int i, dst;
-                    push_target<BC>(x, y, z, j, a.d, i, dst);
-                    v[j] = a.lam_in[static_cast<size_t>(i) * a.d.ncell + dst];
+            for (int it = 0; it < (2 * Q + kPer - 1) / kPer; ++it) {
+                const int i = tid / kCells + it * kPer;
+                float v = 0.0f;  // a cell past the end: no cotangent, so it adds nothing
+                if (valid && i < Q) {
+                    int ip, src;
+                    pull_source<BC>(x, y, z, i, a.d, ip, src);
+                    v = S::ld(static_cast<const typename S::T*>(a.state) + static_cast<size_t>(ip) * a.d.ncell + src);
+                } else if (valid && i < 2 * Q) {
+                    int ip, dst;
+                    push_target<BC>(x, y, z, i - Q, a.d, ip, dst);
+                    v = a.lam_in[static_cast<size_t>(ip) * a.d.ncell + dst];
                 }
-                populations_transpose_inplace(v);  // mu* = M^-T lam* (tensor order)
+                if (i < 2 * Q) raw[i * kCells + tid % kCells] = v;
             }
-        } else {  // a cell past the end: no cotangent, so it adds nothing
+            __syncthreads();
+            if (w < 2 && lane < kCells) {
+                float v[Q];
+                const float* src = raw + w * Q * kCells + lane;
 #pragma unroll
-            for (int e = 0; e < Q; ++e) v[e] = 0.0f;
-            if (w == 0) v[0] = 1.0f;
+                for (int e = 0; e < Q; ++e) v[e] = src[e * kCells];
+                if (w == 0) {
+                    float m[Q];
+                    moments_from_dev(v, m);
+#pragma unroll
+                    for (int e = 0; e < Q; ++e) sh.m[lane][e] = m[e];
+                    sh.m[lane][Q] = 1.0f;
+                } else {
+                    populations_transpose_inplace(v);  // mu* = M^-T lam* (tensor order)
+#pragma unroll
+                    for (int e = 0; e < Q; ++e) sh.mu[lane][e] = v[e];
+                }
+            }
         }
-        float* dst = w == 0 ? sh.m[lane] : sh.mu[lane];
+    } else {
+        if (w < 2 && lane < kCells) {
+            const long long cell = cell0 + lane;
+            float v[Q];
+            if (cell < a.d.ncell) {
+                int x, y, z;
+                cell_coords(cell, a.d, x, y, z);
+                if (w == 0) {
+                    float df[Q];
+                    load_pulled<STORAGE, BC>(a.state, a.d, x, y, z, df);
+                    moments_from_dev(df, v);
+                } else {
 #pragma unroll
-        for (int e = 0; e < Q; ++e) dst[e] = v[e];
-        dst[Q] = 1.0f;
+                    for (int j = 0; j < Q; ++j) {
+                        int i, dst;
+                        push_target<BC>(x, y, z, j, a.d, i, dst);
+                        v[j] = a.lam_in[static_cast<size_t>(i) * a.d.ncell + dst];
+                    }
+                    populations_transpose_inplace(v);  // mu* = M^-T lam* (tensor order)
+                }
+            } else {  // a cell past the end: no cotangent, so it adds nothing
+#pragma unroll
+                for (int e = 0; e < Q; ++e) v[e] = 0.0f;
+                if (w == 0) v[0] = 1.0f;
+            }
+            float* dst = w == 0 ? sh.m[lane] : sh.mu[lane];
+#pragma unroll
+            for (int e = 0; e < Q; ++e) dst[e] = v[e];
+            dst[Q] = 1.0f;
+        }
+        if (w >= 2) load_params(&sh.net, net_in, tid - 64, kAdjThreads - 64);
     }
-    if (w >= 2) load_params(&sh.net, net_in, tid - 64, kAdjThreads - 64);
     __syncthreads();
 
     // ---- first layer

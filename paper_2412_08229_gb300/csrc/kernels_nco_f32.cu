@@ -58,6 +58,27 @@ __device__ __forceinline__ void load_tile(const StepArgs& a, long long cell, flo
     m[lane][Q] = drho;
 }
 
+// The block's first tile, which nothing overlaps, on the reduced domain, whose branches
+// serialise a warp's 27 loads: spread over the network warps.
+template <int STORAGE, int BC>
+__device__ __forceinline__ void load_first_tile(const StepArgs& a, long long cell, float (*df)[kTile], int w, int lane) {
+    using S = Store<STORAGE>;
+    int x = 0, y = 0, z = 0;
+    const bool valid = cell < a.d.ncell;
+    if (valid) cell_coords(cell, a.d, x, y, z);
+#pragma unroll
+    for (int it = 0; it < (Q + kNetWarps - 1) / kNetWarps; ++it) {
+        const int i = w + it * kNetWarps;
+        float v = 0.0f;
+        if (valid && i < Q) {
+            int ip, src;
+            pull_source<BC>(x, y, z, i, a.d, ip, src);
+            v = S::ld(static_cast<const typename S::T*>(a.src) + static_cast<size_t>(ip) * a.d.ncell + src);
+        }
+        if (i < Q) df[i][lane] = v;
+    }
+}
+
 template <int STORAGE, int BC, bool FORCED, bool DEEP>
 __global__ void __launch_bounds__(kThreads, 1) step_nco_f32_kernel(const StepArgs a, const NetParams* __restrict__ net_in,
                                                                    const FusedForce ff, int ntiles) {
@@ -75,8 +96,24 @@ __global__ void __launch_bounds__(kThreads, 1) step_nco_f32_kernel(const StepArg
         frc::load_fh2(ff.fhat, sh.fh2);
         if (tid < frc::kProjValues) sh.red[tid] = 0ull;
     }
-    if (w == kLoader) load_tile<STORAGE, BC>(a, cell_of(0), sh.m[0], sh.df[0], lane);
-    if (w < kNetWarps) load_params(&sh.net, net_in, tid, 32 * kNetWarps);
+    if constexpr (BC == LBM_BC_TGV_REDUCED) {
+        if (w < kNetWarps) load_first_tile<STORAGE, BC>(a, cell_of(0), sh.df[0], w, lane);
+        load_params(&sh.net, net_in, tid, kThreads);
+        __syncthreads();
+        if (w == kLoader) {
+            float v[Q], m[Q];
+#pragma unroll
+            for (int e = 0; e < Q; ++e) v[e] = sh.df[0][e][lane];
+            const float drho = moments_from_dev(v, m);
+            if (cell_of(0) < a.d.ncell && !(m[0] >= a.rho_min && m[0] <= a.rho_max)) atomicOr(a.status, 1);
+#pragma unroll
+            for (int e = 0; e < Q; ++e) sh.m[0][lane][e] = m[e];
+            sh.m[0][lane][Q] = drho;
+        }
+    } else {
+        if (w == kLoader) load_tile<STORAGE, BC>(a, cell_of(0), sh.m[0], sh.df[0], lane);
+        if (w < kNetWarps) load_params(&sh.net, net_in, tid, 32 * kNetWarps);
+    }
     __syncthreads();
 
     long long pacc[3] = {0, 0, 0};  // forced steps: fixed-point projection sums of the finisher's lane
