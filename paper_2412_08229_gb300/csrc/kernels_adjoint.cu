@@ -24,9 +24,12 @@
 // nothing of the forward is computed twice. The weight gradients are outer products summed
 // over columns: a lane has 10 x 6 outputs, 60 FMAs for 15 floats read.
 //
+// A block per SM walks over the tiles and keeps the parameter gradients in FP64 in shared
+// memory, so the global atomics come once per block (a block per tile: 32^3 225 us).
+//
 // What bounds it (32^3, ncu): shared-memory latency and bandwidth between bursts of FMAs
-// (wavefronts 55 %, issue 47 %, three warps a scheduler). One step: 32^3 225 us, with the
-// third hidden layer 409 us, 16^3 40 and 67 us; before (one thread per cell, the forward
+// (wavefronts 55 %, issue 47 %, three warps a scheduler). One step: 32^3 213 us, with the
+// third hidden layer 383 us, 16^3 40 and 64 us; before (one thread per cell, the forward
 // computed twice, outer products by 40 of 128 threads): 723, 1137, 232 and 359 us.
 //
 // Observations of the kinetic energy k = (1/2)<|u|^2> at intermediate steps (the loss of
@@ -131,7 +134,8 @@ struct AdjShared {
     static_assert(2 * Q * kCells <= 32 * kRow, "the moment cotangents fit a warp's rows");
 
     NetParams net;
-    float h1[kNetWarps][32][kRow];  // h1, then delta h1, then E, then the partial cotangent of m
+    double grad[GradLayout<DEEP>::kLen];  // the block's parameter gradients, summed over its tiles
+    float h1[kNetWarps][net_rows(kCols)];  // h1, then delta h1, then E, then the partial cotangent of m
     float h2[DEEP ? kNetWarps : 1][32][DEEP ? kRow : 4];  // h2, then delta h2 (third hidden layer)
     float stage[kNetWarps][kStage];
     float m[kCells][28];      // moments (tensor order), 1 (the bias input)
@@ -198,7 +202,7 @@ struct OuterTile {
 
 template <int STORAGE, int BC, bool DEEP, int LANES>
 __global__ void __launch_bounds__(kAdjThreads, (!DEEP && LANES == 2) ? 2 : 1)
-    adjoint_step_kernel(const AdjArgs a, const NetParams* __restrict__ net_in) {
+    adjoint_step_kernel(const AdjArgs a, const NetParams* __restrict__ net_in, int ntiles) {
     using GL = GradLayout<DEEP>;
     using SH = AdjShared<DEEP, LANES>;
     constexpr int kCells = SH::kCells, C = SH::kCols, kRow = SH::kRow;
@@ -210,428 +214,434 @@ __global__ void __launch_bounds__(kAdjThreads, (!DEEP && LANES == 2) ? 2 : 1)
     const int w = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform, and seen to be
     const int p = w >> 1, half = w & 1;
     const int l = lane & 15, og = lane >> 4;  // the rows l and l + 16, units [10 og, 10 og + 10)
-    const long long cell0 = static_cast<long long>(blockIdx.x) * kCells;
+    load_params(&sh.net, net_in, tid, kAdjThreads);
+    for (int i = tid; i < GL::kLen; i += kAdjThreads) sh.grad[i] = 0.0;
 
-    // ---- moments (warp 0) and cotangents in moment space (warp 1) of the tile's cells
-    if constexpr (BC == LBM_BC_TGV_REDUCED) {
-        // the boundary's branches serialise a warp's 27 loads: spread over the block (into the
-        // rows of h1) they run side by side (16^3, third hidden layer: 77 -> 69 us a step;
-        // on the other boundaries the extra barrier costs more, 32^3 225 -> 236 us)
-        load_params(&sh.net, net_in, tid, kAdjThreads);
-        {
-            constexpr int kPer = kAdjThreads / kCells;
-            float* const raw = &sh.h1[0][0][0];
-            const long long cell = cell0 + tid % kCells;
-            const bool valid = cell < a.d.ncell;
-            int x = 0, y = 0, z = 0;
-            if (valid) cell_coords(cell, a.d, x, y, z);
-            using S = Store<STORAGE>;
+#pragma unroll 1
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const long long cell0 = static_cast<long long>(tile) * kCells;
+
+        // ---- moments (warp 0) and cotangents in moment space (warp 1) of the tile's cells
+        if constexpr (BC == LBM_BC_TGV_REDUCED) {
+            // the boundary's branches serialise a warp's 27 loads: spread over the block (into the
+            // rows of h1) they run side by side (16^3, third hidden layer: 77 -> 69 us a step;
+            // on the other boundaries the extra barrier costs more, 32^3 225 -> 236 us)
+            {
+                constexpr int kPer = kAdjThreads / kCells;
+                float* const raw = sh.h1[0];
+                const long long cell = cell0 + tid % kCells;
+                const bool valid = cell < a.d.ncell;
+                int x = 0, y = 0, z = 0;
+                if (valid) cell_coords(cell, a.d, x, y, z);
+                using S = Store<STORAGE>;
 #pragma unroll
-            for (int it = 0; it < (2 * Q + kPer - 1) / kPer; ++it) {
-                const int i = tid / kCells + it * kPer;
-                float v = 0.0f;  // a cell past the end: no cotangent, so it adds nothing
-                if (valid && i < Q) {
-                    int ip, src;
-                    pull_source<BC>(x, y, z, i, a.d, ip, src);
-                    v = S::ld(static_cast<const typename S::T*>(a.state) + static_cast<size_t>(ip) * a.d.ncell + src);
-                } else if (valid && i < 2 * Q) {
-                    int ip, dst;
-                    push_target<BC>(x, y, z, i - Q, a.d, ip, dst);
-                    v = a.lam_in[static_cast<size_t>(ip) * a.d.ncell + dst];
+                for (int it = 0; it < (2 * Q + kPer - 1) / kPer; ++it) {
+                    const int i = tid / kCells + it * kPer;
+                    float v = 0.0f;  // a cell past the end: no cotangent, so it adds nothing
+                    if (valid && i < Q) {
+                        int ip, src;
+                        pull_source<BC>(x, y, z, i, a.d, ip, src);
+                        v = S::ld(static_cast<const typename S::T*>(a.state) + static_cast<size_t>(ip) * a.d.ncell + src);
+                    } else if (valid && i < 2 * Q) {
+                        int ip, dst;
+                        push_target<BC>(x, y, z, i - Q, a.d, ip, dst);
+                        v = a.lam_in[static_cast<size_t>(ip) * a.d.ncell + dst];
+                    }
+                    if (i < 2 * Q) raw[i * kCells + tid % kCells] = v;
                 }
-                if (i < 2 * Q) raw[i * kCells + tid % kCells] = v;
+                __syncthreads();
+                if (w < 2 && lane < kCells) {
+                    float v[Q];
+                    const float* src = raw + w * Q * kCells + lane;
+#pragma unroll
+                    for (int e = 0; e < Q; ++e) v[e] = src[e * kCells];
+                    if (w == 0) {
+                        float m[Q];
+                        moments_from_dev(v, m);
+#pragma unroll
+                        for (int e = 0; e < Q; ++e) sh.m[lane][e] = m[e];
+                        sh.m[lane][Q] = 1.0f;
+                    } else {
+                        populations_transpose_inplace(v);  // mu* = M^-T lam* (tensor order)
+#pragma unroll
+                        for (int e = 0; e < Q; ++e) sh.mu[lane][e] = v[e];
+                    }
+                }
             }
-            __syncthreads();
+        } else {
             if (w < 2 && lane < kCells) {
+                const long long cell = cell0 + lane;
                 float v[Q];
-                const float* src = raw + w * Q * kCells + lane;
+                if (cell < a.d.ncell) {
+                    int x, y, z;
+                    cell_coords(cell, a.d, x, y, z);
+                    if (w == 0) {
+                        float df[Q];
+                        load_pulled<STORAGE, BC>(a.state, a.d, x, y, z, df);
+                        moments_from_dev(df, v);
+                    } else {
 #pragma unroll
-                for (int e = 0; e < Q; ++e) v[e] = src[e * kCells];
-                if (w == 0) {
-                    float m[Q];
-                    moments_from_dev(v, m);
-#pragma unroll
-                    for (int e = 0; e < Q; ++e) sh.m[lane][e] = m[e];
-                    sh.m[lane][Q] = 1.0f;
-                } else {
-                    populations_transpose_inplace(v);  // mu* = M^-T lam* (tensor order)
-#pragma unroll
-                    for (int e = 0; e < Q; ++e) sh.mu[lane][e] = v[e];
-                }
-            }
-        }
-    } else {
-        if (w < 2 && lane < kCells) {
-            const long long cell = cell0 + lane;
-            float v[Q];
-            if (cell < a.d.ncell) {
-                int x, y, z;
-                cell_coords(cell, a.d, x, y, z);
-                if (w == 0) {
-                    float df[Q];
-                    load_pulled<STORAGE, BC>(a.state, a.d, x, y, z, df);
-                    moments_from_dev(df, v);
-                } else {
-#pragma unroll
-                    for (int j = 0; j < Q; ++j) {
-                        int i, dst;
-                        push_target<BC>(x, y, z, j, a.d, i, dst);
-                        v[j] = a.lam_in[static_cast<size_t>(i) * a.d.ncell + dst];
+                        for (int j = 0; j < Q; ++j) {
+                            int i, dst;
+                            push_target<BC>(x, y, z, j, a.d, i, dst);
+                            v[j] = a.lam_in[static_cast<size_t>(i) * a.d.ncell + dst];
+                        }
+                        populations_transpose_inplace(v);  // mu* = M^-T lam* (tensor order)
                     }
-                    populations_transpose_inplace(v);  // mu* = M^-T lam* (tensor order)
+                } else {  // a cell past the end: no cotangent, so it adds nothing
+#pragma unroll
+                    for (int e = 0; e < Q; ++e) v[e] = 0.0f;
+                    if (w == 0) v[0] = 1.0f;
                 }
-            } else {  // a cell past the end: no cotangent, so it adds nothing
+                float* dst = w == 0 ? sh.m[lane] : sh.mu[lane];
 #pragma unroll
-                for (int e = 0; e < Q; ++e) v[e] = 0.0f;
-                if (w == 0) v[0] = 1.0f;
-            }
-            float* dst = w == 0 ? sh.m[lane] : sh.mu[lane];
-#pragma unroll
-            for (int e = 0; e < Q; ++e) dst[e] = v[e];
-            dst[Q] = 1.0f;
-        }
-        if (w >= 2) load_params(&sh.net, net_in, tid - 64, kAdjThreads - 64);
-    }
-    __syncthreads();
-
-    // ---- first layer
-    float* const rows = &sh.h1[w][0][0];
-    float* const row = sh.h1[w][l];
-    {
-        float m[2 / LANES][28];
-#pragma unroll
-        for (int k = 0; k < 2 / LANES; ++k)
-#pragma unroll
-            for (int e = 0; e < 28; e += 4)
-                *reinterpret_cast<float4*>(&m[k][e]) = *reinterpret_cast<const float4*>(&sh.m[l + 16 * k][e]);
-        first_layer<LANES>(net, p, half, lane, m, &sh.h1[2 * p][0][0]);
-    }
-    pair_sync(p);
-
-    // ---- the layers up to the group sum; mask[r][c] keeps which units of the last hidden layer
-    // are on in column c of row l + 16 r (unit j in bit 31 - j)
-    uint32_t mask[2][C];
-    {
-        float acc[2][C][kHalf];
-        set_bias(net.b2, lane, acc);
-        mat_vec<C>(net.W2, lane, acc, RowColumns<C>{row});
-        if constexpr (DEEP) {
-            float* const row2 = sh.h2[w][l];
-            store_relu(row2, lane, acc);
-            __syncwarp();
-            set_bias(net.bd, lane, acc);
-            mat_vec<C>(net.Wd, lane, acc, RowColumns<C>{row2});
-        }
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            float hs[kHalf];
-#pragma unroll
-            for (int o = 0; o < kHalf; ++o) hs[o] = 0.0f;
-#pragma unroll
-            for (int c = 0; c < C; ++c) {
-                uint32_t k = 0u;
-#pragma unroll
-                for (int o = 0; o < kHalf; ++o) {
-                    const float h = fmaxf(acc[r][c][o], 0.0f);
-                    hs[o] += h;
-                    k = __funnelshift_l(__float_as_uint(0.0f - h), k, 1);  // the sign of -h: h > 0
-                }
-                k <<= og ? 32 - kHidden : 32 - kHalf;
-                mask[r][c] = k | __shfl_xor_sync(0xffffffffu, k, 16);
-            }
-#pragma unroll
-            for (int o = 0; o < kHalf; o += 2)
-                *reinterpret_cast<float2*>(&sh.stage[w][(l + 16 * r) * kHidden + og * kHalf + o]) = make_float2(hs[o], hs[o + 1]);
-        }
-    }
-    __syncthreads();
-    for (int i = tid; i < kCells * kHidden; i += kAdjThreads) {  // group sum, i = cell * 20 + unit
-        float v = 0.0f;
-#pragma unroll
-        for (int q = 0; q < kNetWarps; ++q)
-#pragma unroll
-            for (int l = 0; l < LANES; ++l) v += sh.stage[q][i + l * kCells * kHidden];
-        (&sh.hsum[0][0])[i] = v;
-    }
-    __syncthreads();
-    if (tid < kOut * kCells) {  // rates and the cotangents of tau~, one (cell, output) per thread
-        const int n = tid / kCells, c = tid % kCells;
-        float t = 0.0f;
-#pragma unroll
-        for (int j = 0; j < kHidden; ++j) t = fmaf(net.W3[n][j], sh.hsum[c][j], t);
-        t = t * (1.0f / 48.0f) + net.b3[n];
-        const float e = expf(t);
-        const float tau_n = 0.5f / (1.0f + e) + 0.5f;
-        float gw = 0.0f;
-#pragma unroll
-        for (int k = 0; k < Q; ++k)
-            if (order_of(k) >= 3)
-                gw -= order_of(k) == n + 3 ? sh.mu[c][k] * sh.m[c][k] : 0.0f;
-        // d omega / d tau~ = sigma (1 - sigma) / (2 tau_n^2), sigma = 1 / (1 + e^{tau~})
-        const float sg = 1.0f / (1.0f + e);
-        sh.rates[c][n] = 1.0f / tau_n;
-        sh.gbar[c][n] = cell0 + c < a.d.ncell ? gw * sg * (1.0f - sg) / (2.0f * tau_n * tau_n) : 0.0f;
-    }
-    __syncthreads();
-    for (int i = tid; i < kCells * kHidden; i += kAdjThreads) {  // W3^T gbar / 48
-        const int c = i / kHidden, j = i % kHidden;
-        float v = 0.0f;
-#pragma unroll
-        for (int n = 0; n < kOut; ++n) v = fmaf(net.W3[n][j], sh.gbar[c][n], v);
-        sh.v3[c][j] = v * (1.0f / 48.0f);
-    }
-    __syncthreads();
-
-    // ---- the relaxation's part of dL/dm, one warp (the others run ahead)
-    if (w == kNetWarps - 1 && lane < kCells) {
-        const long long cell = cell0 + lane;
-        const bool valid = cell < a.d.ncell;
-        const float* m = sh.m[lane];
-        float* mu_row = sh.mu[lane];
-        const float omega_nu = 1.0f / a.tau;
-        const float irho = 1.0f / m[0];
-        float dm[Q];
-#pragma unroll
-        for (int e = 0; e < Q; ++e) dm[e] = 0.0f;
-#pragma unroll
-        for (int e = 0; e < Q; ++e) {
-            const int n = order_of(e);
-            const float mu = mu_row[e];
-            if (n <= 1) {
-                dm[e] += mu;
-            } else if (n == 2) {
-                dm[e] += (1.0f - omega_nu) * mu;
-                // m^eq_e = m_a m_b / m_0 for the axes a, b of component e
-                const int ex = ex_of(e), ey = ey_of(e), ez = ez_of(e);
-                int ia = -1, ib = -1, axa = 0, axb = 0;
-                const int cnt[3] = {ex, ey, ez};
-                const int idx[3] = {1, 3, 9};
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    if (cnt[k] == 2) { ia = idx[k]; ib = idx[k]; axa = axb = k; }
-                    if (cnt[k] == 1) {
-                        if (ia < 0) { ia = idx[k]; axa = k; }
-                        else { ib = idx[k]; axb = k; }
-                    }
-                }
-                const float ma = m[ia], mb = m[ib];
-                const float c = omega_nu * mu;
-                dm[ia] += c * mb * irho;
-                dm[ib] += c * ma * irho;
-                dm[0] -= c * ma * mb * irho * irho;
-                if (a.force && valid) {
-                    // Kupershtokh source (Sec. II.A) in moment space: its only state-dependent part
-                    // is order 2, dm*_ab = 3 ((j + F)_a (j + F)_b - j_a j_b) / rho with m_a = sqrt3 j_a,
-                    // i.e. (sqrt3 (m_a F_b + F_a m_b) + 3 F_a F_b) / rho; the force is an input
-                    const float Fa = a.force[static_cast<size_t>(axa) * a.d.ncell + cell];
-                    const float Fb = a.force[static_cast<size_t>(axb) * a.d.ncell + cell];
-                    const float src = (kSqrt3 * (ma * Fb + Fa * mb) + 3.0f * Fa * Fb) * irho;
-                    dm[ia] += mu * kSqrt3 * Fb * irho;
-                    dm[ib] += mu * kSqrt3 * Fa * irho;
-                    dm[0] -= mu * src * irho;
-                }
-            } else {
-                dm[e] += (1.0f - sh.rates[lane][n - 3]) * mu;
+                for (int e = 0; e < Q; ++e) dst[e] = v[e];
+                dst[Q] = 1.0f;
             }
         }
-#pragma unroll
-        for (int e = 0; e < Q; ++e) mu_row[e] = dm[e];
-    }
-    __syncwarp();
+        __syncthreads();
 
-    // units j..j+3 of the last hidden layer's cotangent where they are on: v3 of the cell at a
-    // row, and the bits k of a column
-    auto masked = [](const float4& v, uint32_t k) {
-        return make_float4(static_cast<int>(k) < 0 ? v.x : 0.0f, static_cast<int>(k << 1) < 0 ? v.y : 0.0f,
-                           static_cast<int>(k << 2) < 0 ? v.z : 0.0f, static_cast<int>(k << 3) < 0 ? v.w : 0.0f);
-    };
-    auto v3_at = [&](int r, int j) { return *reinterpret_cast<const float4*>(&sh.v3[r % kCells][j]); };
-    auto last_columns = [&](int j, float4(&v)[2][C]) {
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            const float4 t = v3_at(l + 16 * r, j);
-#pragma unroll
-            for (int c = 0; c < C; ++c) v[r][c] = masked(t, mask[r][c] << j);
-        }
-    };
-    // weight gradient of the layer above the columns h: (v3 masked) times h, a column of every
-    // row staged at a time
-    auto last_layer_grad = [&](const float* h, float* out) {
-        OuterTile t;
-        t.clear();
-        float* const st = sh.stage[w];
-#pragma unroll
-        for (int c = 0; c < C; ++c) {
-            const uint32_t k = og ? mask[1][c] : mask[0][c];
-#pragma unroll
-            for (int j = 0; j < kHidden; j += 4)
-                *reinterpret_cast<float4*>(st + lane * kHidden + j) = masked(v3_at(lane, j), k << j);
-            __syncwarp();
-            t.add(st, kHidden, h + c * kHidden, kRow, lane);
-            __syncwarp();
-        }
-        t.flush(out, lane);
-    };
-    // acc where the unit is on in x replaces x
-    auto gate_into = [&](float* x, const float(&acc)[2][C][kHalf]) {
-        x += og * kHalf;
-#pragma unroll
-        for (int r = 0; r < 2; ++r)
-#pragma unroll
-            for (int c = 0; c < C; ++c)
-#pragma unroll
-                for (int o = 0; o < kHalf; o += 2) {
-                    float2* const q = reinterpret_cast<float2*>(x + 16 * r * kRow + c * kHidden + o);
-                    const float2 h = *q;
-                    *q = make_float2(h.x > 0.0f ? acc[r][c][o] : 0.0f, h.y > 0.0f ? acc[r][c][o + 1] : 0.0f);
-                }
-    };
-
-    // ---- backward through the hidden layers
-    if constexpr (DEEP) {
-        float* const rows2 = &sh.h2[w][0][0];
-        float* const row2 = sh.h2[w][l];
-        last_layer_grad(rows2, sh.stage[w]);
+        // ---- first layer
+        float* const rows = sh.h1[w];
+        float* const row = rows + l * kRow;
         {
-            float acc[2][C][kHalf] = {};
-            mat_vec<C>(net.WdT, lane, acc, last_columns);
-            gate_into(row2, acc);  // delta h2
+            float m[2 / LANES][28];
+#pragma unroll
+            for (int k = 0; k < 2 / LANES; ++k)
+#pragma unroll
+                for (int e = 0; e < 28; e += 4)
+                    *reinterpret_cast<float4*>(&m[k][e]) = *reinterpret_cast<const float4*>(&sh.m[l + 16 * k][e]);
+            first_layer<LANES>(net, p, half, lane, m, sh.h1[2 * p]);
+        }
+        pair_sync(p);
+
+        // ---- the layers up to the group sum; mask[r][c] keeps which units of the last hidden layer
+        // are on in column c of row l + 16 r (unit j in bit 31 - j)
+        uint32_t mask[2][C];
+        {
+            float acc[2][C][kHalf];
+            set_bias(net.b2, lane, acc);
+            mat_vec<C>(net.W2, lane, acc, RowColumns<C>{row});
+            if constexpr (DEEP) {
+                float* const row2 = sh.h2[w][l];
+                store_relu(row2, lane, acc);
+                __syncwarp();
+                set_bias(net.bd, lane, acc);
+                mat_vec<C>(net.Wd, lane, acc, RowColumns<C>{row2});
+            }
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                float hs[kHalf];
+#pragma unroll
+                for (int o = 0; o < kHalf; ++o) hs[o] = 0.0f;
+#pragma unroll
+                for (int c = 0; c < C; ++c) {
+                    uint32_t k = 0u;
+#pragma unroll
+                    for (int o = 0; o < kHalf; ++o) {
+                        const float h = fmaxf(acc[r][c][o], 0.0f);
+                        hs[o] += h;
+                        k = __funnelshift_l(__float_as_uint(0.0f - h), k, 1);  // the sign of -h: h > 0
+                    }
+                    k <<= og ? 32 - kHidden : 32 - kHalf;
+                    mask[r][c] = k | __shfl_xor_sync(0xffffffffu, k, 16);
+                }
+#pragma unroll
+                for (int o = 0; o < kHalf; o += 2)
+                    *reinterpret_cast<float2*>(&sh.stage[w][(l + 16 * r) * kHidden + og * kHalf + o]) = make_float2(hs[o], hs[o + 1]);
+            }
+        }
+        __syncthreads();
+        for (int i = tid; i < kCells * kHidden; i += kAdjThreads) {  // group sum, i = cell * 20 + unit
+            float v = 0.0f;
+#pragma unroll
+            for (int q = 0; q < kNetWarps; ++q)
+#pragma unroll
+                for (int l = 0; l < LANES; ++l) v += sh.stage[q][i + l * kCells * kHidden];
+            (&sh.hsum[0][0])[i] = v;
+        }
+        __syncthreads();
+        if (tid < kOut * kCells) {  // rates and the cotangents of tau~, one (cell, output) per thread
+            const int n = tid / kCells, c = tid % kCells;
+            float t = 0.0f;
+#pragma unroll
+            for (int j = 0; j < kHidden; ++j) t = fmaf(net.W3[n][j], sh.hsum[c][j], t);
+            t = t * (1.0f / 48.0f) + net.b3[n];
+            const float e = expf(t);
+            const float tau_n = 0.5f / (1.0f + e) + 0.5f;
+            float gw = 0.0f;
+#pragma unroll
+            for (int k = 0; k < Q; ++k)
+                if (order_of(k) >= 3)
+                    gw -= order_of(k) == n + 3 ? sh.mu[c][k] * sh.m[c][k] : 0.0f;
+            // d omega / d tau~ = sigma (1 - sigma) / (2 tau_n^2), sigma = 1 / (1 + e^{tau~})
+            const float sg = 1.0f / (1.0f + e);
+            sh.rates[c][n] = 1.0f / tau_n;
+            sh.gbar[c][n] = cell0 + c < a.d.ncell ? gw * sg * (1.0f - sg) / (2.0f * tau_n * tau_n) : 0.0f;
+        }
+        __syncthreads();
+        for (int i = tid; i < kCells * kHidden; i += kAdjThreads) {  // W3^T gbar / 48
+            const int c = i / kHidden, j = i % kHidden;
+            float v = 0.0f;
+#pragma unroll
+            for (int n = 0; n < kOut; ++n) v = fmaf(net.W3[n][j], sh.gbar[c][n], v);
+            sh.v3[c][j] = v * (1.0f / 48.0f);
+        }
+        __syncthreads();
+
+        // ---- the relaxation's part of dL/dm, one warp (the others run ahead)
+        if (w == kNetWarps - 1 && lane < kCells) {
+            const long long cell = cell0 + lane;
+            const bool valid = cell < a.d.ncell;
+            const float* m = sh.m[lane];
+            float* mu_row = sh.mu[lane];
+            const float omega_nu = 1.0f / a.tau;
+            const float irho = 1.0f / m[0];
+            float dm[Q];
+#pragma unroll
+            for (int e = 0; e < Q; ++e) dm[e] = 0.0f;
+#pragma unroll
+            for (int e = 0; e < Q; ++e) {
+                const int n = order_of(e);
+                const float mu = mu_row[e];
+                if (n <= 1) {
+                    dm[e] += mu;
+                } else if (n == 2) {
+                    dm[e] += (1.0f - omega_nu) * mu;
+                    // m^eq_e = m_a m_b / m_0 for the axes a, b of component e
+                    const int ex = ex_of(e), ey = ey_of(e), ez = ez_of(e);
+                    int ia = -1, ib = -1, axa = 0, axb = 0;
+                    const int cnt[3] = {ex, ey, ez};
+                    const int idx[3] = {1, 3, 9};
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        if (cnt[k] == 2) { ia = idx[k]; ib = idx[k]; axa = axb = k; }
+                        if (cnt[k] == 1) {
+                            if (ia < 0) { ia = idx[k]; axa = k; }
+                            else { ib = idx[k]; axb = k; }
+                        }
+                    }
+                    const float ma = m[ia], mb = m[ib];
+                    const float c = omega_nu * mu;
+                    dm[ia] += c * mb * irho;
+                    dm[ib] += c * ma * irho;
+                    dm[0] -= c * ma * mb * irho * irho;
+                    if (a.force && valid) {
+                        // Kupershtokh source (Sec. II.A) in moment space: its only state-dependent part
+                        // is order 2, dm*_ab = 3 ((j + F)_a (j + F)_b - j_a j_b) / rho with m_a = sqrt3 j_a,
+                        // i.e. (sqrt3 (m_a F_b + F_a m_b) + 3 F_a F_b) / rho; the force is an input
+                        const float Fa = a.force[static_cast<size_t>(axa) * a.d.ncell + cell];
+                        const float Fb = a.force[static_cast<size_t>(axb) * a.d.ncell + cell];
+                        const float src = (kSqrt3 * (ma * Fb + Fa * mb) + 3.0f * Fa * Fb) * irho;
+                        dm[ia] += mu * kSqrt3 * Fb * irho;
+                        dm[ib] += mu * kSqrt3 * Fa * irho;
+                        dm[0] -= mu * src * irho;
+                    }
+                } else {
+                    dm[e] += (1.0f - sh.rates[lane][n - 3]) * mu;
+                }
+            }
+#pragma unroll
+            for (int e = 0; e < Q; ++e) mu_row[e] = dm[e];
         }
         __syncwarp();
-        {
+
+        // units j..j+3 of the last hidden layer's cotangent where they are on: v3 of the cell at a
+        // row, and the bits k of a column
+        auto masked = [](const float4& v, uint32_t k) {
+            return make_float4(static_cast<int>(k) < 0 ? v.x : 0.0f, static_cast<int>(k << 1) < 0 ? v.y : 0.0f,
+                               static_cast<int>(k << 2) < 0 ? v.z : 0.0f, static_cast<int>(k << 3) < 0 ? v.w : 0.0f);
+        };
+        auto v3_at = [&](int r, int j) { return *reinterpret_cast<const float4*>(&sh.v3[r % kCells][j]); };
+        auto last_columns = [&](int j, float4(&v)[2][C]) {
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const float4 t = v3_at(l + 16 * r, j);
+#pragma unroll
+                for (int c = 0; c < C; ++c) v[r][c] = masked(t, mask[r][c] << j);
+            }
+        };
+        // weight gradient of the layer above the columns h: (v3 masked) times h, a column of every
+        // row staged at a time
+        auto last_layer_grad = [&](const float* h, float* out) {
             OuterTile t;
             t.clear();
-#pragma unroll 1
-            for (int c = 0; c < C; ++c) t.add(rows2 + c * kHidden, kRow, rows + c * kHidden, kRow, lane);
-            t.flush(sh.stage[w] + kGradBlock, lane);
-        }
-        __syncwarp();
-        float acc[2][C][kHalf] = {};
-        mat_vec<C>(net.W2T, lane, acc, RowColumns<C>{row2});
-        gate_into(row, acc);  // delta h1
-    } else {
-        last_layer_grad(rows, sh.stage[w]);
-        float acc[2][C][kHalf] = {};
-        mat_vec<C>(net.W2T, lane, acc, last_columns);
-        gate_into(row, acc);  // delta h1
-    }
-    pair_sync(p);
-
-    // ---- first layer: E of class c in place of delta h1 of sign vector c, and the cotangent of
-    // m through the lane's five units
-    {
-        using At = ColumnOf<LANES>;
-        constexpr int NC = 2 / LANES;
-        float dm[NC][Q];
+            float* const st = sh.stage[w];
 #pragma unroll
-        for (int k = 0; k < NC; ++k)
+            for (int c = 0; c < C; ++c) {
+                const uint32_t k = og ? mask[1][c] : mask[0][c];
 #pragma unroll
-            for (int t = 0; t < Q; ++t) dm[k][t] = 0.0f;
-        const int j0 = half * kHalf + og * 5;
-        float* const q = &sh.h1[2 * p][l][j0];
-#pragma unroll 1
-        for (int i = 0; i < 5; ++i) {
-            float wt[28];
-#pragma unroll
-            for (int t = 0; t < 28; t += 4)
-                *reinterpret_cast<float4*>(wt + t) = *reinterpret_cast<const float4*>(&net.W1p[p][j0 + i][t]);
-#pragma unroll
-            for (int k = 0; k < NC; ++k) {
-                float e[8];
-                auto at = [&](int s) -> float& {
-                    return q[(At::half(s) * 32 + At::row(s) + 16 * k) * kRow + At::col(s) * kHidden + i];
-                };
-#pragma unroll
-                for (int s = 0; s < 8; ++s) e[s] = at(s);
-                wht<8>(e);
-#pragma unroll
-                for (int s = 0; s < 8; ++s) at(s) = e[s];
-#pragma unroll
-                for (int t = 0; t < Q; ++t) dm[k][t] = fmaf(wt[t], e[odd_mask(t)], dm[k][t]);
+                for (int j = 0; j < kHidden; j += 4)
+                    *reinterpret_cast<float4*>(st + lane * kHidden + j) = masked(v3_at(lane, j), k << j);
+                __syncwarp();
+                t.add(st, kHidden, h + c * kHidden, kRow, lane);
+                __syncwarp();
             }
+            t.flush(out, lane);
+        };
+        // acc where the unit is on in x replaces x
+        auto gate_into = [&](float* x, const float(&acc)[2][C][kHalf]) {
+            x += og * kHalf;
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+#pragma unroll
+                for (int c = 0; c < C; ++c)
+#pragma unroll
+                    for (int o = 0; o < kHalf; o += 2) {
+                        float2* const q = reinterpret_cast<float2*>(x + 16 * r * kRow + c * kHidden + o);
+                        const float2 h = *q;
+                        *q = make_float2(h.x > 0.0f ? acc[r][c][o] : 0.0f, h.y > 0.0f ? acc[r][c][o + 1] : 0.0f);
+                    }
+        };
+
+        // ---- backward through the hidden layers
+        if constexpr (DEEP) {
+            float* const rows2 = &sh.h2[w][0][0];
+            float* const row2 = sh.h2[w][l];
+            last_layer_grad(rows2, sh.stage[w]);
+            {
+                float acc[2][C][kHalf] = {};
+                mat_vec<C>(net.WdT, lane, acc, last_columns);
+                gate_into(row2, acc);  // delta h2
+            }
+            __syncwarp();
+            {
+                OuterTile t;
+                t.clear();
+#pragma unroll 1
+                for (int c = 0; c < C; ++c) t.add(rows2 + c * kHidden, kRow, rows + c * kHidden, kRow, lane);
+                t.flush(sh.stage[w] + kGradBlock, lane);
+            }
+            __syncwarp();
+            float acc[2][C][kHalf] = {};
+            mat_vec<C>(net.W2T, lane, acc, RowColumns<C>{row2});
+            gate_into(row, acc);  // delta h1
+        } else {
+            last_layer_grad(rows, sh.stage[w]);
+            float acc[2][C][kHalf] = {};
+            mat_vec<C>(net.W2T, lane, acc, last_columns);
+            gate_into(row, acc);  // delta h1
         }
         pair_sync(p);
-        // dW1p[j][t] = sum over cells of E[c(t)][j] m_t, lane t (lane 27: db1, the bias input of class 0)
+
+        // ---- first layer: E of class c in place of delta h1 of sign vector c, and the cotangent of
+        // m through the lane's five units
         {
-            const int t = lane < Q ? lane : Q;
-            const int ex = t % 3, ey = (t / 3) % 3, ez = t / 9;
-            const int c = t < Q ? ((ex == 1) << 2) | ((ey == 1) << 1) | (ez == 1) : 0;
-            const float* er = &sh.h1[2 * p + At::half(c)][At::row(c)][At::col(c) * kHidden + half * kHalf];
-            float g[kHalf];
+            using At = ColumnOf<LANES>;
+            constexpr int NC = 2 / LANES;
+            float dm[NC][Q];
 #pragma unroll
-            for (int j = 0; j < kHalf; ++j) g[j] = 0.0f;
-#pragma unroll 2
-            for (int r = 0; r < kCells; ++r) {
-                const float mt = sh.m[r][t];
+            for (int k = 0; k < NC; ++k)
 #pragma unroll
-                for (int j = 0; j < kHalf; j += 2) {
-                    const float2 v = *reinterpret_cast<const float2*>(er + r * kRow + j);
-                    g[j] = fmaf(v.x, mt, g[j]);
-                    g[j + 1] = fmaf(v.y, mt, g[j + 1]);
+                for (int t = 0; t < Q; ++t) dm[k][t] = 0.0f;
+            const int j0 = half * kHalf + og * 5;
+            float* const q = sh.h1[2 * p] + l * kRow + j0;
+#pragma unroll 1
+            for (int i = 0; i < 5; ++i) {
+                float wt[28];
+#pragma unroll
+                for (int t = 0; t < 28; t += 4)
+                    *reinterpret_cast<float4*>(wt + t) = *reinterpret_cast<const float4*>(&net.W1p[p][j0 + i][t]);
+#pragma unroll
+                for (int k = 0; k < NC; ++k) {
+                    float e[8];
+                    auto at = [&](int s) -> float& {
+                        return q[At::half(s) * net_rows(C) + (At::row(s) + 16 * k) * kRow + At::col(s) * kHidden + i];
+                    };
+#pragma unroll
+                    for (int s = 0; s < 8; ++s) e[s] = at(s);
+                    wht<8>(e);
+#pragma unroll
+                    for (int s = 0; s < 8; ++s) at(s) = e[s];
+#pragma unroll
+                    for (int t = 0; t < Q; ++t) dm[k][t] = fmaf(wt[t], e[odd_mask(t)], dm[k][t]);
                 }
             }
-            if (lane <= Q) {
+            pair_sync(p);
+            // dW1p[j][t] = sum over cells of E[c(t)][j] m_t, lane t (lane 27: db1, the bias input of class 0)
+            {
+                const int t = lane < Q ? lane : Q;
+                const int ex = t % 3, ey = (t / 3) % 3, ez = t / 9;
+                const int c = t < Q ? ((ex == 1) << 2) | ((ey == 1) << 1) | (ez == 1) : 0;
+                const float* er = sh.h1[2 * p + At::half(c)] + At::row(c) * kRow + At::col(c) * kHidden + half * kHalf;
+                float g[kHalf];
 #pragma unroll
-                for (int j = 0; j < kHalf; ++j) sh.stage[w][SH::kD1 + t * kHalf + j] = g[j];
+                for (int j = 0; j < kHalf; ++j) g[j] = 0.0f;
+#pragma unroll 2
+                for (int r = 0; r < kCells; ++r) {
+                    const float mt = sh.m[r][t];
+#pragma unroll
+                    for (int j = 0; j < kHalf; j += 2) {
+                        const float2 v = *reinterpret_cast<const float2*>(er + r * kRow + j);
+                        g[j] = fmaf(v.x, mt, g[j]);
+                        g[j + 1] = fmaf(v.y, mt, g[j + 1]);
+                    }
+                }
+                if (lane <= Q) {
+#pragma unroll
+                    for (int j = 0; j < kHalf; ++j) sh.stage[w][SH::kD1 + t * kHalf + j] = g[j];
+                }
             }
+            pair_sync(p);
+            // the rows are free: the two five-unit parts of the cells' cotangents, [t][og][cell]
+#pragma unroll
+            for (int t = 0; t < Q; ++t)
+#pragma unroll
+                for (int k = 0; k < NC; ++k) rows[(2 * t + og) * kCells + l + 16 * k] = dm[k][t];
         }
-        pair_sync(p);
-        // the rows are free: the two five-unit parts of the cells' cotangents, [t][og][cell]
+        __syncthreads();
+        for (int i = tid; i < Q * kCells; i += kAdjThreads) {  // the twelve warps' parts and the relaxation's
+            const int t = i / kCells, c = i % kCells;
+            float v = sh.mu[c][t];
 #pragma unroll
-        for (int t = 0; t < Q; ++t)
+            for (int q = 0; q < kNetWarps; ++q)
 #pragma unroll
-            for (int k = 0; k < NC; ++k) rows[(2 * t + og) * kCells + l + 16 * k] = dm[k][t];
-    }
-    __syncthreads();
-    for (int i = tid; i < Q * kCells; i += kAdjThreads) {  // the twelve warps' parts and the relaxation's
-        const int t = i / kCells, c = i % kCells;
-        float v = sh.mu[c][t];
-#pragma unroll
-        for (int q = 0; q < kNetWarps; ++q)
-#pragma unroll
-            for (int g = 0; g < 2; ++g) v += (&sh.h1[q][0][0])[(2 * t + g) * kCells + c];
-        sh.dm[t][c] = v;
-    }
-    __syncthreads();
+                for (int g = 0; g < 2; ++g) v += sh.h1[q][(2 * t + g) * kCells + c];
+            sh.dm[t][c] = v;
+        }
+        __syncthreads();
 
-    if (w == 0) {  // lam_t = M^T dL/dm
-        const long long cell = cell0 + lane;
-        if (lane < kCells && cell < a.d.ncell) {
-            float v[Q];
+        if (w == 0) {  // lam_t = M^T dL/dm
+            const long long cell = cell0 + lane;
+            if (lane < kCells && cell < a.d.ncell) {
+                float v[Q];
 #pragma unroll
-            for (int e = 0; e < Q; ++e) v[e] = sh.dm[e][lane];
-            moments_transpose_inplace(v);
+                for (int e = 0; e < Q; ++e) v[e] = sh.dm[e][lane];
+                moments_transpose_inplace(v);
 #pragma unroll
-            for (int i = 0; i < Q; ++i) a.lam_out[static_cast<size_t>(i) * a.d.ncell + cell] = v[i];
-        }
-        return;
-    }
-    // parameter gradients of the tile, one per thread: sums over the warps (W1: the six
-    // permutations' columns that a printed column went to), added in FP64
-    for (int i = tid - 32; i < GL::kLen; i += kAdjThreads - 32) {
-        float v = 0.0f;
-        if (i < GL::kW2) {
-            const int j = i < GL::kB1 ? i / Q : i - GL::kB1, k = i < GL::kB1 ? i % Q : Q;
-            const int h = j >= kHalf, jo = j - h * kHalf;
-#pragma unroll
-            for (int q = 0; q < 6; ++q) {
-                const int t = k < Q ? kPermColumns.t[q][k] : Q;
-                v += sh.stage[2 * q + h][SH::kD1 + t * kHalf + jo];
+                for (int i = 0; i < Q; ++i) a.lam_out[static_cast<size_t>(i) * a.d.ncell + cell] = v[i];
             }
-        } else if (i < GL::kW3) {
-            // stage: with the third hidden layer (Wd | bd) then (W2 | b2), else (W2 | b2)
-            int o = i - GL::kW2;
-            if (DEEP) o = o < kGradBlock ? o + kGradBlock : o - kGradBlock;
-#pragma unroll
-            for (int q = 0; q < kNetWarps; ++q) v += sh.stage[q][o];
-        } else {
-            const int o = i - GL::kW3;
-            const int n = o < kOut * kHidden ? o / kHidden : o - kOut * kHidden;
-            for (int c = 0; c < kCells; ++c)
-                v = fmaf(sh.gbar[c][n], o < kOut * kHidden ? sh.hsum[c][o % kHidden] * (1.0f / 48.0f) : 1.0f, v);
+            continue;  // the next tile's first barrier keeps the other warps' sums from it
         }
-        atomicAdd(&a.grad[i], static_cast<double>(v));
+        // parameter gradients of the tile, a thread's own: sums over the warps (W1: the six
+        // permutations' columns that a printed column went to), added in FP64
+        for (int i = tid - 32; i < GL::kLen; i += kAdjThreads - 32) {
+            float v = 0.0f;
+            if (i < GL::kW2) {
+                const int j = i < GL::kB1 ? i / Q : i - GL::kB1, k = i < GL::kB1 ? i % Q : Q;
+                const int h = j >= kHalf, jo = j - h * kHalf;
+#pragma unroll
+                for (int q = 0; q < 6; ++q) {
+                    const int t = k < Q ? kPermColumns.t[q][k] : Q;
+                    v += sh.stage[2 * q + h][SH::kD1 + t * kHalf + jo];
+                }
+            } else if (i < GL::kW3) {
+                // stage: with the third hidden layer (Wd | bd) then (W2 | b2), else (W2 | b2)
+                int o = i - GL::kW2;
+                if (DEEP) o = o < kGradBlock ? o + kGradBlock : o - kGradBlock;
+#pragma unroll
+                for (int q = 0; q < kNetWarps; ++q) v += sh.stage[q][o];
+            } else {
+                const int o = i - GL::kW3;
+                const int n = o < kOut * kHidden ? o / kHidden : o - kOut * kHidden;
+                for (int c = 0; c < kCells; ++c)
+                    v = fmaf(sh.gbar[c][n], o < kOut * kHidden ? sh.hsum[c][o % kHidden] * (1.0f / 48.0f) : 1.0f, v);
+            }
+            sh.grad[i] += static_cast<double>(v);
+        }
     }
+    if (w != 0)
+        for (int i = tid - 32; i < GL::kLen; i += kAdjThreads - 32) atomicAdd(&a.grad[i], sh.grad[i]);
 }
 
 // lam[i] (=, or += when accumulate) sum_a g_a (c_ia - u_a) / rho + dL/drho for the state
@@ -688,8 +698,9 @@ static cudaError_t launch_adjoint_step_t(const AdjArgs& a, const NetParams* net,
     const cudaError_t e = ensure_dynamic_smem(adjoint_step_kernel<LBM_STORE_F32, BC, DEEP, LANES>,
                                               static_cast<int>(smem), attr);
     if (e != cudaSuccess) return e;
-    const unsigned grid = static_cast<unsigned>((a.d.ncell + SH::kCells - 1) / SH::kCells);
-    adjoint_step_kernel<LBM_STORE_F32, BC, DEEP, LANES><<<grid, kAdjThreads, smem, s>>>(a, net);
+    const int ntiles = static_cast<int>((a.d.ncell + SH::kCells - 1) / SH::kCells);
+    const int sms = sm_count();
+    adjoint_step_kernel<LBM_STORE_F32, BC, DEEP, LANES><<<ntiles < sms ? ntiles : sms, kAdjThreads, smem, s>>>(a, net, ntiles);
     return cudaGetLastError();
 }
 

@@ -26,7 +26,7 @@ constexpr int kThreads = 32 * (kNetWarps + 2);
 
 struct NetShared {
     NetParams net;
-    float rows[kNetWarps][kTile][net_row(4)];          // the columns' h1 (then h2)
+    float rows[kNetWarps][net_rows(4)];          // the columns' h1 (then h2)
     float part[2][kNetWarps / 2][kTile][kHidden];      // sums of the last hidden layer over a permutation's sign vectors
     float m[3][kTile][28];                             // moments (tensor order), rho - 1
     float df[3][Q][kTile];                             // the pulled deviations
@@ -130,10 +130,10 @@ __global__ void __launch_bounds__(kThreads, 1) step_nco_f32_kernel(const StepArg
 #pragma unroll
                         for (int e = 0; e < 28; e += 4)
                             *reinterpret_cast<float4*>(&m[k][e]) = *reinterpret_cast<const float4*>(&sh.m[b][l + 16 * k][e]);
-                    first_layer<1>(net, p, half, lane, m, &sh.rows[2 * p][0][0]);
+                    first_layer<1>(net, p, half, lane, m, sh.rows[2 * p]);
                 }
                 pair_sync(p);
-                float* const row = sh.rows[w][l];
+                float* const row = sh.rows[w] + l * net_row(4);
                 float acc[2][4][kHalf];
                 set_bias(net.b2, lane, acc);
                 mat_vec<4>(net.W2, lane, acc, RowColumns<4>{row});

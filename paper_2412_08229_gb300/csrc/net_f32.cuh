@@ -39,6 +39,10 @@ __host__ __device__ constexpr int odd_mask(int t) {
     return ((ex_of(t) == 1) << 2) | ((ey_of(t) == 1) << 1) | (ez_of(t) == 1);
 }
 
+// Floats of a warp's 32 rows: the sixteen at the end shift the second warp of a permutation by
+// half the banks, so that the eight classes of a cell are read without conflicts.
+constexpr int net_rows(int C) { return 32 * net_row(C) + 16; }
+
 // y[s] <- sum_c (-1)^popcount(s & c) y[c] over N = 4 or 8 values, in place (its own inverse
 // up to a factor N)
 template <int N>
@@ -74,7 +78,7 @@ __device__ __forceinline__ void load_params(NetParams* dst, const NetParams* __r
 }
 
 // relu(W1p x^(s) + b1) for the eight sign vectors s of permutation p, into the rows of its two
-// warps (rows: the first warp's; those of the second follow 32 rows later). Of the warp's ten
+// warps (rows: the first warp's; those of the second follow net_rows floats later). Of the warp's ten
 // units a lane takes five, for the cells l = lane % 16 (and l + 16, LANES = 1); m[k] are the
 // moments of its cells in tensor order.
 template <int LANES>
@@ -99,7 +103,7 @@ __device__ __forceinline__ void first_layer(const NetParams& net, int p, int hal
             using At = ColumnOf<LANES>;
 #pragma unroll
             for (int s = 0; s < 8; ++s)
-                out[(At::half(s) * 32 + At::row(s) + 16 * k) * R + At::col(s) * kHidden + i] = fmaxf(y[s] + w[Q], 0.0f);
+                out[At::half(s) * net_rows(C) + (At::row(s) + 16 * k) * R + At::col(s) * kHidden + i] = fmaxf(y[s] + w[Q], 0.0f);
         }
     }
 }
