@@ -111,9 +111,10 @@ struct FusedForce;  // the in-kernel forcing of a forced step (declared with the
 // wait_cycles: limit of the main MMA-completion waits of the pair-pipelined and split
 // tensor-core kernels (kept out of StepArgs: a larger argument block made the CUDA-core
 // network kernel spill).
+// overlap: the BGK, KBC and REG kernels start while the launch before them ends (launch.cuh).
 // ff: the in-kernel forcing of a forced step (nullptr: unforced; a.force is then not read).
 cudaError_t launch_step(const StepArgs& a, const FusedForce* ff, int op, int storage, int bc, int net_prec,
-                        bool deep, const void* net_weights, int tc_shape, long long wait_cycles,
+                        bool deep, const void* net_weights, int tc_shape, long long wait_cycles, bool overlap,
                         cudaStream_t s);
 cudaError_t launch_init_eq(const Dims& d, int storage, int bc, const float* rho, const float* u,
                            void* dst, cudaStream_t s);
@@ -200,7 +201,7 @@ cudaError_t launch_force_coeffs(unsigned long long* proj, double unit, const dou
 // The same with row = min(head + *counter, rows - 1), then *counter += 1 (graph replays).
 cudaError_t launch_force_coeffs_indexed(unsigned long long* proj, double unit, const double* draws,
                                         long long* counter, long long head, long long rows, const double* consts,
-                                        double* fhat, cudaStream_t s);
+                                        double* fhat, bool overlap, cudaStream_t s);
 cudaError_t launch_force_synth(const Dims& d, const double* fhat, const float2* tab, float* force, cudaStream_t s);
 // The in-kernel forcing of a single context's forced step: F(x) from fhat and the phase
 // tables, the step's velocity projected into proj (nullptr: not projected, as in the

@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "force.cuh"
+#include "launch.cuh"
 
 namespace lbm {
 
@@ -218,6 +219,7 @@ __global__ void __launch_bounds__(kCoeffThreads) force_coeffs_kernel(unsigned lo
 __global__ void __launch_bounds__(kCoeffThreads) force_coeffs_indexed_kernel(
     unsigned long long* proj, double unit, const double* draws, long long* counter, long long head, long long rows,
     const double* consts, double* fhat) {
+    overlap_wait();
     long long row = head + *counter;
     if (row > rows - 1) row = rows - 1;
     coeffs_block(proj, unit, draws + row * kDrawRow, consts, fhat);
@@ -247,9 +249,9 @@ cudaError_t launch_force_coeffs(unsigned long long* proj, double unit, const dou
 
 cudaError_t launch_force_coeffs_indexed(unsigned long long* proj, double unit, const double* draws,
                                         long long* counter, long long head, long long rows, const double* consts,
-                                        double* fhat, cudaStream_t s) {
-    force_coeffs_indexed_kernel<<<1, kCoeffThreads, 0, s>>>(proj, unit, draws, counter, head, rows, consts, fhat);
-    return cudaGetLastError();
+                                        double* fhat, bool overlap, cudaStream_t s) {
+    return launch_kernel(force_coeffs_indexed_kernel, 1, kCoeffThreads, 0, s, overlap, proj, unit, draws, counter, head,
+                         rows, consts, fhat);
 }
 
 cudaError_t launch_counter_increment(long long* counter, cudaStream_t s) {

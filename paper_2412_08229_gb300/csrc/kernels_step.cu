@@ -11,6 +11,7 @@
 
 #include "force.cuh"
 #include "internal.h"
+#include "launch.cuh"
 
 namespace lbm {
 
@@ -102,6 +103,7 @@ __device__ __forceinline__ void step_body_forced(const StepArgs& a, const FusedF
 template <int OP, int STORAGE, int BC, bool FORCED>
 __global__ void __launch_bounds__(kStepThreads, OP == LBM_OP_KBC && !FORCED ? 7 : 1)
     step_kernel(const StepArgs a, const FusedForce ff) {
+    overlap_wait();
     if constexpr (FORCED) step_body_forced<OP, STORAGE, BC>(a, ff);
     else step_body<OP, STORAGE, BC>(a);
 }
@@ -124,38 +126,37 @@ static unsigned forced_grid(K kernel, int threads, std::atomic<int>& occ, long l
 }
 
 template <int OP, int STORAGE, int BC, bool FORCED>
-static cudaError_t launch_op(const StepArgs& a, const FusedForce& ff, cudaStream_t s) {
+static cudaError_t launch_op(const StepArgs& a, const FusedForce& ff, bool overlap, cudaStream_t s) {
     unsigned grid = static_cast<unsigned>((a.d.ncell + kStepThreads - 1) / kStepThreads);
     if constexpr (FORCED) {
         static std::atomic<int> occ{0};
         grid = forced_grid(step_kernel<OP, STORAGE, BC, true>, kStepThreads, occ, a.d.ncell);
     }
-    step_kernel<OP, STORAGE, BC, FORCED><<<grid, kStepThreads, 0, s>>>(a, ff);
-    return cudaGetLastError();
+    return launch_kernel(step_kernel<OP, STORAGE, BC, FORCED>, grid, kStepThreads, 0, s, overlap, a, ff);
 }
 
 template <int STORAGE, int BC, bool FORCED>
-static cudaError_t launch_step_t(const StepArgs& a, const FusedForce& ff, int op, cudaStream_t s) {
-    if (op == LBM_OP_BGK) return launch_op<LBM_OP_BGK, STORAGE, BC, FORCED>(a, ff, s);
-    if (op == LBM_OP_KBC) return launch_op<LBM_OP_KBC, STORAGE, BC, FORCED>(a, ff, s);
-    return launch_op<LBM_OP_REG, STORAGE, BC, FORCED>(a, ff, s);
+static cudaError_t launch_step_t(const StepArgs& a, const FusedForce& ff, int op, bool overlap, cudaStream_t s) {
+    if (op == LBM_OP_BGK) return launch_op<LBM_OP_BGK, STORAGE, BC, FORCED>(a, ff, overlap, s);
+    if (op == LBM_OP_KBC) return launch_op<LBM_OP_KBC, STORAGE, BC, FORCED>(a, ff, overlap, s);
+    return launch_op<LBM_OP_REG, STORAGE, BC, FORCED>(a, ff, overlap, s);
 }
 
 // Forcing runs on periodic boxes only (contexts refuse it on the other boundaries).
 template <int STORAGE>
-static cudaError_t launch_step_s(const StepArgs& a, const FusedForce* ff, int op, int bc, cudaStream_t s) {
+static cudaError_t launch_step_s(const StepArgs& a, const FusedForce* ff, int op, int bc, bool overlap, cudaStream_t s) {
     const FusedForce none{};
     if (ff) {
         if (bc != LBM_BC_PERIODIC) return cudaErrorInvalidValue;
-        return launch_step_t<STORAGE, LBM_BC_PERIODIC, true>(a, *ff, op, s);
+        return launch_step_t<STORAGE, LBM_BC_PERIODIC, true>(a, *ff, op, overlap, s);
     }
-    if (bc == LBM_BC_PERIODIC) return launch_step_t<STORAGE, LBM_BC_PERIODIC, false>(a, none, op, s);
-    if (bc == LBM_BC_TGV_REDUCED) return launch_step_t<STORAGE, LBM_BC_TGV_REDUCED, false>(a, none, op, s);
-    return launch_step_t<STORAGE, LBM_BC_MIRROR, false>(a, none, op, s);
+    if (bc == LBM_BC_PERIODIC) return launch_step_t<STORAGE, LBM_BC_PERIODIC, false>(a, none, op, overlap, s);
+    if (bc == LBM_BC_TGV_REDUCED) return launch_step_t<STORAGE, LBM_BC_TGV_REDUCED, false>(a, none, op, overlap, s);
+    return launch_step_t<STORAGE, LBM_BC_MIRROR, false>(a, none, op, overlap, s);
 }
 
 cudaError_t launch_step(const StepArgs& a, const FusedForce* ff, int op, int storage, int bc, int net_prec, bool deep,
-                        const void* net_weights, int tc_shape, long long wait_cycles, cudaStream_t s) {
+                        const void* net_weights, int tc_shape, long long wait_cycles, bool overlap, cudaStream_t s) {
     if (op == LBM_OP_NCO && net_prec == LBM_NET_BF16)
         return launch_step_nco_tc(a, ff, storage, bc, deep, tc_shape, wait_cycles, net_weights, s);
     if (op == LBM_OP_NCO && net_prec == LBM_NET_BF16X3)
@@ -163,9 +164,9 @@ cudaError_t launch_step(const StepArgs& a, const FusedForce* ff, int op, int sto
     if (op == LBM_OP_NCO)
         return launch_step_nco_f32(a, ff, storage, bc, deep, static_cast<const NetParams*>(net_weights), s);
     switch (storage) {
-        case LBM_STORE_F32: return launch_step_s<LBM_STORE_F32>(a, ff, op, bc, s);
-        case LBM_STORE_F16_DEV: return launch_step_s<LBM_STORE_F16_DEV>(a, ff, op, bc, s);
-        default: return launch_step_s<LBM_STORE_BF16_DEV>(a, ff, op, bc, s);
+        case LBM_STORE_F32: return launch_step_s<LBM_STORE_F32>(a, ff, op, bc, overlap, s);
+        case LBM_STORE_F16_DEV: return launch_step_s<LBM_STORE_F16_DEV>(a, ff, op, bc, overlap, s);
+        default: return launch_step_s<LBM_STORE_BF16_DEV>(a, ff, op, bc, overlap, s);
     }
 }
 
