@@ -111,7 +111,7 @@ struct FusedForce;  // the in-kernel forcing of a forced step (declared with the
 // wait_cycles: limit of the main MMA-completion waits of the pair-pipelined and split
 // tensor-core kernels (kept out of StepArgs: a larger argument block made the CUDA-core
 // network kernel spill).
-// overlap: the BGK, KBC and REG kernels start while the launch before them ends (launch.cuh).
+// overlap: the BGK, KBC, REG and FP32-network kernels start while the launch before them ends (launch.cuh).
 // ff: the in-kernel forcing of a forced step (nullptr: unforced; a.force is then not read).
 cudaError_t launch_step(const StepArgs& a, const FusedForce* ff, int op, int storage, int bc, int net_prec,
                         bool deep, const void* net_weights, int tc_shape, long long wait_cycles, bool overlap,
@@ -130,7 +130,7 @@ int kinetic_energy_blocks(const Dims& d);
 
 // FP32 network on the CUDA cores (kernels_nco_f32.cu)
 cudaError_t launch_step_nco_f32(const StepArgs& a, const FusedForce* ff, int storage, int bc, bool deep,
-                                const NetParams* d_net, cudaStream_t s);
+                                const NetParams* d_net, bool overlap, cudaStream_t s);
 
 // Tensor-core network (kernels_nco_tc.cu)
 size_t nco_tc_weight_bytes();

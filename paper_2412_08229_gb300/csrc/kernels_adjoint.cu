@@ -28,14 +28,15 @@
 // memory, so the global atomics come once per block (a block per tile: 32^3 225 us).
 //
 // What bounds it (32^3, ncu): shared-memory latency and bandwidth between bursts of FMAs
-// (wavefronts 55 %, issue 47 %, three warps a scheduler). One step: 32^3 213 us, with the
-// third hidden layer 383 us, 16^3 40 and 64 us; before (one thread per cell, the forward
+// (wavefronts 55 %, issue 47 %, three warps a scheduler). One step: 32^3 206 us, with the
+// third hidden layer 367 us, 16^3 36 and 59 us; before (one thread per cell, the forward
 // computed twice, outer products by 40 of 128 threads): 723, 1137, 232 and 359 us.
 //
 // Observations of the kinetic energy k = (1/2)<|u|^2> at intermediate steps (the loss of
 // Sec. IV is a function of k(t)) enter as extra seeds added to lam_t when the reverse
 // sweep passes step t: dk/df_i = (1/cells) sum_a u_a (c_ia - u_a) / rho.
 #include "cell.cuh"
+#include "launch.cuh"
 #include "net_f32.cuh"
 
 namespace lbm {
@@ -216,6 +217,7 @@ __global__ void __launch_bounds__(kAdjThreads, (!DEEP && LANES == 2) ? 2 : 1)
     const int l = lane & 15, og = lane >> 4;  // the rows l and l + 16, units [10 og, 10 og + 10)
     load_params(&sh.net, net_in, tid, kAdjThreads);
     for (int i = tid; i < GL::kLen; i += kAdjThreads) sh.grad[i] = 0.0;
+    overlap_wait();
 
 #pragma unroll 1
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
@@ -321,13 +323,13 @@ __global__ void __launch_bounds__(kAdjThreads, (!DEEP && LANES == 2) ? 2 : 1)
         {
             float acc[2][C][kHalf];
             set_bias(net.b2, lane, acc);
-            mat_vec<C>(net.W2, lane, acc, RowColumns<C>{row});
+            mat_vec<C, 5>(net.W2, lane, acc, RowColumns<C>{row});
             if constexpr (DEEP) {
                 float* const row2 = sh.h2[w][l];
                 store_relu(row2, lane, acc);
                 __syncwarp();
                 set_bias(net.bd, lane, acc);
-                mat_vec<C>(net.Wd, lane, acc, RowColumns<C>{row2});
+                mat_vec<C, 5>(net.Wd, lane, acc, RowColumns<C>{row2});
             }
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
@@ -501,7 +503,7 @@ __global__ void __launch_bounds__(kAdjThreads, (!DEEP && LANES == 2) ? 2 : 1)
             last_layer_grad(rows2, sh.stage[w]);
             {
                 float acc[2][C][kHalf] = {};
-                mat_vec<C>(net.WdT, lane, acc, last_columns);
+                mat_vec<C, 5>(net.WdT, lane, acc, last_columns);
                 gate_into(row2, acc);  // delta h2
             }
             __syncwarp();
@@ -514,12 +516,12 @@ __global__ void __launch_bounds__(kAdjThreads, (!DEEP && LANES == 2) ? 2 : 1)
             }
             __syncwarp();
             float acc[2][C][kHalf] = {};
-            mat_vec<C>(net.W2T, lane, acc, RowColumns<C>{row2});
+            mat_vec<C, 5>(net.W2T, lane, acc, RowColumns<C>{row2});
             gate_into(row, acc);  // delta h1
         } else {
             last_layer_grad(rows, sh.stage[w]);
             float acc[2][C][kHalf] = {};
-            mat_vec<C>(net.W2T, lane, acc, last_columns);
+            mat_vec<C, 5>(net.W2T, lane, acc, last_columns);
             gate_into(row, acc);  // delta h1
         }
         pair_sync(p);
@@ -700,8 +702,8 @@ static cudaError_t launch_adjoint_step_t(const AdjArgs& a, const NetParams* net,
     if (e != cudaSuccess) return e;
     const int ntiles = static_cast<int>((a.d.ncell + SH::kCells - 1) / SH::kCells);
     const int sms = sm_count();
-    adjoint_step_kernel<LBM_STORE_F32, BC, DEEP, LANES><<<ntiles < sms ? ntiles : sms, kAdjThreads, smem, s>>>(a, net, ntiles);
-    return cudaGetLastError();
+    return launch_kernel(adjoint_step_kernel<LBM_STORE_F32, BC, DEEP, LANES>, static_cast<unsigned>(ntiles < sms ? ntiles : sms),
+                         kAdjThreads, smem, s, true, a, net, ntiles);
 }
 
 template <int BC>

@@ -9,11 +9,14 @@
 //
 // What bounds it (32^3, ncu): issue, 58 % of the cycles, in bursts: the twelve warps go through
 // their FMA and shared-memory phases nearly together; shared-memory wavefronts 48 %. Step of
-// the two-layer network with FP32 storage: 256^3 22.6 ms, 48^3 158 us, 32^3 53 us, 16^3
-// 12.5 us; with one thread per cell and the weights in the constant bank 26.1 ms, 183, 55 and
-// 46.9 us (16^3 fills 32 of 152 SMs that way, here 128). Third hidden layer: 16^3 17 us (70).
+// the two-layer network with FP32 storage: 256^3 22.3 ms, 48^3 153 us, 32^3 49 us, 16^3
+// 10.4 us; with one thread per cell and the weights in the constant bank 26.1 ms, 183, 55 and
+// 46.9 us (16^3 fills 32 of 152 SMs that way, here 128). Third hidden layer: 16^3 15 us (70).
+// The registers are at their limit of 128 (fourteen warps): the network's loop is sensitive to
+// what lives around it (the parameters copied before the first load instead of after: 8 % slower).
 #include "cell.cuh"
 #include "force.cuh"
+#include "launch.cuh"
 #include "net_f32.cuh"
 
 namespace lbm {
@@ -92,6 +95,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_nco_f32_kernel(const StepArg
     auto cell_of = [&](int i) {
         return (static_cast<long long>(blockIdx.x) + static_cast<long long>(i) * gridDim.x) * kTile + lane;
     };
+    overlap_wait();
     if (FORCED) {
         frc::load_fh2(ff.fhat, sh.fh2);
         if (tid < frc::kProjValues) sh.red[tid] = 0ull;
@@ -136,13 +140,13 @@ __global__ void __launch_bounds__(kThreads, 1) step_nco_f32_kernel(const StepArg
                 float* const row = sh.rows[w] + l * net_row(4);
                 float acc[2][4][kHalf];
                 set_bias(net.b2, lane, acc);
-                mat_vec<4>(net.W2, lane, acc, RowColumns<4>{row});
+                mat_vec<4, 1>(net.W2, lane, acc, RowColumns<4>{row});
                 if constexpr (DEEP) {  // 27-20-20-20-4: a third hidden layer before the group sum
                     __syncwarp();      // h1 is read before h2 replaces it
                     store_relu(row, lane, acc);
                     __syncwarp();
                     set_bias(net.bd, lane, acc);
-                    mat_vec<4>(net.Wd, lane, acc, RowColumns<4>{row});
+                    mat_vec<4, 1>(net.Wd, lane, acc, RowColumns<4>{row});
                 }
                 // the sums of the two halves, the first warp's then the second's on top
                 float* const out = &sh.part[i & 1][p][l][(lane >> 4) * kHalf];
@@ -224,43 +228,42 @@ __global__ void __launch_bounds__(kThreads, 1) step_nco_f32_kernel(const StepArg
 }
 
 template <int STORAGE, int BC, bool FORCED, bool DEEP>
-cudaError_t launch_t(const StepArgs& a, const FusedForce& ff, const NetParams* net, cudaStream_t s) {
+cudaError_t launch_t(const StepArgs& a, const FusedForce& ff, const NetParams* net, bool overlap, cudaStream_t s) {
     static std::atomic<unsigned long long> attr{0};
     const cudaError_t e = ensure_dynamic_smem(step_nco_f32_kernel<STORAGE, BC, FORCED, DEEP>,
                                               static_cast<int>(sizeof(NetShared)), attr);
     if (e != cudaSuccess) return e;
     const int ntiles = static_cast<int>((a.d.ncell + kTile - 1) / kTile);
     const int sms = sm_count();
-    step_nco_f32_kernel<STORAGE, BC, FORCED, DEEP><<<ntiles < sms ? ntiles : sms, kThreads, sizeof(NetShared), s>>>(
-        a, net, ff, ntiles);
-    return cudaGetLastError();
+    return launch_kernel(step_nco_f32_kernel<STORAGE, BC, FORCED, DEEP>, static_cast<unsigned>(ntiles < sms ? ntiles : sms),
+                         kThreads, sizeof(NetShared), s, overlap, a, net, ff, ntiles);
 }
 
 template <int STORAGE, int BC, bool FORCED>
-cudaError_t launch_d(const StepArgs& a, const FusedForce& ff, bool deep, const NetParams* net, cudaStream_t s) {
-    return deep ? launch_t<STORAGE, BC, FORCED, true>(a, ff, net, s) : launch_t<STORAGE, BC, FORCED, false>(a, ff, net, s);
+cudaError_t launch_d(const StepArgs& a, const FusedForce& ff, bool deep, const NetParams* net, bool overlap, cudaStream_t s) {
+    return deep ? launch_t<STORAGE, BC, FORCED, true>(a, ff, net, overlap, s) : launch_t<STORAGE, BC, FORCED, false>(a, ff, net, overlap, s);
 }
 
 template <int STORAGE>
-cudaError_t launch_s(const StepArgs& a, const FusedForce* ff, int bc, bool deep, const NetParams* net, cudaStream_t s) {
+cudaError_t launch_s(const StepArgs& a, const FusedForce* ff, int bc, bool deep, const NetParams* net, bool overlap, cudaStream_t s) {
     if (ff) {  // forcing runs on periodic boxes only
         if (bc != LBM_BC_PERIODIC) return cudaErrorInvalidValue;
-        return launch_d<STORAGE, LBM_BC_PERIODIC, true>(a, *ff, deep, net, s);
+        return launch_d<STORAGE, LBM_BC_PERIODIC, true>(a, *ff, deep, net, overlap, s);
     }
     const FusedForce none{};
-    if (bc == LBM_BC_PERIODIC) return launch_d<STORAGE, LBM_BC_PERIODIC, false>(a, none, deep, net, s);
-    if (bc == LBM_BC_TGV_REDUCED) return launch_d<STORAGE, LBM_BC_TGV_REDUCED, false>(a, none, deep, net, s);
-    return launch_d<STORAGE, LBM_BC_MIRROR, false>(a, none, deep, net, s);
+    if (bc == LBM_BC_PERIODIC) return launch_d<STORAGE, LBM_BC_PERIODIC, false>(a, none, deep, net, overlap, s);
+    if (bc == LBM_BC_TGV_REDUCED) return launch_d<STORAGE, LBM_BC_TGV_REDUCED, false>(a, none, deep, net, overlap, s);
+    return launch_d<STORAGE, LBM_BC_MIRROR, false>(a, none, deep, net, overlap, s);
 }
 
 }  // namespace
 
 cudaError_t launch_step_nco_f32(const StepArgs& a, const FusedForce* ff, int storage, int bc, bool deep,
-                                const NetParams* d_net, cudaStream_t s) {
+                                const NetParams* d_net, bool overlap, cudaStream_t s) {
     switch (storage) {
-        case LBM_STORE_F32: return launch_s<LBM_STORE_F32>(a, ff, bc, deep, d_net, s);
-        case LBM_STORE_F16_DEV: return launch_s<LBM_STORE_F16_DEV>(a, ff, bc, deep, d_net, s);
-        default: return launch_s<LBM_STORE_BF16_DEV>(a, ff, bc, deep, d_net, s);
+        case LBM_STORE_F32: return launch_s<LBM_STORE_F32>(a, ff, bc, deep, d_net, overlap, s);
+        case LBM_STORE_F16_DEV: return launch_s<LBM_STORE_F16_DEV>(a, ff, bc, deep, d_net, overlap, s);
+        default: return launch_s<LBM_STORE_BF16_DEV>(a, ff, bc, deep, d_net, overlap, s);
     }
 }
 

@@ -162,7 +162,7 @@ cudaError_t launch_step(const StepArgs& a, const FusedForce* ff, int op, int sto
     if (op == LBM_OP_NCO && net_prec == LBM_NET_BF16X3)
         return launch_step_nco_tc3(a, ff, storage, bc, deep, net_weights, wait_cycles, s);
     if (op == LBM_OP_NCO)
-        return launch_step_nco_f32(a, ff, storage, bc, deep, static_cast<const NetParams*>(net_weights), s);
+        return launch_step_nco_f32(a, ff, storage, bc, deep, static_cast<const NetParams*>(net_weights), overlap, s);
     switch (storage) {
         case LBM_STORE_F32: return launch_step_s<LBM_STORE_F32>(a, ff, op, bc, overlap, s);
         case LBM_STORE_F16_DEV: return launch_step_s<LBM_STORE_F16_DEV>(a, ff, op, bc, overlap, s);

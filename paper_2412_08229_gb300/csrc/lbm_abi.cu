@@ -839,7 +839,7 @@ lbm_status lbm_step(lbm_ctx* c, int nsteps) {
             break;
         }
         const double* row = forced ? c->d_draws + c->draws_head * kDrawRow : nullptr;
-        lbm_status st = enqueue_step(c, c->cur, c->stream, row, false);
+        lbm_status st = enqueue_step(c, c->cur, c->stream, row, false, c->rec_k > 0);
         if (st) return st;
         if (forced) {
             ++c->draws_head;
@@ -1010,7 +1010,7 @@ static lbm_status backward_sweep(lbm_ctx* c, const char* who, const float* dL_du
             const FusedForce ff{forced ? rec_fhat_at(c, t) : nullptr, c->d_ftab, nullptr, c->fscale};
             LBM_CK(c, launch_step(a, forced ? &ff : nullptr, c->cfg.op, c->cfg.storage, c->cfg.boundary,
                                   c->cfg.net_precision, c->net && c->net->deep, c->net_w, c->tc_shape, c->wait_cycles,
-                                  false, c->stream));
+                                  true, c->stream));
         }
         for (long long t = b0 - 1; t >= a0; --t) {
             void* state_t = c->adj_work[static_cast<size_t>(t - a0)];

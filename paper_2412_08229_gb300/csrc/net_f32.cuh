@@ -87,7 +87,7 @@ __device__ __forceinline__ void first_layer(const NetParams& net, int p, int hal
     constexpr int NC = 2 / LANES, C = 4 / LANES, R = net_row(C);
     const int j0 = half * kHalf + (lane >> 4) * 5;
     float* const out = rows + (lane & 15) * R + j0;
-#pragma unroll 1
+#pragma unroll
     for (int i = 0; i < 5; ++i) {
         float w[28];
 #pragma unroll
@@ -109,11 +109,13 @@ __device__ __forceinline__ void first_layer(const NetParams& net, int p, int hal
 }
 
 // acc[r][c][o] += sum_k W[10 og + o][k] x[r][c][k] for the lane's ten units (og = lane / 16)
-// and the columns of the rows l + 16 r; get(k, v) loads v[r][c] = x[r][c][k..k+3].
-template <int C, typename F>
+// and the columns of the rows l + 16 r; get(k, v) loads v[r][c] = x[r][c][k..k+3]. UNROLL:
+// steps of four inputs per loop iteration, all five where registers are left for it (the
+// adjoint, 32^3 210 -> 203 us; the step, at its limit of 128, loses 2 %).
+template <int C, int UNROLL, typename F>
 __device__ __forceinline__ void mat_vec(const float (&W)[kHidden][kHidden], int lane, float (&acc)[2][C][kHalf], F&& get) {
     const float* w0 = &W[(lane >> 4) * kHalf][0];
-#pragma unroll 1
+#pragma unroll UNROLL
     for (int k = 0; k < kHidden; k += 4, w0 += 4) {
         float4 v[2][C];
         get(k, v);
