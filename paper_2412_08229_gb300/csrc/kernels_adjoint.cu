@@ -594,12 +594,12 @@ __global__ void __launch_bounds__(kAdjThreads, (!DEEP && LANES == 2) ? 2 : 1)
         __syncthreads();
         for (int i = tid; i < Q * kCells; i += kAdjThreads) {  // the twelve warps' parts and the relaxation's
             const int t = i / kCells, c = i % kCells;
-            float v = sh.mu[c][t];
+            float v = 0.0f;  // the parts first: one rounding at the size of the relaxation's term
 #pragma unroll
             for (int q = 0; q < kNetWarps; ++q)
 #pragma unroll
                 for (int g = 0; g < 2; ++g) v += sh.h1[q][(2 * t + g) * kCells + c];
-            sh.dm[t][c] = v;
+            sh.dm[t][c] = sh.mu[c][t] + v;
         }
         __syncthreads();
 
