@@ -19,10 +19,34 @@ constexpr int kNumTheta = 27 * 20 + 20 + 20 * 20 + 20 + 20 * 4 + 4;  // 1064 (Se
 constexpr int kNumThetaDeep = kNumTheta + 20 * 20 + 20;  // 1484: a third hidden layer of 20 (Sec. IV)
 constexpr int kForcedModes = 16;  // half-space integer modes with 1 <= |k| <= 2
 
+// Parity class of moment t (tensor order): the axes it is odd in.
+__host__ __device__ constexpr int odd_mask(int t) {
+    return ((ex_of(t) == 1) << 2) | ((ey_of(t) == 1) << 1) | (ez_of(t) == 1);
+}
+
+// Place of moment t in class order: the moments of a class side by side in tensor order, the
+// classes odd in no axis (eight moments), one (four each), two (two each) and three (one), so
+// that aligned groups of four places hold at most two classes.
+__host__ __device__ constexpr int class_rank(int c) { return c < 3 ? c : (c == 3 ? 4 : (c == 4 ? 3 : c)); }
+__host__ __device__ constexpr int class_pos(int t) {
+    int n = 0;
+    for (int u = 0; u < Q; ++u) {
+        const int a = class_rank(odd_mask(u)), b = class_rank(odd_mask(t));
+        n += a < b || (a == b && u < t);
+    }
+    return n;
+}
+// Class of place k.
+__host__ __device__ constexpr int class_at(int k) {
+    for (int t = 0; t < Q; ++t)
+        if (class_pos(t) == k) return odd_mask(t);
+    return 0;
+}
+
 // Parameters of the FP32 network as its kernels lay them out in shared memory (copied as a
 // whole from device memory at the start of a block).
 // W1p[p] = W1 with its columns rearranged for axis permutation p: the input of
-// group element (p, s) is then sgn(s, t) * m_t in tensor order t (net_f32.cuh).
+// group element (p, s) is then sgn(s, t) * m_t (net_f32.cuh); the column of m_t is class_pos(t).
 struct alignas(16) NetParams {
     float W1p[6][kHidden][28];         // 27 columns, then b1: rows of seven 16-byte quadruples
     float W2[kHidden][kHidden];

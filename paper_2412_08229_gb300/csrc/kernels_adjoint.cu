@@ -24,6 +24,12 @@
 // nothing of the forward is computed twice. The weight gradients are outer products summed
 // over columns: a lane has 10 x 6 outputs, 60 FMAs for 15 floats read.
 //
+// lam's arithmetic is that of one thread per cell, bit for bit: the group sum in the order of the
+// group (handed from warp to warp), the cotangent of m as the relaxation's part plus 120 products
+// one after the other. A sweep of 200 steps turns other roundings into up to 3e-5 of the
+// gradient. Sums that end in the gradient are grouped freely. (The two sums in order: 32^3
+// training pass 61.1 -> 64.9 ms.)
+//
 // A block per SM walks over the tiles and keeps the parameter gradients in FP64 in shared
 // memory, so the global atomics come once per block (a block per tile: 32^3 225 us).
 //
@@ -126,27 +132,47 @@ struct AdjShared {
     static constexpr int kCells = 32 / LANES;
     static constexpr int kCols = 4 / LANES;
     static constexpr int kRow = net_row(kCols);
-    // per warp: the staged cotangents of one column per lane (32 x 20), the partial sums of
-    // the last hidden layer, and at the end the weight gradients of the hidden layers and of
-    // the warp's half of W1p
+    // per warp: the staged cotangents of one column per lane (32 x 20), and at the end the weight
+    // gradients of the hidden layers and of the warp's half of W1p
     static constexpr int kD1 = DEEP ? 2 * kGradBlock : kGradBlock;
     static constexpr int kStage = (kD1 + (Q + 1) * kHalf + 3) / 4 * 4;
     static_assert(kStage >= 32 * kHidden, "stage holds a column per lane");
-    static_assert(2 * Q * kCells <= 32 * kRow, "the moment cotangents fit a warp's rows");
 
     NetParams net;
     double grad[GradLayout<DEEP>::kLen];  // the block's parameter gradients, summed over its tiles
-    float h1[kNetWarps][net_rows(kCols)];  // h1, then delta h1, then E, then the partial cotangent of m
+    float h1[kNetWarps][net_rows(kCols)];  // h1, then delta h1, then E
     float h2[DEEP ? kNetWarps : 1][32][DEEP ? kRow : 4];  // h2, then delta h2 (third hidden layer)
     float stage[kNetWarps][kStage];
     float m[kCells][28];      // moments (tensor order), 1 (the bias input)
-    float mu[kCells][28];     // mu*, then the relaxation's part of dL/dm
-    float dm[Q][kCells];
-    float hsum[kCells][kHidden];
+    float mu[kCells][28];     // mu* (class order), then the relaxation's part of dL/dm, then dL/dm
+    float hsum[kCells][kHidden];  // group sum of the last hidden layer
     float v3[kCells][kHidden];  // cotangent of the last hidden layer, the same for every group element
     float gbar[kCells][kOut];
     float rates[kCells][kOut];
 };
+
+// A cell's 27 values to and from a row in class order.
+__device__ __forceinline__ void store_class_order(float* row, const float* v) {
+    static_for<Q>([&](auto T) { row[class_pos(decltype(T)::value)] = v[decltype(T)::value]; });
+}
+__device__ __forceinline__ void load_class_order(float* v, const float* row) {
+    static_for<Q>([&](auto T) { v[decltype(T)::value] = row[class_pos(decltype(T)::value)]; });
+}
+
+// Classes of the places 4 g, 4 g + 1 (bits 8 g..) and 4 g + 2, 4 g + 3 (bits 8 g + 4..).
+constexpr unsigned long long make_class_of_pair() {
+    unsigned long long r = 0;
+    for (int g = 0; g < 7; ++g)
+        for (int i = 0; i < 2; ++i) r |= static_cast<unsigned long long>(class_at(4 * g + 2 * i)) << (8 * g + 4 * i);
+    return r;
+}
+constexpr bool pairs_of_places_share_a_class() {
+    for (int k = 0; k < Q - 1; k += 2)
+        if (class_at(k) != class_at(k + 1)) return false;
+    return true;
+}
+static_assert(pairs_of_places_share_a_class(), "two places, one class");
+constexpr unsigned long long kClassOfPair = make_class_of_pair();
 
 // Outer products summed over columns: a warp's 20 x 21 gradient (W | b) in tiles of 10 x 5
 // (and the bias column) over 2 x 4 lanes; the four groups of eight lanes take the rows
@@ -201,11 +227,18 @@ struct OuterTile {
     }
 };
 
+// Hands the tile's group sums from warp w - 1 to warp w: a named barrier of the two, the pair's
+// own (pair_sync) inside a permutation.
+__device__ __forceinline__ int group_sum_barrier(int w) { return w & 1 ? (w >> 1) + 1 : kNetWarps / 2 + (w >> 1); }
+__device__ __forceinline__ void group_sum_wait(int w) { asm volatile("bar.sync %0, 64;" ::"r"(group_sum_barrier(w)) : "memory"); }
+__device__ __forceinline__ void group_sum_pass(int w) { asm volatile("bar.arrive %0, 64;" ::"r"(group_sum_barrier(w)) : "memory"); }
+
 template <int STORAGE, int BC, bool DEEP, int LANES>
 __global__ void __launch_bounds__(kAdjThreads, (!DEEP && LANES == 2) ? 2 : 1)
     adjoint_step_kernel(const AdjArgs a, const NetParams* __restrict__ net_in, int ntiles) {
     using GL = GradLayout<DEEP>;
     using SH = AdjShared<DEEP, LANES>;
+    using At = BySigns<LANES>;
     constexpr int kCells = SH::kCells, C = SH::kCols, kRow = SH::kRow;
     extern __shared__ __align__(16) uint8_t adj_smem_raw[];
     SH& sh = *reinterpret_cast<SH*>(adj_smem_raw);
@@ -215,6 +248,7 @@ __global__ void __launch_bounds__(kAdjThreads, (!DEEP && LANES == 2) ? 2 : 1)
     const int w = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform, and seen to be
     const int p = w >> 1, half = w & 1;
     const int l = lane & 15, og = lane >> 4;  // the rows l and l + 16, units [10 og, 10 og + 10)
+    const int own = w == 0 ? tid : tid - 32;  // first of a thread's parameters (all warps but 1)
     load_params(&sh.net, net_in, tid, kAdjThreads);
     for (int i = tid; i < GL::kLen; i += kAdjThreads) sh.grad[i] = 0.0;
     overlap_wait();
@@ -264,9 +298,8 @@ __global__ void __launch_bounds__(kAdjThreads, (!DEEP && LANES == 2) ? 2 : 1)
                         for (int e = 0; e < Q; ++e) sh.m[lane][e] = m[e];
                         sh.m[lane][Q] = 1.0f;
                     } else {
-                        populations_transpose_inplace(v);  // mu* = M^-T lam* (tensor order)
-#pragma unroll
-                        for (int e = 0; e < Q; ++e) sh.mu[lane][e] = v[e];
+                        populations_transpose_inplace(v);  // mu* = M^-T lam*
+                        store_class_order(sh.mu[lane], v);
                     }
                 }
             }
@@ -288,17 +321,20 @@ __global__ void __launch_bounds__(kAdjThreads, (!DEEP && LANES == 2) ? 2 : 1)
                             push_target<BC>(x, y, z, j, a.d, i, dst);
                             v[j] = a.lam_in[static_cast<size_t>(i) * a.d.ncell + dst];
                         }
-                        populations_transpose_inplace(v);  // mu* = M^-T lam* (tensor order)
+                        populations_transpose_inplace(v);  // mu* = M^-T lam*
                     }
                 } else {  // a cell past the end: no cotangent, so it adds nothing
 #pragma unroll
                     for (int e = 0; e < Q; ++e) v[e] = 0.0f;
                     if (w == 0) v[0] = 1.0f;
                 }
-                float* dst = w == 0 ? sh.m[lane] : sh.mu[lane];
+                if (w == 0) {
 #pragma unroll
-                for (int e = 0; e < Q; ++e) dst[e] = v[e];
-                dst[Q] = 1.0f;
+                    for (int e = 0; e < Q; ++e) sh.m[lane][e] = v[e];
+                    sh.m[lane][Q] = 1.0f;
+                } else {
+                    store_class_order(sh.mu[lane], v);
+                }
             }
         }
         __syncthreads();
@@ -313,7 +349,7 @@ __global__ void __launch_bounds__(kAdjThreads, (!DEEP && LANES == 2) ? 2 : 1)
 #pragma unroll
                 for (int e = 0; e < 28; e += 4)
                     *reinterpret_cast<float4*>(&m[k][e]) = *reinterpret_cast<const float4*>(&sh.m[l + 16 * k][e]);
-            first_layer<LANES>(net, p, half, lane, m, sh.h1[2 * p]);
+            first_layer<At>(net, p, half, lane, m, sh.h1[2 * p]);
         }
         pair_sync(p);
 
@@ -332,35 +368,37 @@ __global__ void __launch_bounds__(kAdjThreads, (!DEEP && LANES == 2) ? 2 : 1)
                 mat_vec<C, 5>(net.Wd, lane, acc, RowColumns<C>{row2});
             }
 #pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                float hs[kHalf];
-#pragma unroll
-                for (int o = 0; o < kHalf; ++o) hs[o] = 0.0f;
+            for (int r = 0; r < 2; ++r)
 #pragma unroll
                 for (int c = 0; c < C; ++c) {
                     uint32_t k = 0u;
 #pragma unroll
                     for (int o = 0; o < kHalf; ++o) {
-                        const float h = fmaxf(acc[r][c][o], 0.0f);
-                        hs[o] += h;
-                        k = __funnelshift_l(__float_as_uint(0.0f - h), k, 1);  // the sign of -h: h > 0
+                        acc[r][c][o] = fmaxf(acc[r][c][o], 0.0f);
+                        k = __funnelshift_l(__float_as_uint(0.0f - acc[r][c][o]), k, 1);  // the sign of -h: h > 0
                     }
                     k <<= og ? 32 - kHidden : 32 - kHalf;
                     mask[r][c] = k | __shfl_xor_sync(0xffffffffu, k, 16);
                 }
+            // the group sum, element by element in the order of the group (the rates are those of the
+            // step, bit for bit): warp after warp adds its sign vectors to it
+            if (w > 0) group_sum_wait(w);
 #pragma unroll
-                for (int o = 0; o < kHalf; o += 2)
-                    *reinterpret_cast<float2*>(&sh.stage[w][(l + 16 * r) * kHidden + og * kHalf + o]) = make_float2(hs[o], hs[o + 1]);
-            }
-        }
-        __syncthreads();
-        for (int i = tid; i < kCells * kHidden; i += kAdjThreads) {  // group sum, i = cell * 20 + unit
-            float v = 0.0f;
+            for (int k = 0; k < At::kCells; ++k)
 #pragma unroll
-            for (int q = 0; q < kNetWarps; ++q)
+                for (int o = 0; o < kHalf; o += 2) {
+                    float2* const q = reinterpret_cast<float2*>(&sh.hsum[l + 16 * k][og * kHalf + o]);
+                    float2 h = w > 0 ? *q : make_float2(0.0f, 0.0f);
 #pragma unroll
-                for (int l = 0; l < LANES; ++l) v += sh.stage[q][i + l * kCells * kHidden];
-            (&sh.hsum[0][0])[i] = v;
+                    for (int r = k; r < k + LANES; ++r)
+#pragma unroll
+                        for (int c = 0; c < C; ++c) {
+                            h.x += acc[r][c][o];
+                            h.y += acc[r][c][o + 1];
+                        }
+                    *q = h;
+                }
+            if (w + 1 < kNetWarps) group_sum_pass(w + 1);
         }
         __syncthreads();
         if (tid < kOut * kCells) {  // rates and the cotangents of tau~, one (cell, output) per thread
@@ -372,10 +410,10 @@ __global__ void __launch_bounds__(kAdjThreads, (!DEEP && LANES == 2) ? 2 : 1)
             const float e = expf(t);
             const float tau_n = 0.5f / (1.0f + e) + 0.5f;
             float gw = 0.0f;
-#pragma unroll
-            for (int k = 0; k < Q; ++k)
-                if (order_of(k) >= 3)
-                    gw -= order_of(k) == n + 3 ? sh.mu[c][k] * sh.m[c][k] : 0.0f;
+            static_for<Q>([&](auto K) {
+                constexpr int k = decltype(K)::value, q = class_pos(k);
+                if (order_of(k) >= 3 && order_of(k) == n + 3) gw = fmaf(-sh.mu[c][q], sh.m[c][k], gw);
+            });
             // d omega / d tau~ = sigma (1 - sigma) / (2 tau_n^2), sigma = 1 / (1 + e^{tau~})
             const float sg = 1.0f / (1.0f + e);
             sh.rates[c][n] = 1.0f / tau_n;
@@ -396,7 +434,8 @@ __global__ void __launch_bounds__(kAdjThreads, (!DEEP && LANES == 2) ? 2 : 1)
             const long long cell = cell0 + lane;
             const bool valid = cell < a.d.ncell;
             const float* m = sh.m[lane];
-            float* mu_row = sh.mu[lane];
+            float mus[Q];
+            load_class_order(mus, sh.mu[lane]);
             const float omega_nu = 1.0f / a.tau;
             const float irho = 1.0f / m[0];
             float dm[Q];
@@ -405,7 +444,7 @@ __global__ void __launch_bounds__(kAdjThreads, (!DEEP && LANES == 2) ? 2 : 1)
 #pragma unroll
             for (int e = 0; e < Q; ++e) {
                 const int n = order_of(e);
-                const float mu = mu_row[e];
+                const float mu = mus[e];
                 if (n <= 1) {
                     dm[e] += mu;
                 } else if (n == 2) {
@@ -443,8 +482,7 @@ __global__ void __launch_bounds__(kAdjThreads, (!DEEP && LANES == 2) ? 2 : 1)
                     dm[e] += (1.0f - sh.rates[lane][n - 3]) * mu;
                 }
             }
-#pragma unroll
-            for (int e = 0; e < Q; ++e) mu_row[e] = dm[e];
+            store_class_order(sh.mu[lane], dm);
         }
         __syncwarp();
 
@@ -526,46 +564,33 @@ __global__ void __launch_bounds__(kAdjThreads, (!DEEP && LANES == 2) ? 2 : 1)
         }
         pair_sync(p);
 
-        // ---- first layer: E of class c in place of delta h1 of sign vector c, and the cotangent of
-        // m through the lane's five units
+        // ---- first layer: E of class c in place of delta h1 of sign vector c
         {
-            using At = ColumnOf<LANES>;
-            constexpr int NC = 2 / LANES;
-            float dm[NC][Q];
-#pragma unroll
-            for (int k = 0; k < NC; ++k)
-#pragma unroll
-                for (int t = 0; t < Q; ++t) dm[k][t] = 0.0f;
             const int j0 = half * kHalf + og * 5;
             float* const q = sh.h1[2 * p] + l * kRow + j0;
 #pragma unroll 1
-            for (int i = 0; i < 5; ++i) {
-                float wt[28];
+            for (int i = 0; i < 5; ++i)
 #pragma unroll
-                for (int t = 0; t < 28; t += 4)
-                    *reinterpret_cast<float4*>(wt + t) = *reinterpret_cast<const float4*>(&net.W1p[p][j0 + i][t]);
-#pragma unroll
-                for (int k = 0; k < NC; ++k) {
+                for (int k = 0; k < At::kCells; ++k) {
                     float e[8];
                     auto at = [&](int s) -> float& {
-                        return q[At::half(s) * net_rows(C) + (At::row(s) + 16 * k) * kRow + At::col(s) * kHidden + i];
+                        return q[At::half(s, k) * net_rows(C) + At::row(s, k) * kRow + At::col(s, k) * kHidden + i];
                     };
 #pragma unroll
                     for (int s = 0; s < 8; ++s) e[s] = at(s);
                     wht<8>(e);
 #pragma unroll
                     for (int s = 0; s < 8; ++s) at(s) = e[s];
-#pragma unroll
-                    for (int t = 0; t < Q; ++t) dm[k][t] = fmaf(wt[t], e[odd_mask(t)], dm[k][t]);
                 }
-            }
-            pair_sync(p);
+        }
+        pair_sync(p);
+        {
+            const int t = lane < Q ? lane : Q;
+            const int ex = t % 3, ey = (t / 3) % 3, ez = t / 9;
+            const int c = t < Q ? ((ex == 1) << 2) | ((ey == 1) << 1) | (ez == 1) : 0;
             // dW1p[j][t] = sum over cells of E[c(t)][j] m_t, lane t (lane 27: db1, the bias input of class 0)
             {
-                const int t = lane < Q ? lane : Q;
-                const int ex = t % 3, ey = (t / 3) % 3, ez = t / 9;
-                const int c = t < Q ? ((ex == 1) << 2) | ((ey == 1) << 1) | (ez == 1) : 0;
-                const float* er = sh.h1[2 * p + At::half(c)] + At::row(c) * kRow + At::col(c) * kHidden + half * kHalf;
+                const float* er = sh.h1[2 * p + At::half(c, 0)] + At::row(c, 0) * kRow + At::col(c, 0) * kHidden + half * kHalf;
                 float g[kHalf];
 #pragma unroll
                 for (int j = 0; j < kHalf; ++j) g[j] = 0.0f;
@@ -584,40 +609,55 @@ __global__ void __launch_bounds__(kAdjThreads, (!DEEP && LANES == 2) ? 2 : 1)
                     for (int j = 0; j < kHalf; ++j) sh.stage[w][SH::kD1 + t * kHalf + j] = g[j];
                 }
             }
-            pair_sync(p);
-            // the rows are free: the two five-unit parts of the cells' cotangents, [t][og][cell]
+            __syncthreads();
+            // the network's part of the cotangent of m, W1p[j][t] E[c(t)][j] on top of the relaxation's
+            // part, permutation by permutation and unit by unit (a sum whose last bits the sweep carries to
+            // the first step): a lane has a cell and four places of the class order. Warps 0 to 6 have 32
+            // cells each (LANES = 1), or 0 to 3 16 cells and two groups of places
+            const int g = LANES == 1 ? w : 2 * w + og, cell = LANES == 1 ? lane : l;
+            if (g < 7) {
+                const int ca = (kClassOfPair >> (8 * g)) & 7, cb = (kClassOfPair >> (8 * g + 4)) & 7;
+                auto e_of = [&](int k) { return sh.h1[At::half(k, 0)] + (At::row(k, 0) + cell) * kRow + At::col(k, 0) * kHidden; };
+                const float *ea = e_of(ca), *eb = e_of(cb);
+                float4* const q = reinterpret_cast<float4*>(&sh.mu[cell][4 * g]);
+                float4 dm = *q;
+#pragma unroll 1
+                for (int pp = 0; pp < kNetWarps / 2; ++pp, ea += 2 * net_rows(C), eb += 2 * net_rows(C))
 #pragma unroll
-            for (int t = 0; t < Q; ++t)
-#pragma unroll
-                for (int k = 0; k < NC; ++k) rows[(2 * t + og) * kCells + l + 16 * k] = dm[k][t];
-        }
-        __syncthreads();
-        for (int i = tid; i < Q * kCells; i += kAdjThreads) {  // the twelve warps' parts and the relaxation's
-            const int t = i / kCells, c = i % kCells;
-            float v = 0.0f;  // the parts first: one rounding at the size of the relaxation's term
-#pragma unroll
-            for (int q = 0; q < kNetWarps; ++q)
-#pragma unroll
-                for (int g = 0; g < 2; ++g) v += sh.h1[q][(2 * t + g) * kCells + c];
-            sh.dm[t][c] = sh.mu[c][t] + v;
+                    for (int j = 0; j < kHidden; j += 4) {
+                        const float4 a4 = *reinterpret_cast<const float4*>(ea + j);
+                        const float4 b4 = LANES == 1 && ca == cb ? a4 : *reinterpret_cast<const float4*>(eb + j);
+                        auto add = [&](int jj, float a1, float b1) {
+                            const float4 wt = *reinterpret_cast<const float4*>(&net.W1p[pp][jj][4 * g]);
+                            dm.x = fmaf(wt.x, a1, dm.x);
+                            dm.y = fmaf(wt.y, a1, dm.y);
+                            dm.z = fmaf(wt.z, b1, dm.z);
+                            dm.w = fmaf(wt.w, b1, dm.w);
+                        };
+                        add(j, a4.x, b4.x);
+                        add(j + 1, a4.y, b4.y);
+                        add(j + 2, a4.z, b4.z);
+                        add(j + 3, a4.w, b4.w);
+                    }
+                *q = dm;
+            }
         }
         __syncthreads();
 
-        if (w == 0) {  // lam_t = M^T dL/dm
+        if (w == 1) {  // lam_t = M^T dL/dm, by the warp that fills mu again
             const long long cell = cell0 + lane;
             if (lane < kCells && cell < a.d.ncell) {
                 float v[Q];
-#pragma unroll
-                for (int e = 0; e < Q; ++e) v[e] = sh.dm[e][lane];
+                load_class_order(v, sh.mu[lane]);
                 moments_transpose_inplace(v);
 #pragma unroll
                 for (int i = 0; i < Q; ++i) a.lam_out[static_cast<size_t>(i) * a.d.ncell + cell] = v[i];
             }
-            continue;  // the next tile's first barrier keeps the other warps' sums from it
+            continue;  // until the next tile's first barrier it writes nothing that the others still read
         }
         // parameter gradients of the tile, a thread's own: sums over the warps (W1: the six
         // permutations' columns that a printed column went to), added in FP64
-        for (int i = tid - 32; i < GL::kLen; i += kAdjThreads - 32) {
+        for (int i = own; i < GL::kLen; i += kAdjThreads - 32) {
             float v = 0.0f;
             if (i < GL::kW2) {
                 const int j = i < GL::kB1 ? i / Q : i - GL::kB1, k = i < GL::kB1 ? i % Q : Q;
@@ -642,8 +682,8 @@ __global__ void __launch_bounds__(kAdjThreads, (!DEEP && LANES == 2) ? 2 : 1)
             sh.grad[i] += static_cast<double>(v);
         }
     }
-    if (w != 0)
-        for (int i = tid - 32; i < GL::kLen; i += kAdjThreads - 32) atomicAdd(&a.grad[i], sh.grad[i]);
+    if (w != 1)
+        for (int i = own; i < GL::kLen; i += kAdjThreads - 32) atomicAdd(&a.grad[i], sh.grad[i]);
 }
 
 // lam[i] (=, or += when accumulate) sum_a g_a (c_ia - u_a) / rho + dL/drho for the state

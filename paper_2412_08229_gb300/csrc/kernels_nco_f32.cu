@@ -2,10 +2,15 @@
 // network in FP32 on the CUDA cores.
 //
 // A persistent block per SM takes tiles of 32 cells. Its twelve network warps evaluate one
-// (permutation, half of the sign vectors) each (net_f32.cuh); beside them a loader warp pulls
-// the next tile's populations and forms its moments, and a finisher warp sums the previous
-// tile's group sum over the twelve warps, forms the rates, relaxes and stores. The three
-// stages are one tile apart and meet at one barrier per tile.
+// (permutation, half of the cells) each (net_f32.cuh) and add their sign vectors to the group sum
+// in the order of the group, permutation after permutation; beside them a loader warp pulls the
+// next tile's populations and forms its moments, and a finisher warp takes the previous tile's
+// group sum, forms the rates, relaxes and stores. The three stages are one tile apart and meet
+// at one barrier per tile.
+//
+// The order of the group sum and of everything after it is that of one thread per cell, bit for
+// bit: a long unroll carries a last bit to 1e-5 of its gradient (handing the sum from one
+// permutation to the next costs 32^3 50.2 -> 52.9 us, 96^3 1185 -> 1264).
 //
 // What bounds it (32^3, ncu): issue, 58 % of the cycles, in bursts: the twelve warps go through
 // their FMA and shared-memory phases nearly together; shared-memory wavefronts 48 %. Step of
@@ -30,23 +35,27 @@ constexpr int kThreads = 32 * (kNetWarps + 2);
 struct NetShared {
     NetParams net;
     float rows[kNetWarps][net_rows(4)];          // the columns' h1 (then h2)
-    float part[2][kNetWarps / 2][kTile][kHidden];      // sums of the last hidden layer over a permutation's sign vectors
-    float m[3][kTile][28];                             // moments (tensor order), rho - 1
+    float part[2][kTile][kHidden];                     // sums of the last hidden layer over the group, permutation by permutation
+    float m[2][kTile][28];                             // moments (tensor order)
     float df[3][Q][kTile];                             // the pulled deviations
     float fh2[kForcedModes * 6];                       // forced steps: 2 F^
     unsigned long long red[frc::kProjValues];          // forced steps: the block's projection sums
 };
 static_assert(sizeof(NetShared) <= 227 * 1024, "shared memory budget");
 
+// Hands the tile's group sums from the two warps of permutation p - 1 to those of p: a named
+// barrier of the four (pair_sync has the ids 1 to 6).
+__device__ __forceinline__ void group_sum_wait(int p) { asm volatile("bar.sync %0, 128;" ::"r"(kNetWarps / 2 + p) : "memory"); }
+__device__ __forceinline__ void group_sum_pass(int p) { asm volatile("bar.arrive %0, 128;" ::"r"(kNetWarps / 2 + p) : "memory"); }
+
 template <int STORAGE, int BC>
 __device__ __forceinline__ void load_tile(const StepArgs& a, long long cell, float (*m)[28], float (*df)[kTile], int lane) {
     float v[Q], mo[Q];
-    float drho = 0.0f;
     if (cell < a.d.ncell) {
         int x, y, z;
         cell_coords(cell, a.d, x, y, z);
         load_pulled_offsets<STORAGE, BC>(a.src, a.d, x, y, z, v);
-        drho = moments_from_dev(v, mo);
+        moments_from_dev(v, mo);
         if (!(mo[0] >= a.rho_min && mo[0] <= a.rho_max)) atomicOr(a.status, 1);
     } else {
 #pragma unroll
@@ -58,7 +67,6 @@ __device__ __forceinline__ void load_tile(const StepArgs& a, long long cell, flo
         df[e][lane] = v[e];
         m[lane][e] = mo[e];
     }
-    m[lane][Q] = drho;
 }
 
 // The block's first tile, which nothing overlaps, on the reduced domain, whose branches
@@ -108,11 +116,10 @@ __global__ void __launch_bounds__(kThreads, 1) step_nco_f32_kernel(const StepArg
             float v[Q], m[Q];
 #pragma unroll
             for (int e = 0; e < Q; ++e) v[e] = sh.df[0][e][lane];
-            const float drho = moments_from_dev(v, m);
+            moments_from_dev(v, m);
             if (cell_of(0) < a.d.ncell && !(m[0] >= a.rho_min && m[0] <= a.rho_max)) atomicOr(a.status, 1);
 #pragma unroll
             for (int e = 0; e < Q; ++e) sh.m[0][lane][e] = m[e];
-            sh.m[0][lane][Q] = drho;
         }
     } else {
         if (w == kLoader) load_tile<STORAGE, BC>(a, cell_of(0), sh.m[0], sh.df[0], lane);
@@ -121,7 +128,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_nco_f32_kernel(const StepArg
     __syncthreads();
 
     long long pacc[3] = {0, 0, 0};  // forced steps: fixed-point projection sums of the finisher's lane
-    int b = 0;                      // i modulo 3: buffers of tile i; (b + 1) of tile i + 1, (b + 2) of tile i - 1
+    int b = 0;                      // i modulo 3: df of tile i; (b + 1) of tile i + 1, (b + 2) of tile i - 1
     for (int i = 0; i <= n; ++i) {
         const int bn = b == 2 ? 0 : b + 1, bp = b == 0 ? 2 : b - 1;
         if (w < kNetWarps) {
@@ -133,8 +140,8 @@ __global__ void __launch_bounds__(kThreads, 1) step_nco_f32_kernel(const StepArg
                     for (int k = 0; k < 2; ++k)
 #pragma unroll
                         for (int e = 0; e < 28; e += 4)
-                            *reinterpret_cast<float4*>(&m[k][e]) = *reinterpret_cast<const float4*>(&sh.m[b][l + 16 * k][e]);
-                    first_layer<1>(net, p, half, lane, m, sh.rows[2 * p]);
+                            *reinterpret_cast<float4*>(&m[k][e]) = *reinterpret_cast<const float4*>(&sh.m[i & 1][l + 16 * k][e]);
+                    first_layer<ByCells>(net, p, half, lane, m, sh.rows[2 * p]);
                 }
                 pair_sync(p);
                 float* const row = sh.rows[w] + l * net_row(4);
@@ -148,41 +155,46 @@ __global__ void __launch_bounds__(kThreads, 1) step_nco_f32_kernel(const StepArg
                     set_bias(net.bd, lane, acc);
                     mat_vec<4, 1>(net.Wd, lane, acc, RowColumns<4>{row});
                 }
-                // the sums of the two halves, the first warp's then the second's on top
-                float* const out = &sh.part[i & 1][p][l][(lane >> 4) * kHalf];
-                if (half) pair_sync(p);
+                // the group sum, element by element in the order of the group: the eight sign vectors of
+                // this permutation on top of the permutations before it
+                float* const out = &sh.part[i & 1][16 * half + l][(lane >> 4) * kHalf];
+                float h[kHalf];
+                if (p > 0) {
+                    group_sum_wait(p);
+#pragma unroll
+                    for (int o = 0; o < kHalf; o += 2) {
+                        const float2 t = *reinterpret_cast<const float2*>(out + o);
+                        h[o] = t.x;
+                        h[o + 1] = t.y;
+                    }
+                } else {
+#pragma unroll
+                    for (int o = 0; o < kHalf; ++o) h[o] = 0.0f;
+                }
 #pragma unroll
                 for (int r = 0; r < 2; ++r)
 #pragma unroll
-                    for (int o = 0; o < kHalf; o += 2) {
-                        float2* const dst = reinterpret_cast<float2*>(out + 16 * r * kHidden + o);
-                        float2 h = half ? *dst : make_float2(0.0f, 0.0f);
-                        h.x += (fmaxf(acc[r][0][o], 0.0f) + fmaxf(acc[r][1][o], 0.0f)) +
-                               (fmaxf(acc[r][2][o], 0.0f) + fmaxf(acc[r][3][o], 0.0f));
-                        h.y += (fmaxf(acc[r][0][o + 1], 0.0f) + fmaxf(acc[r][1][o + 1], 0.0f)) +
-                               (fmaxf(acc[r][2][o + 1], 0.0f) + fmaxf(acc[r][3][o + 1], 0.0f));
-                        *dst = h;
-                    }
-                if (!half) pair_arrive(p);
+                    for (int c = 0; c < 4; ++c)
+#pragma unroll
+                        for (int o = 0; o < kHalf; ++o) h[o] += fmaxf(acc[r][c][o], 0.0f);
+#pragma unroll
+                for (int o = 0; o < kHalf; o += 2) *reinterpret_cast<float2*>(out + o) = make_float2(h[o], h[o + 1]);
+                if (p + 1 < kNetWarps / 2) group_sum_pass(p + 1);
             }
         } else if (w == kLoader) {
-            if (i + 1 < n) load_tile<STORAGE, BC>(a, cell_of(i + 1), sh.m[bn], sh.df[bn], lane);
+            if (i + 1 < n) load_tile<STORAGE, BC>(a, cell_of(i + 1), sh.m[(i + 1) & 1], sh.df[bn], lane);
         } else if (i >= 1) {
             const long long cell = cell_of(i - 1);
             const bool valid = cell < a.d.ncell;
             float h[kHidden];
 #pragma unroll
-            for (int j = 0; j < kHidden; ++j) h[j] = 0.0f;
-#pragma unroll 2
-            for (int q = 0; q < kNetWarps / 2; ++q)
-#pragma unroll
-                for (int j = 0; j < kHidden; j += 4) {
-                    const float4 v = *reinterpret_cast<const float4*>(&sh.part[(i - 1) & 1][q][lane][j]);
-                    h[j] += v.x;
-                    h[j + 1] += v.y;
-                    h[j + 2] += v.z;
-                    h[j + 3] += v.w;
-                }
+            for (int j = 0; j < kHidden; j += 4) {
+                const float4 v = *reinterpret_cast<const float4*>(&sh.part[(i - 1) & 1][lane][j]);
+                h[j] = v.x;
+                h[j + 1] = v.y;
+                h[j + 2] = v.z;
+                h[j + 3] = v.w;
+            }
             float rates[kOut];
 #pragma unroll
             for (int o = 0; o < kOut; ++o) {
@@ -193,11 +205,11 @@ __global__ void __launch_bounds__(kThreads, 1) step_nco_f32_kernel(const StepArg
             }
             float df[Q], m[Q];
 #pragma unroll
-            for (int e = 0; e < Q; ++e) {
-                df[e] = sh.df[bp][e][lane];
-                m[e] = sh.m[bp][lane][e];
-            }
-            Macro q = macro_from_moments(m, sh.m[bp][lane][Q]);
+            for (int e = 0; e < Q; ++e) df[e] = sh.df[bp][e][lane];
+            // the moments once more, not read back: the compiler then contracts their last products into the
+            // relaxation as it does for one thread per cell
+            const float drho = moments_from_dev(df, m);
+            Macro q = macro_from_moments(m, drho);
             collide_mrt(df, m, q, 1.0f / a.tau, rates);
             if constexpr (FORCED) {  // every lane takes part in the projection, cells past the end with u = 0
                 int x = 0, y = 0, z = 0;

@@ -260,7 +260,7 @@ void make_net_params(const float* theta, bool deep, NetParams* out) {
     for (int p = 0; p < 6; ++p) {
         const int gp = p * 8;  // element with axis permutation p and no reflection
         for (int j = 0; j < kHidden; ++j) {
-            for (int k = 0; k < Q; ++k) out->W1p[p][j][g.mperm_t[gp][kPrinted.e[k]]] = W1[j * Q + k];
+            for (int k = 0; k < Q; ++k) out->W1p[p][j][class_pos(g.mperm_t[gp][kPrinted.e[k]])] = W1[j * Q + k];
             out->W1p[p][j][Q] = b1[j];
         }
     }

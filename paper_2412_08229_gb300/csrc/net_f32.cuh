@@ -9,11 +9,10 @@
 // 8-point Walsh-Hadamard transform of the 8 class sums y_c = sum_{t in class c} W1p[:, t] m_t:
 // 20 x 27 MAC and 20 x 24 additions per permutation instead of 8 x 20 x 27 MAC.
 //
-// Warp (p, half) evaluates the sign vectors [4 half, 4 half + 4) of permutation p. Its 32 rows
-// of shared memory hold the columns' hidden layer: a tile of 32 cells has a row per cell with
-// the four columns of the half's sign vectors (LANES = 1), a tile of 16 cells two rows per
-// cell, r and r + 16, with two columns each (LANES = 2; row r + 16 has the sign vectors with
-// bit 1 set).
+// Warps (p, 0) and (p, 1) evaluate permutation p. Which columns (cell, sign vector) each of them
+// has in its 32 rows of shared memory is one of the placements below: by halves of the sign
+// vectors (the adjoint) or by halves of the cells (the step, whose group sum runs over the sign
+// vectors of a cell in their order).
 //
 // What bounds it, and the layout: FP32 FMAs need their operands from shared memory at 16 bytes
 // a lane per four cycles and SM, the time of four FMAs per lane on each scheduler; weights
@@ -27,17 +26,13 @@
 
 namespace lbm {
 
-constexpr int kNetWarps = 12;       // (axis permutation, half of its sign vectors)
+constexpr int kNetWarps = 12;       // two per axis permutation
 constexpr int kHalf = kHidden / 2;  // hidden units of the first layer per warp
 
 // Floats of a lane's row for C columns, a multiple of 4 whose quarter is odd: the 16-byte
 // accesses of eight lanes to their own rows fall in different banks.
 constexpr int net_row(int C) { return C * kHidden + 4; }
 static_assert(net_row(4) / 4 % 2 == 1 && net_row(2) / 4 % 2 == 1, "bank-conflict-free rows");
-
-__host__ __device__ constexpr int odd_mask(int t) {
-    return ((ex_of(t) == 1) << 2) | ((ey_of(t) == 1) << 1) | (ez_of(t) == 1);
-}
 
 // Floats of a warp's 32 rows: the sixteen at the end shift the second warp of a permutation by
 // half the banks, so that the eight classes of a cell are read without conflicts.
@@ -60,15 +55,25 @@ __device__ __forceinline__ void wht(float* y) {
 
 __device__ __forceinline__ void pair_sync(int p) { asm volatile("bar.sync %0, 64;" ::"r"(p + 1) : "memory"); }
 
-__device__ __forceinline__ void pair_arrive(int p) { asm volatile("bar.arrive %0, 64;" ::"r"(p + 1) : "memory"); }
-
-// Place of sign vector (or parity class) s of a cell: which of the two warps of the
-// permutation, how many rows after the cell's, and which column.
+// Place of sign vector (or parity class) s of cell l + 16 k, l = lane % 16: which of the two warps
+// of the permutation, how many rows after l, and which of the row's kCols columns.
+// By sign vectors: warp (p, half) has [4 half, 4 half + 4) of every cell; a tile of 32 cells has
+// a row per cell (LANES = 1), one of 16 cells two rows of two columns (LANES = 2; the second row
+// has the sign vectors with bit 1 set).
 template <int LANES>
-struct ColumnOf {
-    static __host__ __device__ constexpr int half(int s) { return s >> 2; }
-    static __host__ __device__ constexpr int row(int s) { return LANES == 1 ? 0 : 16 * ((s >> 1) & 1); }
-    static __host__ __device__ constexpr int col(int s) { return LANES == 1 ? s & 3 : s & 1; }
+struct BySigns {
+    static constexpr int kCells = 2 / LANES, kCols = 4 / LANES;  // cells per lane, columns per row
+    static __host__ __device__ constexpr int half(int s, int) { return s >> 2; }
+    static __host__ __device__ constexpr int row(int s, int k) { return LANES == 1 ? 16 * k : 16 * ((s >> 1) & 1); }
+    static __host__ __device__ constexpr int col(int s, int) { return LANES == 1 ? s & 3 : s & 1; }
+};
+// By cells: warp (p, half) has all eight of the cells [16 half, 16 half + 16), the first four in
+// row l and the others in row l + 16.
+struct ByCells {
+    static constexpr int kCells = 2, kCols = 4;
+    static __host__ __device__ constexpr int half(int, int k) { return k; }
+    static __host__ __device__ constexpr int row(int s, int) { return 16 * (s >> 2); }
+    static __host__ __device__ constexpr int col(int s, int) { return s & 3; }
 };
 
 // The block's copy of the parameters (the caller syncs).
@@ -78,13 +83,13 @@ __device__ __forceinline__ void load_params(NetParams* dst, const NetParams* __r
 }
 
 // relu(W1p x^(s) + b1) for the eight sign vectors s of permutation p, into the rows of its two
-// warps (rows: the first warp's; those of the second follow net_rows floats later). Of the warp's ten
-// units a lane takes five, for the cells l = lane % 16 (and l + 16, LANES = 1); m[k] are the
-// moments of its cells in tensor order.
-template <int LANES>
+// warps (rows: the first warp's; those of the second follow net_rows floats later) as At places
+// them. Of the warp's ten units a lane takes five, for the cells l = lane % 16 (and l + 16); m[k]
+// are the moments of its cells in tensor order.
+template <typename At>
 __device__ __forceinline__ void first_layer(const NetParams& net, int p, int half, int lane, const float (*m)[28],
                                             float* rows) {
-    constexpr int NC = 2 / LANES, C = 4 / LANES, R = net_row(C);
+    constexpr int NC = At::kCells, C = At::kCols, R = net_row(C);
     const int j0 = half * kHalf + (lane >> 4) * 5;
     float* const out = rows + (lane & 15) * R + j0;
 #pragma unroll
@@ -97,13 +102,14 @@ __device__ __forceinline__ void first_layer(const NetParams& net, int p, int hal
             float y[8];
 #pragma unroll
             for (int c = 0; c < 8; ++c) y[c] = 0.0f;
-#pragma unroll
-            for (int t = 0; t < Q; ++t) y[odd_mask(t)] = fmaf(w[t], m[k][t], y[odd_mask(t)]);
+            static_for<Q>([&](auto T) {
+                constexpr int t = decltype(T)::value, c = odd_mask(t), q = class_pos(t);
+                y[c] = fmaf(w[q], m[k][t], y[c]);
+            });
             wht<8>(y);
-            using At = ColumnOf<LANES>;
 #pragma unroll
             for (int s = 0; s < 8; ++s)
-                out[At::half(s) * net_rows(C) + (At::row(s) + 16 * k) * R + At::col(s) * kHidden + i] = fmaxf(y[s] + w[Q], 0.0f);
+                out[At::half(s, k) * net_rows(C) + At::row(s, k) * R + At::col(s, k) * kHidden + i] = fmaxf(y[s] + w[Q], 0.0f);
         }
     }
 }
