@@ -13,23 +13,27 @@
 
 namespace lbm {
 
+// Stored populations. Plain loads, not the non-coherent path of __ldg: that one promises data
+// that nobody writes while the kernel runs, but a kernel launched with overlap (launch.cuh) is
+// resident while its predecessor still writes the buffer, and the compiler may move a
+// non-coherent load up across overlap_wait().
 template <int STORAGE> struct Store;
 template <> struct Store<LBM_STORE_F32> {
     using T = float;
     static __device__ __forceinline__ float cvt(T v) { return v; }
-    static __device__ __forceinline__ float ld(const T* p) { return __ldg(p); }
+    static __device__ __forceinline__ float ld(const T* p) { return *p; }
     static __device__ __forceinline__ void st(T* p, float v) { *p = v; }
 };
 template <> struct Store<LBM_STORE_F16_DEV> {
     using T = __half;
     static __device__ __forceinline__ float cvt(T v) { return __half2float(v); }
-    static __device__ __forceinline__ float ld(const T* p) { return cvt(__ldg(p)); }
+    static __device__ __forceinline__ float ld(const T* p) { return cvt(*p); }
     static __device__ __forceinline__ void st(T* p, float v) { *p = __float2half_rn(v); }
 };
 template <> struct Store<LBM_STORE_BF16_DEV> {
     using T = __nv_bfloat16;
     static __device__ __forceinline__ float cvt(T v) { return __bfloat162float(v); }
-    static __device__ __forceinline__ float ld(const T* p) { return cvt(__ldg(p)); }
+    static __device__ __forceinline__ float ld(const T* p) { return cvt(*p); }
     static __device__ __forceinline__ void st(T* p, float v) { *p = __float2bfloat16_rn(v); }
 };
 

@@ -3,8 +3,10 @@
 // A kernel launched with `overlap` on a stream (or captured into a graph) right behind
 // another starts as soon as every block of that one has begun, and waits in overlap_wait()
 // for its results; nothing that an earlier kernel writes may be read, and nothing that it
-// reads may be written, before that. The wait covers all launches before, because the
-// launch waited for has itself waited for its own predecessor.
+// reads may be written, before that. What an earlier kernel writes is read by plain loads:
+// the compiler and the caches may take a __ldg as good at any time of the kernel's life. The
+// wait covers all launches before, because the launch waited for has itself waited for its own
+// predecessor.
 #pragma once
 
 #include <cuda_runtime.h>
