@@ -24,10 +24,12 @@
 // pair); tensor pipe 44 % (five N 48 MMAs of 24.5 cycles per pair and tile), FMA pipe 44 %,
 // DRAM 6 %. The 256^3 mixed step takes 2.97 ms, 3.36 ms with two tiles of two warpgroups per SM
 // that both converted and summed, waiting for each pair's layer 2 before the next (325 cycles per
-// pair and SM, here 275). What each part brought, 256^3, from 3.36 ms: relu on the FMA pipe, 32-bit
-// offsets and A2 in place with three chains 3.27; converters and summers apart 3.16; an issuer
-// warp 3.11; named barriers instead of polls 3.05; D2 read whole before the sum and layer 1 two
-// pairs ahead 2.97.
+// pair and SM, here 275). What each part brought, 256^3, from 3.36 ms, each with relu as
+// (b + |b|) / 2: 32-bit offsets and A2 in place with three chains 3.27; converters and summers
+// apart 3.16; an issuer warp 3.11; named barriers instead of polls 3.05; D2 read whole before the
+// sum and layer 1 two pairs ahead 2.97. That relu runs on the FMA pipe where max runs on the ALU
+// pipe at half the rate, but turns minus infinity into NaN and overflows above half of the largest
+// float: with max, as everywhere else, four steps and the read-back take 13.37 instead of 13.05 ms.
 //
 // Hand-overs, per chain (n = 0..23 of a tile, b = n & 1):
 //   a1full            A1 of the tile written (4 converter warps)      -> issuer: layer 1 of pairs 0, 1
@@ -360,7 +362,7 @@ __global__ void __launch_bounds__(kThreads, 1) nco_tcp_kernel(const __grid_const
         const float* b3 = reinterpret_cast<const float*>(smem + kB3Off);
         mbar_arrive_lane0(&bars[kD2Free], lane_id);  // D2 is free
         for (int it = 0; gtile < ntiles; gtile += stride, ++it) {
-            // 2 relu(h) summed over the even and over the odd pairs
+            // relu(h) summed over the even and over the odd pairs
             float acc[2][kHidden];
 #pragma unroll
             for (int j = 0; j < kHidden; ++j) acc[0][j] = acc[1][j] = 0.0f;
@@ -380,8 +382,8 @@ __global__ void __launch_bounds__(kThreads, 1) nco_tcp_kernel(const __grid_const
                     mbar_arrive_lane0(&bars[kD2Free], lane_id);  // before the sum: layer 2 of the next pair waits for it
 #pragma unroll
                     for (int j = 0; j < kHidden; j += 2) {
-                        add2_relu2(acc[b][j], acc[b][j + 1], as_f(v[j]), as_f(v[j + 1]));
-                        add2_relu2(acc[b][j], acc[b][j + 1], as_f(v[kHidden + j]), as_f(v[kHidden + j + 1]));
+                        add2_relu(acc[b][j], acc[b][j + 1], as_f(v[j]), as_f(v[j + 1]));
+                        add2_relu(acc[b][j], acc[b][j + 1], as_f(v[kHidden + j]), as_f(v[kHidden + j + 1]));
                     }
                 }
             }
@@ -407,7 +409,7 @@ __global__ void __launch_bounds__(kThreads, 1) nco_tcp_kernel(const __grid_const
                         t = fmaf(w.z, acc[0][j + 2], t);
                         t = fmaf(w.w, acc[0][j + 3], t);
                     }
-                    rates[k] = rate_from_output(t * (0.5f / 48.0f) + b3[k]);
+                    rates[k] = rate_from_output(t * (1.0f / 48.0f) + b3[k]);
                 }
                 float F[3];
                 if (FORCED) {  // F(x) from this step's coefficients

@@ -92,17 +92,5 @@ __device__ __forceinline__ void add2_relu(float& a0, float& a1, float b0, float 
         : "f"(b0), "f"(b1));
 }
 
-// (a0, a1) += 2 (relu(b0), relu(b1)): 2 relu(b) = b + |b| exactly, which runs on the FMA pipe
-// (one cycle per warp instruction) where max runs on the ALU pipe (two). A sum of doubled
-// terms is the doubled sum, bit for bit.
-__device__ __forceinline__ void add2_relu2(float& a0, float& a1, float b0, float b1) {
-    b0 = b0 + fabsf(b0);
-    b1 = b1 + fabsf(b1);
-    asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%0, %1};\n\tmov.b64 y, {%2, %3};\n\t"
-        "add.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
-        : "+f"(a0), "+f"(a1)
-        : "f"(b0), "f"(b1));
-}
-
 }  // namespace tcc
 }  // namespace lbm
