@@ -62,12 +62,13 @@ struct lbm_ctx {
     int adj_grad_len = 0;
     long long wait_cycles = kDefaultWaitCycles;  // limit of the tensor-core kernels' MMA waits
     int tc_shape = 0;  // tile shape of the BF16 tensor-core network (a batch's autotuned choice)
-    // one step per buffer parity captured in CUDA graphs (lbm_step with nsteps >= 2, not
-    // recording): captured on a private stream, launched on `stream`; a forced step reads its
-    // row of draws at graph_head + *d_counter
+    // one step per buffer parity and kChunkSteps steps from it, captured in CUDA graphs when first
+    // used (lbm_step with nsteps >= 2, not recording): captured on a private stream, launched on
+    // `stream`; a forced step reads its row of draws at graph_head + *d_counter
     cudaStream_t gstream = nullptr;
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
-    cudaGraphExec_t chunk[2] = {nullptr, nullptr};  // kChunkSteps steps from parity 0 / 1, captured when first used
+    cudaGraphExec_t chunk[2] = {nullptr, nullptr};
+    long long chunk_due[2] = {0, 0};  // chunks that could have been replayed while there was none
     long long* d_counter = nullptr;
     long long graph_head = 0;
     const double* graph_draws = nullptr;
@@ -81,6 +82,7 @@ static void drop_step_graphs(lbm_ctx* c) {
             cudaGraphExecDestroy(*g);
             *g = nullptr;
         }
+    c->chunk_due[0] = c->chunk_due[1] = 0;
 }
 
 // Makes a context's device current for the duration of an entry point and restores the
@@ -635,8 +637,9 @@ lbm_status nco_set_weights(lbm_ctx* c, const float* theta, int n) {
         c->net = new (std::nothrow) NetParams();
         if (!c->net) return fail(c, LBM_ERR_OOM, "nco_set_weights: host allocation failed");
     }
+    // the captured steps read the weights from net_w and are those of the old network's depth
+    if ((c->net->deep != 0) != deep) drop_step_graphs(c);
     make_net_params(h.data(), deep, c->net);
-    drop_step_graphs(c);  // the captured steps are those of the old network's depth
     if (c->net_w && c->cfg.net_precision == LBM_NET_F32) {
         LBM_CK(c, cudaMemcpyAsync(c->net_w, c->net, sizeof(NetParams), cudaMemcpyHostToDevice, c->stream));
         LBM_CK(c, cudaStreamSynchronize(c->stream));
@@ -760,12 +763,25 @@ static lbm_status enqueue_step(lbm_ctx* c, int p, cudaStream_t s, const double* 
     return LBM_OK;
 }
 
-// Steps of a chunk graph (even: the buffer parity comes back), and the largest grid stepped by
-// chunks. A graph launch per step costs 4.2 us between starts, more than a small grid's step
-// takes; inside a chunk the kernels follow each other without the host and with their starts
-// overlapped (16^3 BGK: 4.2 -> 2.05 us a step, forced 64^3 BGK 27.0 -> 24.9). From 128^3 on a step takes 60 us and more.
+// Steps of a chunk graph (even: the buffer parity comes back). A graph launch per step costs
+// 4.2 us between starts, more than a small grid's step takes; inside a chunk the kernels follow
+// each other without the host and, but for the tensor-core ones, with their starts overlapped
+// (16^3 BGK: 4.2 -> 2.05 us a step, forced 64^3 BGK 27.0 -> 24.9).
 constexpr int kChunkSteps = 16;
-constexpr long long kChunkCells = 128LL * 128 * 128;
+
+// The largest grid stepped by chunks, which save 2 to 3 us a step: where a step takes about half
+// a millisecond, the plain operators' 128^3 apart (60 us; 2^18 cells with the FP32 network 360 us,
+// 2^20 with the split one 550, 2^21 with the BF16 one 380; the third hidden layer takes nearly
+// twice as long).
+static long long chunk_cells(const lbm_ctx* c) {
+    if (c->cfg.op != LBM_OP_NCO) return 1LL << 21;
+    const int log2 = c->cfg.net_precision == LBM_NET_F32 ? 18 : c->cfg.net_precision == LBM_NET_BF16X3 ? 20 : 21;
+    return 1LL << (c->net && c->net->deep ? log2 - 1 : log2);
+}
+
+// Capturing costs 45 us (a forced step is two launches: 95), a replay saves 30 to 50: from this
+// many replays on, counted over the calls, a chunk pays for itself.
+static long long chunk_pays(bool forced) { return forced ? 3 : 2; }
 
 // `count` steps from buffer parity p as a graph.
 static lbm_status capture_steps(lbm_ctx* c, int p, int count, cudaGraphExec_t* out) {
@@ -785,21 +801,18 @@ static lbm_status capture_steps(lbm_ctx* c, int p, int count, cudaGraphExec_t* o
     return LBM_OK;
 }
 
-// Capture one step per buffer parity unless the graphs in hand still fit (a forced step's
+// Makes ready for captures and drops the graphs in hand if they no longer fit (a forced step's
 // graph depends on the draw queue it reads).
-static lbm_status ensure_step_graphs(lbm_ctx* c) {
+static lbm_status ready_step_graphs(lbm_ctx* c) {
     const bool forced = c->cfg.forcing == 1;
-    if (c->graph[0] && (!forced || (c->graph_draws == c->d_draws && c->graph_cap == c->draws_cap))) return LBM_OK;
-    drop_step_graphs(c);
     if (!c->gstream) LBM_CK(c, cudaStreamCreateWithFlags(&c->gstream, cudaStreamNonBlocking));
-    if (forced && !c->d_counter) LBM_CK(c, cudaMalloc(reinterpret_cast<void**>(&c->d_counter), sizeof(long long)));
+    if (!forced) return LBM_OK;
+    if (!c->d_counter) LBM_CK(c, cudaMalloc(reinterpret_cast<void**>(&c->d_counter), sizeof(long long)));
+    if (c->graph_draws == c->d_draws && c->graph_cap == c->draws_cap) return LBM_OK;
+    drop_step_graphs(c);
     c->graph_head = c->draws_head;
     c->graph_draws = c->d_draws;
     c->graph_cap = c->draws_cap;
-    for (int p = 0; p < 2; ++p) {
-        const lbm_status st = capture_steps(c, p, 1, &c->graph[p]);
-        if (st) return st;
-    }
     return LBM_OK;
 }
 
@@ -816,21 +829,26 @@ lbm_status lbm_step(lbm_ctx* c, int nsteps) {
     const bool graphs = nsteps >= 2 && c->rec_k == 0;
     for (int k = 0; k < nsteps; ++k) {
         if (graphs && k == 1) {
-            lbm_status st = ensure_step_graphs(c);
+            lbm_status st = ready_step_graphs(c);
             if (st) return st;
             if (forced) LBM_CK(c, launch_counter_set(c->d_counter, c->draws_head - c->graph_head, c->stream));
-            if (c->d.ncell <= kChunkCells && nsteps - k >= kChunkSteps) {
-                if (!c->chunk[c->cur]) {
+            const int chunks = (nsteps - k) / kChunkSteps;
+            if (chunks > 0 && c->d.ncell <= chunk_cells(c)) {
+                if (!c->chunk[c->cur] && (c->chunk_due[c->cur] += chunks) >= chunk_pays(forced)) {
                     st = capture_steps(c, c->cur, kChunkSteps, &c->chunk[c->cur]);
                     if (st) return st;
                 }
-                for (; nsteps - k >= kChunkSteps; k += kChunkSteps) {
+                for (; c->chunk[c->cur] && nsteps - k >= kChunkSteps; k += kChunkSteps) {
                     LBM_CK(c, cudaGraphLaunch(c->chunk[c->cur], c->stream));
                     c->t += kChunkSteps;
                     if (forced) c->draws_head += kChunkSteps;
                 }
             }
             for (; k < nsteps; ++k) {
+                if (!c->graph[c->cur]) {
+                    st = capture_steps(c, c->cur, 1, &c->graph[c->cur]);
+                    if (st) return st;
+                }
                 LBM_CK(c, cudaGraphLaunch(c->graph[c->cur], c->stream));
                 c->cur = 1 - c->cur;
                 ++c->t;
