@@ -12,6 +12,9 @@ pull-stream-collide kernel over the whole grid. Forms:
 The state (1.8 GB FP32, 0.9 GB FP16) is far larger than the 129 MB L2, so no flush is
 needed between steps.
 
+The result is one JSON line on stdout, short enough (3 KB) to be kept whole by whoever keeps the
+end of a log; the same with every figure and the extra workloads goes to stderr before it.
+
 `--impl reference` times the FP64 CPU oracle (the only reference this method has) on
 the machine's host cores, on a bounded slab sample of the same workload.
 """
@@ -950,6 +953,32 @@ def oracle_grid_timings():
     return out
 
 
+def headline(line):
+    """`line` without the extras and the long notes: the keys of the bench contract."""
+    def short(x):
+        if isinstance(x, dict):
+            return {k: short(v) for k, v in x.items()}
+        if isinstance(x, (list, tuple)):
+            return [short(v) for v in x]
+        return float(f"{x:.9g}") if isinstance(x, float) else x
+
+    def without(x, *names):
+        return {k: v for k, v in x.items() if k not in names} if isinstance(x, dict) else x
+
+    keys = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "config", "roofline", "cpu_baseline", "e2e", "gpu_launches", "clocks")
+    out = {k: line[k] for k in keys}
+    roof = without(line["roofline"], "traffic_source", "peak_source")
+    if "hbm" in roof:
+        roof["hbm"] = without(roof["hbm"], "peak_source")
+    out["roofline"] = roof
+    out["cpu_baseline"] = without(line["cpu_baseline"], "mlups_by_grid_and_threads")
+    out["e2e"] = without(line["e2e"], "note", "repetitions_s")
+    out["forms"] = {f: {k: v for k, v in r.items() if k in ("mlups", "ms_per_step", "unavailable")}
+                    for f, r in line["forms"].items()}
+    return {k: v if k in ("value", "ms_per_step") else short(v) for k, v in out.items()}
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -1098,7 +1127,8 @@ def main():
         "roofline": roof, "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": args.steps,
         "clocks": clocks, "forms": forms, **extras,
     }
-    print(json.dumps(line), flush=True)
+    print(json.dumps(line), file=sys.stderr, flush=True)
+    print(json.dumps(headline(line)), flush=True)
 
 
 if __name__ == "__main__":
