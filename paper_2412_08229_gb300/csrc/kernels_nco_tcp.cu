@@ -213,7 +213,10 @@ __global__ void __launch_bounds__(kThreads, 1) nco_tcp_kernel(const __grid_const
             };
             for (int it = 0; gtile < ntiles; gtile += stride, ++it) {
                 poll_warps(&bars[kA1Full], static_cast<uint32_t>(it) & 1u);
-                if (it == 0) wait(bar_w, 0, kDefaultWaitCycles);  // the weights have arrived
+                if (it == 0 && !mbar_try_wait(bar_w, 0) && !wait_phase(bar_w, 0, kDefaultWaitCycles)) {
+                    ok = false;  // the weights have not arrived: waits for them once more before the block ends
+                    *abort_flag = 1;
+                }
                 if (elect_one()) {
                     issue_l1(0, 0);
                     issue_l1(1, 1);
