@@ -234,8 +234,8 @@ __device__ __forceinline__ void group_sum_wait(int w) { asm volatile("bar.sync %
 __device__ __forceinline__ void group_sum_pass(int w) { asm volatile("bar.arrive %0, 64;" ::"r"(group_sum_barrier(w)) : "memory"); }
 
 template <int STORAGE, int BC, bool DEEP, int LANES>
-__global__ void __launch_bounds__(kAdjThreads, (!DEEP && LANES == 2) ? 2 : 1)
-    adjoint_step_kernel(const AdjArgs a, const NetParams* __restrict__ net_in, int ntiles) {
+__global__ void __launch_bounds__(kAdjThreads, 1) adjoint_step_kernel(const AdjArgs a,
+                                                                      const NetParams* __restrict__ net_in, int ntiles) {
     using GL = GradLayout<DEEP>;
     using SH = AdjShared<DEEP, LANES>;
     using At = BySigns<LANES>;
