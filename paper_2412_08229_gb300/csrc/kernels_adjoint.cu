@@ -26,9 +26,9 @@
 //
 // lam's arithmetic is that of one thread per cell, bit for bit: the group sum in the order of the
 // group (handed from warp to warp), the cotangent of m as the relaxation's part plus 120 products
-// one after the other. A sweep of 200 steps turns other roundings into up to 3e-5 of the
-// gradient. Sums that end in the gradient are grouped freely. (The two sums in order: 32^3
-// training pass 61.1 -> 64.9 ms.)
+// one after the other, on small grids in 2, 3 or 6 parts. A sweep of 200 steps turns other
+// roundings into up to 3e-5 of the gradient. Sums that end in the gradient are grouped freely.
+// (The two sums in order: 32^3 training pass 61.1 -> 63.6 ms.)
 //
 // A block per SM walks over the tiles and keeps the parameter gradients in FP64 in shared
 // memory, so the global atomics come once per block (a block per tile: 32^3 225 us).
@@ -121,13 +121,15 @@ struct AdjArgs {
     double* grad;        // GradLayout<DEEP>::kLen accumulators
     float tau;
     const float* force;  // forced step: the force field of step t (3 planes), else null
+    int parts;           // SPLIT: parts of the cotangent of m, the axis permutations in 2, 3 or 6 groups
 };
 
 constexpr int kAdjThreads = 32 * kNetWarps;
 constexpr int kGradBlock = kHidden * kHidden + kHidden;  // dW and db of a 20 x 20 layer
 
-// LANES lanes share a cell, each holding COLS of the half's four sign vectors.
-template <bool DEEP, int LANES>
+// LANES lanes share a cell, each holding COLS of the half's four sign vectors. SPLIT: the
+// cotangent of m in parts.
+template <bool DEEP, int LANES, bool SPLIT>
 struct AdjShared {
     static constexpr int kCells = 32 / LANES;
     static constexpr int kCols = 4 / LANES;
@@ -149,6 +151,13 @@ struct AdjShared {
     float v3[kCells][kHidden];  // cotangent of the last hidden layer, the same for every group element
     float gbar[kCells][kOut];
     float rates[kCells][kOut];
+    // dL/dm of the second to sixth part (the deep network's h2 is free by then)
+    float more[SPLIT && !DEEP ? 5 : 1][SPLIT && !DEEP ? kCells : 1][28];
+    __device__ __forceinline__ float (*part(int i))[28] {
+        if (i == 0) return mu;
+        return reinterpret_cast<float(*)[28]>(DEEP ? &h2[0][0][0] : &more[0][0][0]) + (i - 1) * kCells;
+    }
+    static_assert(!DEEP || 5 * kCells * 28 <= kNetWarps * 32 * kRow, "the parts fit h2");
 };
 
 // A cell's 27 values to and from a row in class order.
@@ -233,11 +242,11 @@ __device__ __forceinline__ int group_sum_barrier(int w) { return w & 1 ? (w >> 1
 __device__ __forceinline__ void group_sum_wait(int w) { asm volatile("bar.sync %0, 64;" ::"r"(group_sum_barrier(w)) : "memory"); }
 __device__ __forceinline__ void group_sum_pass(int w) { asm volatile("bar.arrive %0, 64;" ::"r"(group_sum_barrier(w)) : "memory"); }
 
-template <int STORAGE, int BC, bool DEEP, int LANES>
+template <int STORAGE, int BC, bool DEEP, int LANES, bool SPLIT>
 __global__ void __launch_bounds__(kAdjThreads, 1) adjoint_step_kernel(const AdjArgs a,
                                                                       const NetParams* __restrict__ net_in, int ntiles) {
     using GL = GradLayout<DEEP>;
-    using SH = AdjShared<DEEP, LANES>;
+    using SH = AdjShared<DEEP, LANES, SPLIT>;
     using At = BySigns<LANES>;
     constexpr int kCells = SH::kCells, C = SH::kCols, kRow = SH::kRow;
     extern __shared__ __align__(16) uint8_t adj_smem_raw[];
@@ -612,17 +621,26 @@ __global__ void __launch_bounds__(kAdjThreads, 1) adjoint_step_kernel(const AdjA
             __syncthreads();
             // the network's part of the cotangent of m, W1p[j][t] E[c(t)][j] on top of the relaxation's
             // part, permutation by permutation and unit by unit (a sum whose last bits the sweep carries to
-            // the first step): a lane has a cell and four places of the class order. Warps 0 to 6 have 32
-            // cells each (LANES = 1), or 0 to 3 16 cells and two groups of places
+            // the first step), SPLIT in sums of 6 / a.parts permutations each: a lane has a cell and four
+            // places of the class order. Warps 0 to 6 have 32 cells each (LANES = 1), or 0 to 3 16 cells
+            // and two groups of places
             const int g = LANES == 1 ? w : 2 * w + og, cell = LANES == 1 ? lane : l;
             if (g < 7) {
                 const int ca = (kClassOfPair >> (8 * g)) & 7, cb = (kClassOfPair >> (8 * g + 4)) & 7;
                 auto e_of = [&](int k) { return sh.h1[At::half(k, 0)] + (At::row(k, 0) + cell) * kRow + At::col(k, 0) * kHidden; };
                 const float *ea = e_of(ca), *eb = e_of(cb);
-                float4* const q = reinterpret_cast<float4*>(&sh.mu[cell][4 * g]);
+                float4* q = reinterpret_cast<float4*>(&sh.mu[cell][4 * g]);
                 float4 dm = *q;
+                const int per = SPLIT ? 6 / a.parts : 6;
+                int left = per, part = 0;
 #pragma unroll 1
-                for (int pp = 0; pp < kNetWarps / 2; ++pp, ea += 2 * net_rows(C), eb += 2 * net_rows(C))
+                for (int pp = 0; pp < kNetWarps / 2; ++pp, ea += 2 * net_rows(C), eb += 2 * net_rows(C)) {
+                    if (SPLIT && left-- == 0) {  // the next part
+                        *q = dm;
+                        q = reinterpret_cast<float4*>(&sh.part(++part)[cell][4 * g]);
+                        dm = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                        left = per - 1;
+                    }
 #pragma unroll
                     for (int j = 0; j < kHidden; j += 4) {
                         const float4 a4 = *reinterpret_cast<const float4*>(ea + j);
@@ -639,6 +657,7 @@ __global__ void __launch_bounds__(kAdjThreads, 1) adjoint_step_kernel(const AdjA
                         add(j + 2, a4.z, b4.z);
                         add(j + 3, a4.w, b4.w);
                     }
+                }
                 *q = dm;
             }
         }
@@ -650,6 +669,16 @@ __global__ void __launch_bounds__(kAdjThreads, 1) adjoint_step_kernel(const AdjA
                 float v[Q];
                 load_class_order(v, sh.mu[lane]);
                 moments_transpose_inplace(v);
+                if constexpr (SPLIT) {
+#pragma unroll 1
+                    for (int i = 1; i < a.parts; ++i) {
+                        float more[Q];
+                        load_class_order(more, sh.part(i)[lane]);
+                        moments_transpose_inplace(more);
+#pragma unroll
+                        for (int e = 0; e < Q; ++e) v[e] += more[e];
+                    }
+                }
 #pragma unroll
                 for (int i = 0; i < Q; ++i) a.lam_out[static_cast<size_t>(i) * a.d.ncell + cell] = v[i];
             }
@@ -731,31 +760,40 @@ cudaError_t launch_adjoint_seed(const Dims& d, int storage, int bc, const void* 
     return cudaGetLastError();
 }
 
-template <int BC, bool DEEP, int LANES>
+template <int BC, bool DEEP, int LANES, bool SPLIT>
 static cudaError_t launch_adjoint_step_t(const AdjArgs& a, const NetParams* net, cudaStream_t s) {
-    using SH = AdjShared<DEEP, LANES>;
+    using SH = AdjShared<DEEP, LANES, SPLIT>;
     constexpr size_t smem = sizeof(SH);
     static_assert(smem <= 227 * 1024, "shared memory budget");
     static std::atomic<unsigned long long> attr{0};  // one set of per-device flags per instantiation
-    const cudaError_t e = ensure_dynamic_smem(adjoint_step_kernel<LBM_STORE_F32, BC, DEEP, LANES>,
-                                              static_cast<int>(smem), attr);
+    const auto kernel = adjoint_step_kernel<LBM_STORE_F32, BC, DEEP, LANES, SPLIT>;
+    const cudaError_t e = ensure_dynamic_smem(kernel, static_cast<int>(smem), attr);
     if (e != cudaSuccess) return e;
     const int ntiles = static_cast<int>((a.d.ncell + SH::kCells - 1) / SH::kCells);
     const int sms = sm_count();
-    return launch_kernel(adjoint_step_kernel<LBM_STORE_F32, BC, DEEP, LANES>, static_cast<unsigned>(ntiles < sms ? ntiles : sms),
-                         kAdjThreads, smem, s, true, a, net, ntiles);
+    return launch_kernel(kernel, static_cast<unsigned>(ntiles < sms ? ntiles : sms), kAdjThreads, smem, s, true, a, net,
+                         ntiles);
+}
+
+template <int BC, bool SPLIT>
+static cudaError_t launch_adjoint_step_d(const AdjArgs& a, bool deep, const NetParams* net, cudaStream_t s) {
+    return deep ? launch_adjoint_step_t<BC, true, 2, SPLIT>(a, net, s) : launch_adjoint_step_t<BC, false, 1, SPLIT>(a, net, s);
 }
 
 template <int BC>
 static cudaError_t launch_adjoint_step_bc(const AdjArgs& a, bool deep, const NetParams* net, cudaStream_t s) {
-    return deep ? launch_adjoint_step_t<BC, true, 2>(a, net, s) : launch_adjoint_step_t<BC, false, 1>(a, net, s);
+    return a.parts > 1 ? launch_adjoint_step_d<BC, true>(a, deep, net, s) : launch_adjoint_step_d<BC, false>(a, deep, net, s);
 }
 
 cudaError_t launch_adjoint_step(const Dims& d, int storage, int bc, const void* state, const float* lam_in,
                                 float* lam_out, double* grad, float tau, const float* force, bool deep,
                                 const NetParams* d_net, cudaStream_t s) {
     if (storage != LBM_STORE_F32) return cudaErrorInvalidValue;
-    const AdjArgs a{d, state, lam_in, lam_out, grad, tau, force};
+    // as many parts as one thread per cell took blocks of 128 cells for grids of fewer of them than
+    // SMs: the roundings, and with them the gradient of given inputs, stay the same at every size
+    const long long tiles = (d.ncell + 127) / 128, sms = sm_count();
+    const int parts = tiles >= sms ? 1 : tiles * 2 >= sms ? 2 : tiles * 3 >= sms ? 3 : 6;
+    const AdjArgs a{d, state, lam_in, lam_out, grad, tau, force, parts};
     switch (bc) {
         case LBM_BC_PERIODIC: return launch_adjoint_step_bc<LBM_BC_PERIODIC>(a, deep, d_net, s);
         case LBM_BC_MIRROR: return launch_adjoint_step_bc<LBM_BC_MIRROR>(a, deep, d_net, s);
