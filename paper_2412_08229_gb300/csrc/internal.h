@@ -133,8 +133,7 @@ struct FusedForce;  // the in-kernel forcing of a forced step (declared with the
 // net_weights: the context's weights in device memory, a NetParams for the FP32 network or
 // the packed operands of a tensor-core network; deep: a third hidden layer.
 // wait_cycles: limit of the main MMA-completion waits of the pair-pipelined and split
-// tensor-core kernels (kept out of StepArgs: a larger argument block made the CUDA-core
-// network kernel spill).
+// tensor-core kernels.
 // overlap: the BGK, KBC, REG and FP32-network kernels start while the launch before them ends (launch.cuh).
 // ff: the in-kernel forcing of a forced step (nullptr: unforced; a.force is then not read).
 cudaError_t launch_step(const StepArgs& a, const FusedForce* ff, int op, int storage, int bc, int net_prec,

@@ -34,8 +34,8 @@
 // memory, so the global atomics come once per block (a block per tile: 32^3 225 us).
 //
 // What bounds it (32^3, ncu): shared-memory latency and bandwidth between bursts of FMAs
-// (wavefronts 55 %, issue 47 %, three warps a scheduler). One step: 32^3 206 us, with the
-// third hidden layer 367 us, 16^3 36 and 59 us; before (one thread per cell, the forward
+// (wavefronts 50 %, issue 47 %, three warps a scheduler). One step: 32^3 213 us, with the
+// third hidden layer 382 us, 16^3 38 and 61 us; before (one thread per cell, the forward
 // computed twice, outer products by 40 of 128 threads): 723, 1137, 232 and 359 us.
 //
 // Observations of the kinetic energy k = (1/2)<|u|^2> at intermediate steps (the loss of

@@ -10,13 +10,14 @@
 //
 // The order of the group sum and of everything after it is that of one thread per cell, bit for
 // bit: a long unroll carries a last bit to 1e-5 of its gradient (handing the sum from one
-// permutation to the next costs 32^3 50.2 -> 52.9 us, 96^3 1185 -> 1264).
+// permutation to the next costs 32^3 50.2 -> 52.9 us, 96^3 1185 -> 1264, starts not overlapped).
 //
-// What bounds it (32^3, ncu): issue, 58 % of the cycles, in bursts: the twelve warps go through
-// their FMA and shared-memory phases nearly together; shared-memory wavefronts 48 %. Step of
-// the two-layer network with FP32 storage: 256^3 22.3 ms, 48^3 153 us, 32^3 49 us, 16^3
-// 10.4 us; with one thread per cell and the weights in the constant bank 26.1 ms, 183, 55 and
-// 46.9 us (16^3 fills 32 of 152 SMs that way, here 128). Third hidden layer: 16^3 15 us (70).
+// What bounds it (32^3, ncu): issue, 53 % of the cycles, in bursts: the twelve warps go through
+// their FMA and shared-memory phases nearly together and hand on the group sum one after the
+// other; shared-memory wavefronts 40 %. Step of the two-layer network with FP32 storage: 256^3
+// 23.8 ms, 48^3 163 us, 32^3 52 us, 16^3 10.8 us; with one thread per cell and the weights in the
+// constant bank 26.1 ms, 183, 55 and 47 us (16^3 fills 32 of 152 SMs that way, here 128). Third
+// hidden layer: 16^3 15.6 us (70).
 // The registers are at their limit of 128 (fourteen warps): the network's loop is sensitive to
 // what lives around it (the parameters copied before the first load instead of after: 8 % slower).
 #include "cell.cuh"

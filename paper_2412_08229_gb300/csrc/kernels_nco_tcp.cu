@@ -19,17 +19,17 @@
 // half-way through the walk; the moments reach the summers through shared memory,
 // double-buffered.
 //
-// What bounds it (128^3, mixed form, ncu): instruction issue, 71 % of the cycles with 197
-// instructions per pair of elements and warp, then the chain's own latency (~840 cycles per
-// pair); tensor pipe 44 % (five N 48 MMAs of 24.5 cycles per pair and tile), FMA pipe 44 %,
-// DRAM 6 %. The 256^3 mixed step takes 2.97 ms, 3.36 ms with two tiles of two warpgroups per SM
-// that both converted and summed, waiting for each pair's layer 2 before the next (325 cycles per
-// pair and SM, here 275). What each part brought, 256^3, from 3.36 ms, each with relu as
-// (b + |b|) / 2: 32-bit offsets and A2 in place with three chains 3.27; converters and summers
-// apart 3.16; an issuer warp 3.11; named barriers instead of polls 3.05; D2 read whole before the
-// sum and layer 1 two pairs ahead 2.97. That relu runs on the FMA pipe where max runs on the ALU
-// pipe at half the rate, but turns minus infinity into NaN and overflows above half of the largest
-// float: with max, as everywhere else, four steps and the read-back take 13.37 instead of 13.05 ms.
+// What bounds it (160^3, mixed form, ncu): instruction issue, 66 % of the cycles with 148 warp
+// instructions per cell, then the chain's own latency (~840 cycles per pair) and the ALU pipe,
+// 55 %; tensor pipe 41 % (five N 48 MMAs of 24.5 cycles per pair and tile), DRAM 7 %. The 256^3
+// mixed step takes 3.16 ms, 3.36 ms with two tiles of two warpgroups per SM that both converted and
+// summed, waiting for each pair's layer 2 before the next. What each part brought, 256^3, from
+// 3.36 ms, each with relu as (b + |b|) / 2: 32-bit offsets and A2 in place with three chains 3.27;
+// converters and summers apart 3.16; an issuer warp 3.11; named barriers instead of polls 3.05; D2
+// read whole before the sum and layer 1 two pairs ahead 2.97. That relu runs on the FMA pipe where
+// max runs on the ALU pipe at half the rate, but turns minus infinity into NaN and overflows above
+// half of the largest float: with max, as everywhere else, the step takes 3.16 ms where it took 3.05
+// on the same GPU.
 //
 // Hand-overs, per chain (n = 0..23 of a tile, b = n & 1):
 //   a1full            A1 of the tile written (4 converter warps)      -> issuer: layer 1 of pairs 0, 1

@@ -13,8 +13,8 @@
 
 namespace lbm {
 
-// At the start of a kernel: lets the next launch begin, then waits for the one before (both
-// do nothing in a kernel launched plainly).
+// At the start of a kernel: lets a next launch made with `overlap` begin, however this one was
+// made, then waits for the one before (nothing to wait for in a kernel launched plainly).
 __device__ __forceinline__ void overlap_wait() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");

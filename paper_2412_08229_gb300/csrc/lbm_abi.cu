@@ -25,7 +25,7 @@ struct lbm_ctx {
     int cur = 0;
     float tau = 0.5f;
     bool have_weights = false;
-    NetParams* net = nullptr;  // host copy handed to FP32 NCO launches by value
+    NetParams* net = nullptr;  // host copy of the FP32 network's parameters (its depth selects the kernels)
     void* net_w = nullptr;     // device: NetParams of the FP32 network or the packed operands of a tensor-core network
     int* d_status = nullptr;
     double* d_partials = nullptr;

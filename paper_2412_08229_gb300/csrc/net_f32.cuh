@@ -3,7 +3,7 @@
 //
 // The 48 elements of O_h are (axis permutation p, sign vector s). With the columns of W1
 // rearranged per p (W1p, built on the host from the group tables) the first layer of element
-// (p, s) reads sgn(s, t) m_t in tensor order t, where sgn flips the moments that are odd in a
+// (p, s) reads sgn(s, t) m_t, where sgn flips the moments that are odd in a
 // reflected axis: sgn(s, t) = (-1)^popcount(s & c(t)) with c(t) the parity class of t (which
 // axes t is odd in). Grouping the sum by class, the 8 sign vectors of one permutation are an
 // 8-point Walsh-Hadamard transform of the 8 class sums y_c = sum_{t in class c} W1p[:, t] m_t:
