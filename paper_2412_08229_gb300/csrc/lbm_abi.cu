@@ -258,11 +258,20 @@ void make_net_params(const float* theta, bool deep, NetParams* out) {
     const float* W3 = deep ? bd + kHidden : b2 + kHidden;
     const float* b3 = W3 + kOut * kHidden;
     const GroupTables& g = group_tables();
+    struct Places {
+        int of[Q];
+    };
+    constexpr auto make = [] {
+        Places p{};
+        for (int t = 0; t < Q; ++t) p.of[t] = class_pos(t);
+        return p;
+    };
+    constexpr Places place = make();  // (class_pos at run time takes half a millisecond for all columns)
     *out = NetParams{};
     for (int p = 0; p < 6; ++p) {
         const int gp = p * 8;  // element with axis permutation p and no reflection
         for (int j = 0; j < kHidden; ++j) {
-            for (int k = 0; k < Q; ++k) out->W1p[p][j][class_pos(g.mperm_t[gp][kPrinted.e[k]])] = W1[j * Q + k];
+            for (int k = 0; k < Q; ++k) out->W1p[p][j][place.of[g.mperm_t[gp][kPrinted.e[k]]]] = W1[j * Q + k];
             out->W1p[p][j][Q] = b1[j];
         }
     }
